@@ -175,7 +175,7 @@ def _day_departures(n: int, rng: np.random.Generator) -> np.ndarray:
 
 
 REACH = 25.0  # lattice lines a trip wants to cover in each direction, on average (the network's edge cuts some short)
-LINK_STEPS = 24.0  # steps per link at a window's load, signals included, about
+LINK_STEPS = {"roads": 24.0, "grid": 110.0}  # steps per link at a window's load, signals included, about
 WARM_STEPS = 3072  # steps before a window: the network has filled
 
 
@@ -184,10 +184,10 @@ def _links(rows: int, cols: int, reach: float) -> float:
     return reach * (rows / (rows + 2.0 * reach) + cols / (cols + 2.0 * reach))
 
 
-def _window_demand(lay: dict, vehicles: int, rng: np.random.Generator, horizon: int) -> dict:
+def _window_demand(lay: dict, style: str, vehicles: int, rng: np.random.Generator, horizon: int) -> dict:
     """Steady departures that keep about `vehicles` on the network."""
     rows, cols = len(lay["eid"]) // lay["cols"], lay["cols"]
-    n = max(8, int(vehicles * horizon / (LINK_STEPS * _links(rows, cols, REACH))))
+    n = max(8, int(vehicles * horizon / (LINK_STEPS[style] * _links(rows, cols, REACH))))
     return _trips(lay, n, rng, rng.integers(0, horizon, n), REACH)
 
 
@@ -385,16 +385,16 @@ def prepare(case: dict, seed: int):
     if k == "window":
         net, lay = _network(case["rows"], case["cols"], "roads", rng)
         sim = L.Simulation(net, dict(bin_steps=BIN_STEPS, n_bins=4, seed=seed))
-        sim.load_demand(_window_demand(lay, case["vehicles"], rng, WARM_STEPS + case["steps"]))
+        sim.load_demand(_window_demand(lay, "roads", case["vehicles"], rng, WARM_STEPS + case["steps"]))
     elif k == "batch":
         nets, dems = [], []
         size = np.exp(np.random.default_rng(case["scenarios"]).uniform(-1.0, 1.0, case["scenarios"]))
         for s in range(case["scenarios"]):
             f = math.sqrt(size[s])
-            net, lay = _network(max(9, int(case["rows"] * f)), max(9, int(case["cols"] * f)),
-                                "roads" if s % 2 else "grid", rng)
+            style = "roads" if s % 2 else "grid"
+            net, lay = _network(max(9, int(case["rows"] * f)), max(9, int(case["cols"] * f)), style, rng)
             nets.append(net)
-            dems.append(_window_demand(lay, int(case["vehicles"] * size[s] / size.sum()), rng,
+            dems.append(_window_demand(lay, style, int(case["vehicles"] * size[s] / size.sum()), rng,
                                        WARM_STEPS + case["steps"]))
         sim = L.BatchSimulation(nets, dict(bin_steps=BIN_STEPS, n_bins=4))
         sim.load_demand(dems, seeds=rng.integers(1, 1 << 40, case["scenarios"]))
