@@ -2,20 +2,15 @@
 //
 // Network: inputs (padded to 64) -> 256 -> 256 -> 256 -> 1, GELU after each
 // hidden layer, BF16 weights and activations, FP32 accumulation, MSE loss,
-// Adam.  Every dense layer, forward and backward, is one BF16 GEMM
-// D[M x N] = A[M x K] . B[N x K]^T with both operands K-major:
-//   forward   Z_l   = H_{l-1} . W_l^T                  (A = H_{l-1}, B = W_l)
-//   backward  dH_l  = dZ_{l+1} . W_{l+1}               (A = dZ, B = W^T copy)
-//   weights   dW_l  = dZ_l^T . H_{l-1}                 (A = dZ^T, B = H^T copies,
-//                                                       K = samples, split over CTAs)
-// GEMM kernel: one 128 x BN output tile per CTA (BN = 256 or 64), K in
-// 64-element slices.  One thread issues TMA loads (128-byte swizzle) of the
-// A and B slices into a 4-stage shared-memory ring guarded by mbarriers,
-// one thread issues tcgen05.mma (M = 128, N = BN, K = 16 per instruction)
-// accumulating in tensor memory, and all eight warps read the accumulator
-// back with tcgen05.ld for a fused epilogue (bias, GELU and its derivative,
-// the output head, transposed copies for the weight gradients, bias-gradient
-// column sums, or FP32 atomics).
+// Adam.  Four kernels:
+//   mlp_forward_fused  inference: all layers of a 128-row tile in one CTA
+//   mlp_train_fused    training: forward and backward of a 128-row tile in a
+//                      cluster of two CTAs (each half the columns of every layer)
+//   mlp_wgrad          dW_l = dZ_l^T . H_{l-1}, split over the samples
+//   mlp_update         split sums, gradients and the Adam step
+// and a plain GEMM D = A . B^T (gemm_bf16_tn, the diagnostic entry).  All use
+// TMA loads (128-byte swizzle) into mbarrier-guarded shared memory, one thread
+// issuing tcgen05.mma into tensor memory and tcgen05.ld in the epilogues.
 // Every wait on an mbarrier is bounded; on timeout the kernel records an
 // error, stops issuing work and frees its tensor memory before returning.
 #include <cuda.h>
@@ -53,30 +48,11 @@ constexpr int kBK = 64;  // one 128-byte swizzle atom of BF16
 constexpr int kStages = 4;
 constexpr uint32_t kSpinLimit = 1u << 26;
 
-enum Epi : int {
-    kEpiGelu = 0,      // Z = acc + b -> H = GELU(Z) (bf16, row-major and transposed), GELU'(Z) (f32) for training
-    kEpiGeluHead = 1,  // as kEpiGelu, plus y = H . w4 + b4 (f32)
-    kEpiDgelu = 2,     // dZ = acc * GELU'(Z_prev) -> bf16 row-major and transposed, per-tile column sums
-    kEpiAtomic = 3,    // out (f32) += acc
-    kEpiStore = 4,     // out (f32) = acc
-};
-
 constexpr int kThreads = 256;  // eight warps: all take part in the epilogue
 
 struct GemmArgs {
     int M, N, K;
-    int ktiles_per_split;
-    int stages;            // depth of the operand ring (1..kStages)
-    const float *bias;     // N
-    float *gout;           // M x N: GELU'(Z) (kEpiGelu*, nullable)
-    __nv_bfloat16 *hout;   // M x N
-    __nv_bfloat16 *htout;  // N x M (nullable)
-    const float *gprev;    // M x N: GELU'(Z_prev) (kEpiDgelu)
-    float *colpart;        // (M / 128) x N: per-row-tile column sums of the output (kEpiDgelu, nullable)
-    const float *w4;       // N (kEpiGeluHead)
-    const float *b4;       // 1 (kEpiGeluHead)
-    float *yout;           // M (kEpiGeluHead)
-    float *fout;           // M x N (kEpiAtomic, kEpiStore)
+    float *fout;  // M x N
     uint32_t *err;
 };
 
@@ -86,6 +62,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)_
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
@@ -158,11 +138,10 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 }
 
 
-// Writers of a staged 32 x 32 slice (row pitch 33 floats, so that a warp's
-// accesses fall in 32 different banks).  Row r of the slice is output row
-// rw0 + r, column j is output column col0 + j; rows at or past M are skipped.
-
-// f32 rows, four columns per thread: a warp instruction writes 4 whole rows
+// Writer of a staged 32 x 32 slice (row pitch 33 floats, so that a warp's
+// accesses fall in 32 different banks): row r of the slice is output row
+// rw0 + r, column j output column col0 + j; rows at or past M are skipped.
+// Four columns per thread: a warp instruction writes 4 whole rows.
 __device__ __forceinline__ void store_rows_f32(const float *stage, float *out, int N, int M, int rw0, int col0,
                                                int lane) {
 #pragma unroll
@@ -174,48 +153,9 @@ __device__ __forceinline__ void store_rows_f32(const float *stage, float *out, i
     }
 }
 
-// f32 accumulation into rows (split-K partial sums)
-__device__ __forceinline__ void add_rows_f32(const float *stage, float *out, int N, int M, int rw0, int col0,
-                                             int lane) {
-#pragma unroll 4
-    for (int r = 0; r < 32; r++) {
-        if (rw0 + r >= M) break;
-        atomicAdd(out + (size_t)(rw0 + r) * N + col0 + lane, stage[r * 33 + lane]);
-    }
-}
-
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t *>(&p);
-}
-
-// bf16 rows (the staged values are already bf16-representable), eight
-// columns per thread: a warp instruction writes 8 whole 64-byte row pieces
-__device__ __forceinline__ void store_rows_bf16(const float *stage, __nv_bfloat16 *out, int N, int M, int rw0,
-                                                int col0, int lane) {
-#pragma unroll
-    for (int it = 0; it < 4; it++) {
-        const int r = it * 8 + (lane >> 2), q = (lane & 3) * 8;
-        if (rw0 + r >= M) continue;
-        const float *sp = stage + r * 33 + q;
-        const uint4 v = make_uint4(pack_bf16x2(sp[0], sp[1]), pack_bf16x2(sp[2], sp[3]), pack_bf16x2(sp[4], sp[5]),
-                                   pack_bf16x2(sp[6], sp[7]));
-        *reinterpret_cast<uint4 *>(out + (size_t)(rw0 + r) * N + col0 + q) = v;
-    }
-}
-
-// bf16 transposed copy (out is N x M): eight rows of one column per thread
-__device__ __forceinline__ void store_cols_bf16(const float *stage, __nv_bfloat16 *outT, int M, int rw0, int col0,
-                                                int lane) {
-#pragma unroll
-    for (int it = 0; it < 4; it++) {
-        const int j = it * 8 + (lane >> 2), r0 = (lane & 3) * 8;
-        if (rw0 + r0 >= M) continue;
-        const float *sp = stage + r0 * 33 + j;
-        const uint4 v = make_uint4(pack_bf16x2(sp[0], sp[33]), pack_bf16x2(sp[66], sp[99]),
-                                   pack_bf16x2(sp[132], sp[165]), pack_bf16x2(sp[198], sp[231]));
-        *reinterpret_cast<uint4 *>(outT + (size_t)(col0 + j) * M + rw0 + r0) = v;
-    }
 }
 
 // Standard normal CDF for GELU(z) = z Phi(z), as a logistic of an odd
@@ -291,32 +231,29 @@ __device__ __forceinline__ void gelu_pair(float acc0, float acc1, float b0, floa
 __device__ __forceinline__ float norm_pdf(float z) { return 0.3989422804f * ex2_fast(-0.7213475204f * (z * z)); }
 
 // ------------------------------------------------------------- GEMM kernel
+//
+// D[M x N] = A[M x K] . B[N x K]^T, both operands K-major: one 128 x BN tile
+// per CTA (BN = 256 or 64), K in 64-element slices through a ring of kStages.
 
-template <int BN, int EPI>
-__global__ void __launch_bounds__(kThreads, 2)
+template <int BN>
+__global__ void __launch_bounds__(kThreads)
     gemm_bf16_tn(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, GemmArgs g) {
     constexpr uint32_t kABytes = kBM * kBK * 2;
     constexpr uint32_t kBBytes = BN * kBK * 2;
-    constexpr bool kGelu = EPI == kEpiGelu || EPI == kEpiGeluHead;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *sA = smem;
-    const int ns = g.stages;
+    constexpr int ns = kStages;
     uint8_t *sB = smem + ns * kABytes;
     uint64_t *full = reinterpret_cast<uint64_t *>(sB + ns * kBBytes);
     uint64_t *empty = full + ns;
     uint64_t *done = empty + ns;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
     __shared__ int s_fail;
-    __shared__ float s_head[2][kBM];  // output-head partial sums of the two column halves
-    __shared__ float s_col[4][BN];    // column sums of the four 32-row quarters
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
-    const int kt0 = blockIdx.z * g.ktiles_per_split;
-    const int kt_total = (g.K + kBK - 1) / kBK;
-    const int kt1 = min(kt_total, kt0 + g.ktiles_per_split);
-    const int nk = kt1 - kt0;
+    const int nk = g.K / kBK;
 
     if (threadIdx.x == 0) {
         s_fail = 0;
@@ -329,7 +266,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(BN < 32 ? 32 : BN));
+                     "r"(BN));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -337,157 +274,67 @@ __global__ void __launch_bounds__(kThreads, 2)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
 
-    bool ok = false;
-    if (nk > 0) {
-        if (warp == 0 && lane == 0) {
-            // TMA producer
-            for (int i = 0; i < nk; i++) {
-                const int s = i % ns;
-                if (i >= ns && !mbar_wait(&empty[s], ((i / ns) - 1) & 1)) {
-                    atomicOr(g.err, 1u);
-                    s_fail = 1;
-                    break;
-                }
-                if (s_fail) break;
-                mbar_expect_tx(&full[s], kABytes + kBBytes);
-                tma_load_2d(sA + s * kABytes, &tA, &full[s], (kt0 + i) * kBK, m0);
-                tma_load_2d(sB + s * kBBytes, &tB, &full[s], (kt0 + i) * kBK, n0);
+    if (warp == 0 && lane == 0) {
+        // TMA producer
+        for (int i = 0; i < nk; i++) {
+            const int s = i % ns;
+            if (i >= ns && !mbar_wait(&empty[s], ((i / ns) - 1) & 1)) {
+                atomicOr(g.err, 1u);
+                s_fail = 1;
+                break;
             }
-        } else if (warp == 1 && lane == 0) {
-            // MMA issuer
-            const uint32_t idesc = umma_idesc(BN);
-            for (int i = 0; i < nk; i++) {
-                const int s = i % ns;
-                if (!mbar_wait(&full[s], (i / ns) & 1)) {
-                    atomicOr(g.err, 2u);
-                    s_fail = 1;
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t a0 = smem_u32(sA + s * kABytes), b0 = smem_u32(sB + s * kBBytes);
-#pragma unroll
-                for (int kk = 0; kk < kBK / 16; kk++)
-                    umma_f16(tmem, umma_desc(a0 + kk * 32), umma_desc(b0 + kk * 32), idesc, (i | kk) != 0);
-                umma_commit(&empty[s]);
-            }
-            umma_commit(done);
+            if (s_fail) break;
+            mbar_expect_tx(&full[s], kABytes + kBBytes);
+            tma_load_2d(sA + s * kABytes, &tA, &full[s], i * kBK, m0);
+            tma_load_2d(sB + s * kBBytes, &tB, &full[s], i * kBK, n0);
         }
-        __syncwarp();
-        // Epilogue, all eight warps.  A warp may only read the tensor-memory
-        // lanes of its quarter (warp % 4), i.e. accumulator rows
-        // m0 + 32 (warp % 4) .. + 31, one row per thread; warps 0-3 take the
-        // first half of the columns and warps 4-7 the second.  Every 32-column
-        // slice is staged through shared memory (the operand ring is idle once
-        // the last MMA has completed) so that the global reads and writes are
-        // whole rows (or whole transposed columns) per warp instruction.
-        ok = mbar_wait(done, 0);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (!ok) atomicOr(g.err, 4u);
-        const int q = warp & 3, ch = warp >> 2;
-        float *stZ = reinterpret_cast<float *>(smem) + warp * (2 * 32 * 33);  // 32 x 32 slices, row pitch 33
-        float *stH = stZ + 32 * 33;
-        const int rw0 = m0 + q * 32;
-        float head = 0.0f;
-        if (ok && !s_fail) {
+    } else if (warp == 1 && lane == 0) {
+        // MMA issuer
+        const uint32_t idesc = umma_idesc(BN);
+        for (int i = 0; i < nk; i++) {
+            const int s = i % ns;
+            if (!mbar_wait(&full[s], (i / ns) & 1)) {
+                atomicOr(g.err, 2u);
+                s_fail = 1;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t a0 = smem_u32(sA + s * kABytes), b0 = smem_u32(sB + s * kBBytes);
+#pragma unroll
+            for (int kk = 0; kk < kBK / 16; kk++)
+                umma_f16(tmem, umma_desc(a0 + kk * 32), umma_desc(b0 + kk * 32), idesc, (i | kk) != 0);
+            umma_commit(&empty[s]);
+        }
+        umma_commit(done);
+    }
+    __syncwarp();
+    // Epilogue, all eight warps.  A warp may only read the tensor-memory
+    // lanes of its quarter (warp % 4), i.e. accumulator rows
+    // m0 + 32 (warp % 4) .. + 31, one row per thread; warps 0-3 take the
+    // first half of the columns and warps 4-7 the second.  Every 32-column
+    // slice is staged through shared memory (the operand ring is idle once
+    // the last MMA has completed) so that the writes are whole rows.
+    const bool ok = mbar_wait(done, 0);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (!ok) atomicOr(g.err, 4u);
+    const int q = warp & 3, ch = warp >> 2;
+    float *stage = reinterpret_cast<float *>(smem) + warp * (32 * 33);
+    if (ok && !s_fail) {
 #pragma unroll 1
-            for (int cc = 0; cc < BN / 2; cc += 32) {
-                const int c0 = ch * (BN / 2) + cc;
-                const int col0 = n0 + c0;
-                if (EPI == kEpiDgelu) {
-                    // GELU'(Z_prev) slice, read row by row
+        for (int cc = 0; cc < BN / 2; cc += 32) {
+            const int c0 = ch * (BN / 2) + cc;
+            uint32_t r[32];
+            tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
 #pragma unroll
-                    for (int it = 0; it < 8; it++) {
-                        const int r = it * 4 + (lane >> 3), qq = (lane & 7) * 4;
-                        float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (rw0 + r < g.M)
-                            z4 = *reinterpret_cast<const float4 *>(g.gprev + (size_t)(rw0 + r) * g.N + col0 + qq);
-                        float *sp = stZ + r * 33 + qq;
-                        sp[0] = z4.x;
-                        sp[1] = z4.y;
-                        sp[2] = z4.z;
-                        sp[3] = z4.w;
-                    }
-                    __syncwarp();
-                }
-                uint32_t r[32];
-                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-                float *mz = stZ + lane * 33, *mh = stH + lane * 33;
-                if (kGelu) {
-                    // bias (and head weights) four columns at a time: 16-byte loads, the same for every lane
-                    uint32_t hp[16];  // the row's 32 activations as bf16 pairs
-#pragma unroll
-                    for (int q4 = 0; q4 < 8; q4++) {
-                        const float4 b4v = reinterpret_cast<const float4 *>(g.bias + col0)[q4];
-                        float4 w4v = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (EPI == kEpiGeluHead) w4v = reinterpret_cast<const float4 *>(g.w4 + col0)[q4];
-                        const float bq[4] = {b4v.x, b4v.y, b4v.z, b4v.w};
-                        const float wq[4] = {w4v.x, w4v.y, w4v.z, w4v.w};
-                        __nv_bfloat16 hb[4];
-#pragma unroll
-                        for (int u = 0; u < 4; u++) {
-                            const int j = 4 * q4 + u;
-                            const float z = __uint_as_float(r[j]) + bq[u];
-                            const float cdf = norm_cdf(z);
-                            hb[u] = __float2bfloat16_rn(z * cdf);
-                            const float h = __bfloat162float(hb[u]);
-                            if (g.htout) mh[j] = h;
-                            if (g.gout) mz[j] = cdf + z * norm_pdf(z);
-                            if (EPI == kEpiGeluHead) head += h * wq[u];
-                        }
-                        const __nv_bfloat162 p0 = __halves2bfloat162(hb[0], hb[1]);
-                        const __nv_bfloat162 p1 = __halves2bfloat162(hb[2], hb[3]);
-                        hp[2 * q4] = *reinterpret_cast<const uint32_t *>(&p0);
-                        hp[2 * q4 + 1] = *reinterpret_cast<const uint32_t *>(&p1);
-                    }
-                    // the row-major activations straight from registers: 64 contiguous bytes per row
-                    if (g.hout && rw0 + lane < g.M) {
-                        uint4 *dst = reinterpret_cast<uint4 *>(g.hout + (size_t)(rw0 + lane) * g.N + col0);
-#pragma unroll
-                        for (int q4 = 0; q4 < 4; q4++)
-                            dst[q4] = make_uint4(hp[4 * q4], hp[4 * q4 + 1], hp[4 * q4 + 2], hp[4 * q4 + 3]);
-                    }
-                } else if (EPI == kEpiDgelu) {
-#pragma unroll
-                    for (int j = 0; j < 32; j++)
-                        mh[j] = __bfloat162float(__float2bfloat16_rn(__uint_as_float(r[j]) * mz[j]));
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 32; j++) mh[j] = __uint_as_float(r[j]);
-                }
-                __syncwarp();
-                if (kGelu) {
-                    if (g.gout) store_rows_f32(stZ, g.gout, g.N, g.M, rw0, col0, lane);
-                    if (g.htout) store_cols_bf16(stH, g.htout, g.M, rw0, col0, lane);
-                } else if (EPI == kEpiDgelu) {
-                    store_rows_bf16(stH, g.hout, g.N, g.M, rw0, col0, lane);
-                    if (g.htout) store_cols_bf16(stH, g.htout, g.M, rw0, col0, lane);
-                } else if (EPI == kEpiAtomic) {
-                    add_rows_f32(stH, g.fout, g.N, g.M, rw0, col0, lane);
-                } else {
-                    store_rows_f32(stH, g.fout, g.N, g.M, rw0, col0, lane);
-                }
-                if (EPI == kEpiDgelu && g.colpart) {
-                    float cs = 0.0f;
-                    for (int rr = 0; rr < 32; rr++)
-                        if (rw0 + rr < g.M) cs += stH[rr * 33 + lane];
-                    s_col[q][c0 + lane] = cs;
-                }
-                __syncwarp();
-            }
+            for (int j = 0; j < 32; j++) stage[lane * 33 + j] = __uint_as_float(r[j]);
+            __syncwarp();
+            store_rows_f32(stage, g.fout, g.N, g.M, m0 + q * 32, n0 + c0, lane);
+            __syncwarp();
         }
-        if (EPI == kEpiGeluHead) s_head[ch][q * 32 + lane] = head;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN < 32 ? 32 : BN));
-    if (nk > 0 && ok && !s_fail) {
-        if (EPI == kEpiGeluHead && threadIdx.x < kBM && m0 + (int)threadIdx.x < g.M)
-            g.yout[m0 + threadIdx.x] = (s_head[0][threadIdx.x] + s_head[1][threadIdx.x]) + *g.b4;
-        if (EPI == kEpiDgelu && g.colpart && threadIdx.x < BN)
-            g.colpart[(size_t)blockIdx.x * g.N + n0 + threadIdx.x] =
-                ((s_col[0][threadIdx.x] + s_col[1][threadIdx.x]) + s_col[2][threadIdx.x]) + s_col[3][threadIdx.x];
-    }
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN));
 }
 
 
@@ -527,10 +374,6 @@ struct FwdArgs {
     float *y;
     uint32_t *err;
 };
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 
 __global__ void __launch_bounds__(kFwdThreads, 1)
     mlp_forward_fused(const __grid_constant__ CUtensorMap tX, const __grid_constant__ CUtensorMap tW1,
@@ -761,120 +604,13 @@ __global__ void gelu_eval(const float *z, uint64_t n, float *gelu, float *dgelu)
     }
 }
 
-// X (n x nf f32, host layout) -> Xb (n_pad x 64 bf16, zero padded) and its
-// transpose.  Block (32, 8) handles a 32-row x 32-column tile; the transposed
-// copy goes through shared memory so both writes are whole rows.
-__global__ void pack_inputs(const float *X, int n, int nf, int n_pad, __nv_bfloat16 *Xb, __nv_bfloat16 *XbT) {
-    __shared__ __nv_bfloat16 tile[32][34];
-    const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32, tx = threadIdx.x, ty = threadIdx.y;
-    for (int rr = ty; rr < 32; rr += 8) {
-        const int r = r0 + rr, c = c0 + tx;
-        const float v = (r < n && c < nf) ? X[(size_t)r * nf + c] : 0.0f;
-        const __nv_bfloat16 b = __float2bfloat16_rn(v);
-        Xb[(size_t)r * 64 + c] = b;
-        tile[rr][tx] = b;
-    }
-    if (!XbT) return;
-    __syncthreads();
-    for (int cc = ty; cc < 32; cc += 8) XbT[(size_t)(c0 + cc) * n_pad + r0 + tx] = tile[tx][cc];
-}
-
-// dy = 2/n (y - t) on real rows; dZ3 = dy * w4 * GELU'(Z3) (bf16, row-major and
-// transposed; GELU'(Z3) was stored by the forward pass); per-row dy kept for
-// dW4 / db4; the squared errors summed into loss_acc.  Tiles of 32 rows x 32
-// columns as in pack_inputs.
-__global__ void head_backward(const float *y, const float *t, int n, int n_pad, const float *w4, const float *G3,
-                              __nv_bfloat16 *dZ3, __nv_bfloat16 *dZ3T, float *dy, float *loss_acc) {
-    __shared__ __nv_bfloat16 tile[32][34];
-    const float scale = 2.0f / (float)n;
-    const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32, tx = threadIdx.x, ty = threadIdx.y;
-    for (int rr = ty; rr < 32; rr += 8) {
-        const int r = r0 + rr, c = c0 + tx;
-        const float d = r < n ? scale * (y[r] - t[r]) : 0.0f;
-        const __nv_bfloat16 b = __float2bfloat16_rn(d * w4[c] * G3[(size_t)r * 256 + c]);
-        dZ3[(size_t)r * 256 + c] = b;
-        tile[rr][tx] = b;
-    }
-    if (blockIdx.y == 0 && ty == 0) {
-        // one warp per 32 rows: dy and the loss
-        const int r = r0 + tx;
-        const float e = r < n ? y[r] - t[r] : 0.0f;
-        dy[r] = r < n ? scale * e : 0.0f;
-        float sq = e * e;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
-        if (tx == 0 && sq != 0.0f) atomicAdd(loss_acc, sq);
-    }
-    __syncthreads();
-    for (int cc = ty; cc < 32; cc += 8) dZ3T[(size_t)(c0 + cc) * n_pad + r0 + tx] = tile[tx][cc];
-}
-
-// Column sums of A (rows x cols bf16), optionally weighted by rowscale[r]:
-// the bias gradients (column sums of dZ) and dW4 (dy-weighted sums of H3).
-// Stage 1: block (32, 8) sums a band of rows for 32 columns into part[band][c];
-// stage 2 adds the bands in order.
-constexpr int kSumBands = 256;
-
-__global__ void column_partials(const __nv_bfloat16 *A, int rows, int cols, const float *rowscale, float *part) {
-    __shared__ float red[8][33];
-    const int c = blockIdx.x * 32 + threadIdx.x;
-    const int band = (rows + kSumBands - 1) / kSumBands;
-    const int rb = blockIdx.y * band, re = min(rows, rb + band);
-    float acc = 0.0f;
-    for (int r = rb + threadIdx.y; r < re; r += 8) {
-        const float a = __bfloat162float(A[(size_t)r * cols + c]);
-        acc += rowscale ? a * rowscale[r] : a;
-    }
-    red[threadIdx.y][threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.y == 0) {
-        float s2 = 0.0f;
-        for (int q = 0; q < 8; q++) s2 += red[q][threadIdx.x];
-        part[(size_t)blockIdx.y * cols + c] = s2;
-    }
-}
-
-// out[c] = sum over bands b of part[b][c], in a fixed order (a block per column)
-__global__ void reduce_bands(const float *part, int n_bands, int cols, float *out) {
-    __shared__ float red[256];
-    const int c = blockIdx.x;
-    float acc = 0.0f;
-    for (int b = threadIdx.x; b < n_bands; b += 256) acc += part[(size_t)b * cols + c];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[c] = red[0];
-}
-
-// part[b] = sum of v over band b of kSumBands equal bands
-__global__ void vector_partials(const float *v, int n, float *part) {
-    __shared__ float red[256];
-    const int band = (n + kSumBands - 1) / kSumBands;
-    const int rb = blockIdx.x * band, re = min(n, rb + band);
-    float acc = 0.0f;
-    for (int i = rb + threadIdx.x; i < re; i += 256) acc += v[i];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = red[0];
-}
-
-// Adam (Kingma and Ba 2015, Algorithm 1) on f32 master weights
-__global__ void adam_update(float *p, const float *grad, float *m, float *v, int n, float lr, float b1, float b2,
-                            float eps, float c1, float c2) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const float gi = grad[i];
-        const float mi = b1 * m[i] + (1.0f - b1) * gi;
-        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+// X (n x nf f32, host layout) -> Xb (n_pad x 64 bf16, zero padded); block
+// (32, 8) handles a 32-row x 32-column tile
+__global__ void pack_inputs(const float *X, int n, int nf, __nv_bfloat16 *Xb) {
+    const int r0 = blockIdx.x * 32, c = blockIdx.y * 32 + threadIdx.x;
+    for (int rr = threadIdx.y; rr < 32; rr += 8) {
+        const int r = r0 + rr;
+        Xb[(size_t)r * 64 + c] = __float2bfloat16_rn((r < n && c < nf) ? X[(size_t)r * nf + c] : 0.0f);
     }
 }
 
@@ -914,24 +650,749 @@ __device__ __forceinline__ uint64_t feistel(uint64_t x, uint32_t h, uint64_t key
     return (L << h) | R;
 }
 
-// batch rows j < nb: pool row perm_pass(pos % n) for pos = pos0 + j
-__global__ void gather_batch(const float *PX, const float *Pt, uint64_t n, int nf, uint32_t h, uint64_t seed,
-                             uint64_t pos0, uint32_t nb, float *Xf, float *t, uint32_t *err) {
-    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < nb; j += gridDim.x * blockDim.x) {
-        const uint64_t pos = pos0 + j, pass = pos / n;
-        const uint64_t key = mix64(seed ^ (pass * 0xD1B54A32D192ED03ull));
-        uint64_t r = pos % n;
-        uint32_t walk = 0;
-        do {
-            r = feistel(r, h, key);
-        } while (r >= n && ++walk < 4096u);
-        if (r >= n) {
-            atomicOr(err, 64u);
-            r = pos % n;
-        }
-        for (int c = 0; c < nf; c++) Xf[(size_t)j * nf + c] = PX[r * nf + c];
-        t[j] = Pt[r];
+// ------------------------------------------- fused training forward + backward
+//
+// The forward of a 128-row tile, its loss and the backward down to dZ1 in one
+// cluster of two CTAs.  CTA r computes all 128 rows of columns
+// [128 r, 128 r + 128) of every layer; each layer's input has to be whole, so
+// a finished half goes to the partner's shared memory by bulk copy (32 KB per
+// layer, in 4 KB pieces as the warps finish them) beside the CTA's own copy.
+// A batch of 8192 rows is 64 tiles: one tile per CTA would leave 88 of the 152
+// SMs idle while the others run a serial chain of five MMAs and five
+// epilogues, so the chain itself is cut in two.
+//
+//   s = 0, 1   Z = A . W^T + b, H = GELU(Z)     MMA s -> T[s]
+//   s = 2      the same, y = H . w4 + b4, dy, dZ3 = dy w4 GELU'(Z3)
+//   s = 3, 4   dZ = (dZ_above . W) GELU'(Z)     MMA 3 -> T[3], MMA 4 -> T[2]
+//
+// T[0..3] are the four 128-column f32 accumulators that fill tensor memory:
+// GELU'(Z1) and GELU'(Z2) replace Z1 and Z2 in place (f32, as computed) until
+// the backward needs them, so only the BF16 operands of the weight gradients
+// (X, H1, H2, dZ1..3, row-major) leave the chip, by TMA straight from the
+// swizzled shared-memory tiles.  The column sums (bias gradients, dW4) are
+// taken from those tiles while the next MMA runs and kept in registers
+// over the CTA's tiles.  Training rows are drawn from the pool by the kernel
+// itself (no gathered copy, no packing pass).
+//
+// Sums that decide a BF16 rounding keep one order whatever the tile's CTA: K
+// ascending in every MMA, the head's 128 columns ascending per half, so dZ is the
+// same wherever a row lands in a batch.
+//
+// Bound by latency: one tile's chain of five MMAs (0.55 us of tensor work
+// each) and five epilogues.  A training step of 8192 rows (this kernel, mlp_wgrad
+// and mlp_update) takes 40.5 us, 155648 rows 440 us; with one GEMM launch per
+// layer and gradient (transposed copies and f32 GELU' through memory, 47
+// launches and memsets a step) it took 279 us and 908 us.
+//
+// The activation buffers alternate: X in 0, H1 in 1, H2 in 0, H3 in 1 (own
+// half only), dZ3 in 0, dZ2 in 1, dZ1 in 0 (own half only).  A half may be
+// written into the partner's buffer once the partner's MMA that last read
+// that buffer is complete; the data received since then says so (its H1 follows
+// its MMA 0, its head sum its MMA 2, and so on), except across tiles, where
+// the partner reports the end of MMA 4 (peer_free).
+
+constexpr int kTrEpiWarps = 16;
+constexpr int kTrThreads = (2 + kTrEpiWarps) * 32;
+constexpr int kTrBStages = 5;
+constexpr uint32_t kTrSliceB = 128 * kBK * 2;  // one 64-wide K slice of half a weight matrix: 16 KB
+constexpr size_t kTrSmem = 1024 + 2 * kFwdBuf + kTrBStages * kTrSliceB + 256;
+constexpr int kSmall = 1026;  // per-cluster sums: db1, db2, db3, dW4 (256 each), squared errors, db4
+
+struct TrainMaps {
+    CUtensorMap w[5];   // operand B of MMA s: W1, W2, W3, W3^T, W2^T (boxes of 128 rows x 64)
+    CUtensorMap x0;     // X (boxes of 128 x 64)
+    CUtensorMap h[2];   // H1, H2 (boxes of 32 x 64)
+    CUtensorMap dz[3];  // dZ1..3 (boxes of 32 x 64)
+};
+
+struct TrainArgs {
+    int n_rows, n_tiles;  // rows of the batch; 128-row tiles that hold them (missing rows count as zero error)
+    int nf, l1_k16;
+    const float *X, *t;   // the batch, or the training pool
+    uint64_t pool_n;      // 0: rows in order; else rows drawn from a pool of pool_n
+    uint64_t seed, pos0;
+    uint32_t h;
+    const float *b1, *b2, *b3, *w4, *b4;
+    float *small;         // clusters x kSmall
+    uint32_t *err;
+};
+
+// bounded wait that also sees what the partner CTA wrote before completing the phase
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity) {
+    const uint32_t a = smem_u32(bar);
+    for (uint32_t i = 0; i < kSpinLimit; i++) {
+        uint32_t done;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+            " selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(a), "r"(parity)
+            : "memory");
+        if (done) return true;
     }
+    return false;
+}
+
+__device__ __forceinline__ uint32_t mapa_u32(uint32_t saddr, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+    return r;
+}
+
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, const void *src, int x, int y) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"((uint64_t)map),
+                 "r"(smem_u32(src)), "r"(x), "r"(y)
+                 : "memory");
+}
+
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
+        "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
+        "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+        : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+// GELU and GELU' of two activations on the paired FP32 instructions, each
+// lane rounded as z * norm_cdf(z) and norm_cdf(z) + z * norm_pdf(z) round it
+__device__ __forceinline__ void gelu_grad_pair(float acc0, float acc1, float b0, float b1, float &h0, float &h1,
+                                               uint32_t &g0, uint32_t &g1) {
+    const f32x2_t z = f2_add(f2_pack(acc0, acc1), f2_pack(b0, b1));
+    const f32x2_t z2 = f2_mul(z, z);
+    f32x2_t q = f2_fma(f2_pack(-3.231081337e-06f, -3.231081337e-06f), z2, f2_pack(8.827482816e-05f, 8.827482816e-05f));
+    q = f2_fma(q, z2, f2_pack(3.600096097e-04f, 3.600096097e-04f));
+    q = f2_fma(q, z2, f2_pack(-1.052259058e-01f, -1.052259058e-01f));
+    q = f2_fma(q, z2, f2_pack(-2.302046061e+00f, -2.302046061e+00f));
+    float s0, s1, d0, d1, p0, p1;
+    f2_unpack(f2_mul(z, q), s0, s1);
+    f2_unpack(f2_add(f2_pack(1.0f, 1.0f), f2_pack(ex2_fast(s0), ex2_fast(s1))), d0, d1);
+    const f32x2_t cdf = f2_pack(rcp_fast(d0), rcp_fast(d1));
+    f2_unpack(f2_mul(z, cdf), h0, h1);
+    f2_unpack(f2_mul(f2_pack(-0.7213475204f, -0.7213475204f), z2), p0, p1);
+    const f32x2_t pdf = f2_mul(f2_pack(0.3989422804f, 0.3989422804f), f2_pack(ex2_fast(p0), ex2_fast(p1)));
+    float u0, u1;
+    f2_unpack(f2_add(cdf, f2_mul(z, pdf)), u0, u1);
+    g0 = __float_as_uint(u0);
+    g1 = __float_as_uint(u1);
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrThreads, 1)
+    mlp_train_fused(const __grid_constant__ TrainMaps mp, TrainArgs g) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *sA = smem;              // two activation buffers (kFwdBuf each: four K slices of 128 rows)
+    uint8_t *sB = sA + 2 * kFwdBuf;  // weight-slice ring
+    uint64_t *b_full = reinterpret_cast<uint64_t *>(sB + kTrBStages * kTrSliceB);
+    uint64_t *b_empty = b_full + kTrBStages;
+    uint64_t *peer_full = b_empty + kTrBStages;  // [2] the partner's half of MMA s's input landed, s = 1, 3 / 2, 4
+    uint64_t *acc_full = peer_full + 2;          // MMA -> epilogue
+    uint64_t *ep_done = acc_full + 1;            // epilogue -> MMA: own half written, accumulator drained
+    uint64_t *head_full = ep_done + 1;           // the partner's head sums landed
+    uint64_t *peer_free = head_full + 1;         // the partner's MMA 4 of a tile is complete
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(peer_free + 1);
+    __shared__ volatile int s_fail;
+    __shared__ __align__(16) float s_par[4][128];  // b1, b2, b3, w4 of this CTA's columns
+    __shared__ __align__(16) float s_hr[128];      // the partner's head sums
+    __shared__ float s_sum[2][4];                  // squared errors and db4 of the four row quarters
+    __shared__ float s_t[128], s_dy[128];
+    __shared__ __align__(8) float s_col[8][128];   // column sums of the eight 16-row groups
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = blockIdx.x & 1u;  // clusters are pairs of neighbouring blocks
+    const int cl = (int)(blockIdx.x >> 1), n_cl = (int)(gridDim.x >> 1);
+    const int nt = cl < g.n_tiles ? (g.n_tiles - 1 - cl) / n_cl + 1 : 0;  // tiles cl + i n_cl
+    if (threadIdx.x == 0) {
+        s_fail = 0;
+        for (int s = 0; s < kTrBStages; s++) {
+            mbar_init(&b_full[s], 1);
+            mbar_init(&b_empty[s], 1);
+        }
+        mbar_init(&peer_full[0], 1);
+        mbar_init(&peer_full[1], 1);
+        mbar_init(acc_full, 1);
+        mbar_init(ep_done, kTrEpiWarps);
+        mbar_init(head_full, 1);
+        mbar_init(peer_free, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    // the partner's barriers are initialised before anything is sent there
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+    // the previous step's weights, and the buffers its weight gradients read
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
+    auto give_up = [&](uint32_t code) {
+        atomicOr(g.err, code);
+        s_fail = 1;
+    };
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // weight slices in the order the MMAs take them
+            uint32_t bi = 0;
+            for (int ti = 0; ti < nt && !s_fail; ti++) {
+                for (int s = 0; s < 5 && !s_fail; s++) {
+                    const int nks = s == 0 ? 1 : 4;
+                    for (int i = 0; i < nks && !s_fail; i++, bi++) {
+                        const int st = bi % kTrBStages;
+                        if (bi >= kTrBStages && !mbar_wait(&b_empty[st], ((bi / kTrBStages) - 1) & 1)) {
+                            give_up(8u);
+                            break;
+                        }
+                        mbar_expect_tx(&b_full[st], kTrSliceB);
+                        tma_load_2d(sB + st * kTrSliceB, &mp.w[s], &b_full[st], i * kBK, 128 * (int)rank);
+                    }
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t idesc = umma_idesc(128);
+            uint32_t bi = 0;
+            for (int ti = 0; ti < nt && !s_fail; ti++) {
+                for (int s = 0; s < 5 && !s_fail; s++) {
+                    if (!mbar_wait(ep_done, (5 * ti + s) & 1)) {
+                        give_up(16u);
+                        break;
+                    }
+                    // the half that comes from the partner: announced now, waited for before it is read
+                    if (s > 0) mbar_expect_tx(&peer_full[(s - 1) & 1], 2 * kSliceA);
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint8_t *abuf = sA + ((s == 1 || s == 4) ? kFwdBuf : 0);
+                    const uint32_t acc = tmem + (uint32_t)(s == 4 ? 2 : s) * 128u;
+                    const int nks = s == 0 ? 1 : 4;
+                    for (int i = 0; i < nks; i++, bi++) {
+                        const int st = bi % kTrBStages;
+                        // K slices 0, 1 come from CTA 0, slices 2, 3 from CTA 1
+                        if ((s > 0 && i == 2 * (int)(rank ^ 1u) && !mbar_wait_cluster(&peer_full[(s - 1) & 1], (2 * ti + ((s - 1) >> 1)) & 1)) ||
+                            !mbar_wait(&b_full[st], (bi / kTrBStages) & 1)) {
+                            give_up(16u);
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t a0 = smem_u32(abuf + i * kSliceA), b0 = smem_u32(sB + st * kTrSliceB);
+                        const int nkk = s == 0 ? g.l1_k16 : kBK / 16;
+#pragma unroll
+                        for (int kk = 0; kk < kBK / 16; kk++)
+                            if (kk < nkk)
+                                umma_f16(acc, umma_desc(a0 + kk * 32), umma_desc(b0 + kk * 32), idesc, (i | kk) != 0);
+                        umma_commit(&b_empty[st]);
+                    }
+                    umma_commit(acc_full);
+                }
+            }
+        }
+    } else {
+        // epilogue: row q * 32 + lane of the tile, columns [32 cq, 32 cq + 32) of this CTA's half
+        const int et = (int)threadIdx.x - 64;  // 0..511
+        const int q = warp & 3, cq = (warp - 2) >> 2;
+        const int row = q * 32 + lane;
+        const uint32_t peer = rank ^ 1u;
+        const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cq * 32);
+        // the two warps of rows 32 q.. and K slice 2 rank + cq / 2 write one contiguous 4 KB piece;
+        // lane 0 of the even one sends it on
+        const int pair_bar = 2 + 2 * q + (cq >> 1);
+        const bool sender = lane == 0 && (cq & 1) == 0;
+        const uint32_t piece = (uint32_t)(2 * rank + (cq >> 1)) * kSliceA + (uint32_t)q * 4096u;
+        const uint32_t rowoff = (uint32_t)(2 * rank + (cq >> 1)) * kSliceA + (uint32_t)(row >> 3) * 1024u +
+                                (uint32_t)(row & 7) * 128u;
+        const int ch0 = (cq & 1) * 4;
+        auto put_row = [&](uint8_t *buf, const uint32_t(&hp)[16]) {
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+                *reinterpret_cast<uint4 *>(buf + rowoff + (((ch0 + i) ^ (row & 7)) << 4)) =
+                    make_uint4(hp[4 * i], hp[4 * i + 1], hp[4 * i + 2], hp[4 * i + 3]);
+        };
+        auto wait_acc = [&](uint32_t n) {
+            if (!s_fail && !mbar_wait(acc_full, n & 1)) give_up(32u);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        };
+        // own half of buf written: to the MMA thread, to the partner (pf >= 0) and to global memory
+        auto hand_over = [&](uint8_t *buf, int pf, const CUtensorMap *gm, int r0) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0 && pf >= 0) mbar_arrive(ep_done);
+            asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
+            if (sender && !s_fail) {
+                if (pf >= 0)
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+                            "r"(mapa_u32(smem_u32(buf + piece), peer)),
+                        "r"(smem_u32(buf + piece)), "r"(4096u), "r"(mapa_u32(smem_u32(&peer_full[pf]), peer))
+                        : "memory");
+                tma_store_2d(gm, buf + piece, (int)(2 * rank + (cq >> 1)) * kBK, r0 + q * 32);
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            }
+        };
+        // the TMA stores so far have read their tiles, for the pair of warps that writes there next
+        auto tiles_read = [&]() {
+            if (sender) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
+        };
+        // sums over the tile's rows of this CTA's columns of buf, weighted by dy or not; thread et < 128 keeps column et
+        auto column_sum = [&](const uint8_t *buf, bool weighted, float &sum) {
+            asm volatile("bar.sync 1, %0;" ::"r"(kTrEpiWarps * 32) : "memory");
+            const int cp = et & 63, rg = et >> 6;
+            const uint8_t *base = buf + (size_t)(2 * rank + (cp >> 5)) * kSliceA + (cp & 3) * 4;
+            const int chunk = (cp & 31) >> 2;
+            float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll
+            for (int i = 0; i < 16; i++) {
+                const int r = rg * 16 + i;
+                const uint32_t v = *reinterpret_cast<const uint32_t *>(base + (r >> 3) * 1024 + (r & 7) * 128 +
+                                                                       ((chunk ^ (r & 7)) << 4));
+                const float lo = __uint_as_float(v << 16), hi = __uint_as_float(v & 0xFFFF0000u);
+                const float w = weighted ? s_dy[r] : 1.0f;
+                a0 += weighted ? lo * w : lo;
+                a1 += weighted ? hi * w : hi;
+            }
+            *reinterpret_cast<float2 *>(&s_col[rg][2 * cp]) = make_float2(a0, a1);
+            asm volatile("bar.sync 1, %0;" ::"r"(kTrEpiWarps * 32) : "memory");
+            if (et < 128) {
+                float c = 0.0f;
+#pragma unroll
+                for (int i = 0; i < 8; i++) c += s_col[i][et];
+                sum += c;
+            }
+        };
+        const float scale = 2.0f / (float)g.n_rows;
+        s_par[et >> 7][et & 127] = (et < 128 ? g.b1 : et < 256 ? g.b2 : et < 384 ? g.b3 : g.w4)[128 * rank + (et & 127)];
+        const float b4 = *g.b4;
+        float db1 = 0.0f, db2 = 0.0f, db3 = 0.0f, dw4 = 0.0f, sq = 0.0f, db4 = 0.0f;
+        for (int ti = 0; ti < nt; ti++) {
+            const int r0 = (cl + ti * n_cl) * 128;
+            // the batch rows: four threads per row, 16 columns each
+            tiles_read();
+            asm volatile("bar.sync 1, %0;" ::"r"(kTrEpiWarps * 32) : "memory");
+            {
+                const int xr = et >> 2, sub = et & 3;
+                const bool valid = r0 + xr < g.n_rows;
+                uint64_t src = (uint64_t)(r0 + xr);
+                if (g.pool_n && valid) {
+                    const uint64_t pos = g.pos0 + src, pass = pos / g.pool_n;
+                    const uint64_t key = mix64(g.seed ^ (pass * 0xD1B54A32D192ED03ull));
+                    const uint64_t r_first = pos - pass * g.pool_n;
+                    uint64_t r = r_first;
+                    uint32_t walk = 0;
+                    do {
+                        r = feistel(r, g.h, key);
+                    } while (r >= g.pool_n && ++walk < 4096u);
+                    if (r >= g.pool_n) {
+                        atomicOr(g.err, 64u);
+                        r = r_first;
+                    }
+                    src = r;
+                }
+                const float *xp = g.X + src * (uint64_t)g.nf;
+                float v[16];
+#pragma unroll
+                for (int i = 0; i < 16; i++) v[i] = valid && sub * 16 + i < g.nf ? xp[sub * 16 + i] : 0.0f;
+                uint8_t *xrow = sA + (xr >> 3) * 1024 + (xr & 7) * 128;
+#pragma unroll
+                for (int i = 0; i < 2; i++)
+                    *reinterpret_cast<uint4 *>(xrow + (((2 * sub + i) ^ (xr & 7)) << 4)) =
+                        make_uint4(pack_bf16x2(v[8 * i], v[8 * i + 1]), pack_bf16x2(v[8 * i + 2], v[8 * i + 3]),
+                                   pack_bf16x2(v[8 * i + 4], v[8 * i + 5]), pack_bf16x2(v[8 * i + 6], v[8 * i + 7]));
+                if (sub == 0) s_t[xr] = valid ? g.t[src] : 0.0f;
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            asm volatile("bar.sync 1, %0;" ::"r"(kTrEpiWarps * 32) : "memory");
+            if (lane == 0) mbar_arrive(ep_done);
+            if (sender && q == 0 && cq == 0 && rank == 0 && !s_fail) {
+                tma_store_2d(&mp.x0, sA, 0, r0);
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            }
+            // layers 1 and 2
+#pragma unroll 1
+            for (int s = 0; s < 2; s++) {
+                uint8_t *buf = sA + (s == 0 ? kFwdBuf : 0);
+                tiles_read();
+                wait_acc(5 * ti + s);
+                // the partner's MMA 4 of the tile before: its buffer 1 may be written, and it has this CTA's dZ2
+                if (s == 0 && ti > 0 && !s_fail && !mbar_wait_cluster(peer_free, (ti - 1) & 1)) give_up(32u);
+                uint32_t r[32], hp[16];
+                tmem_ld32(tlane + s * 128, r);
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    const float2 b = *reinterpret_cast<const float2 *>(&s_par[s][cq * 32 + 2 * j]);
+                    float h0, h1;
+                    gelu_grad_pair(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]), b.x, b.y, h0, h1, r[2 * j],
+                                   r[2 * j + 1]);
+                    hp[j] = pack_bf16x2(h0, h1);
+                }
+                put_row(buf, hp);
+                tmem_st32(tlane + s * 128, r);
+                hand_over(buf, s, &mp.h[s], r0);
+            }
+            // layer 3, the head and dZ3
+            tiles_read();
+            wait_acc(5 * ti + 2);
+            {
+                uint32_t r[32], hp[16];
+                tmem_ld32(tlane + 2 * 128, r);
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    const float2 b = *reinterpret_cast<const float2 *>(&s_par[2][cq * 32 + 2 * j]);
+                    float h0, h1;
+                    gelu_grad_pair(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]), b.x, b.y, h0, h1, r[2 * j],
+                                   r[2 * j + 1]);
+                    hp[j] = pack_bf16x2(h0, h1);
+                }
+                put_row(sA + kFwdBuf, hp);
+                if (et == 0) mbar_expect_tx(head_full, 512);
+                asm volatile("bar.sync 1, %0;" ::"r"(kTrEpiWarps * 32) : "memory");
+                if (cq == 0) {
+                    // the head over this CTA's columns in ascending order, one thread per row
+                    float own = 0.0f;
+#pragma unroll 4
+                    for (int c = 0; c < 16; c++) {
+                        const uint4 hv = *reinterpret_cast<const uint4 *>(
+                            sA + kFwdBuf + (size_t)(2 * rank + (c >> 3)) * kSliceA + (row >> 3) * 1024 +
+                            (row & 7) * 128 + (((c & 7) ^ (row & 7)) << 4));
+                        const float4 w0 = *reinterpret_cast<const float4 *>(&s_par[3][8 * c]);
+                        const float4 w1 = *reinterpret_cast<const float4 *>(&s_par[3][8 * c + 4]);
+                        own += __uint_as_float(hv.x << 16) * w0.x;
+                        own += __uint_as_float(hv.x & 0xFFFF0000u) * w0.y;
+                        own += __uint_as_float(hv.y << 16) * w0.z;
+                        own += __uint_as_float(hv.y & 0xFFFF0000u) * w0.w;
+                        own += __uint_as_float(hv.z << 16) * w1.x;
+                        own += __uint_as_float(hv.z & 0xFFFF0000u) * w1.y;
+                        own += __uint_as_float(hv.w << 16) * w1.z;
+                        own += __uint_as_float(hv.w & 0xFFFF0000u) * w1.w;
+                    }
+                    if (!s_fail)
+                        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::
+                                         "r"(mapa_u32(smem_u32(&s_hr[row]), peer)),
+                                     "r"(__float_as_uint(own)), "r"(mapa_u32(smem_u32(head_full), peer))
+                                     : "memory");
+                    if (!s_fail && !mbar_wait_cluster(head_full, ti & 1)) give_up(32u);
+                    const float e = r0 + row < g.n_rows ? (own + s_hr[row]) + b4 - s_t[row] : 0.0f;
+                    s_dy[row] = scale * e;
+                    sq += e * e;
+                    db4 += scale * e;
+                }
+                asm volatile("bar.sync 1, %0;" ::"r"(kTrEpiWarps * 32) : "memory");
+                const float dy = s_dy[row];
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    const float2 w = *reinterpret_cast<const float2 *>(&s_par[3][cq * 32 + 2 * j]);
+                    hp[j] = pack_bf16x2(dy * w.x * __uint_as_float(r[2 * j]), dy * w.y * __uint_as_float(r[2 * j + 1]));
+                }
+                put_row(sA, hp);
+                hand_over(sA, 0, &mp.dz[2], r0);
+            }
+            column_sum(sA + kFwdBuf, true, dw4);
+            column_sum(sA, false, db3);
+            // dZ2 and dZ1
+#pragma unroll 1
+            for (int s = 3; s < 5; s++) {
+                uint8_t *buf = sA + (s == 3 ? kFwdBuf : 0);
+                tiles_read();
+                wait_acc(5 * ti + s);
+                if (s == 4 && et == 0 && !s_fail)
+                    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
+                                     mapa_u32(smem_u32(peer_free), peer))
+                                 : "memory");
+                uint32_t r[32], gp[32], hp[16];
+                tmem_ld32(tlane + (s == 3 ? 3 : 2) * 128, r);
+                tmem_ld32(tlane + (s == 3 ? 1 : 0) * 128, gp);
+#pragma unroll
+                for (int j = 0; j < 16; j++)
+                    hp[j] = pack_bf16x2(__uint_as_float(r[2 * j]) * __uint_as_float(gp[2 * j]),
+                                        __uint_as_float(r[2 * j + 1]) * __uint_as_float(gp[2 * j + 1]));
+                put_row(buf, hp);
+                hand_over(buf, s == 3 ? 1 : -1, &mp.dz[s == 3 ? 1 : 0], r0);
+                float db = 0.0f;
+                column_sum(buf, false, db);
+                if (s == 3) db2 += db;
+                else db1 += db;
+            }
+        }
+        // this cluster's sums
+        float *sm = g.small + (size_t)cl * kSmall;
+        if (et < 128) {
+            const int c = 128 * (int)rank + et;
+            sm[c] = db1;
+            sm[256 + c] = db2;
+            sm[512 + c] = db3;
+            sm[768 + c] = dw4;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
+            db4 += __shfl_xor_sync(0xFFFFFFFFu, db4, o);
+        }
+        asm volatile("bar.sync 1, %0;" ::"r"(kTrEpiWarps * 32) : "memory");
+        if (cq == 0 && lane == 0) {
+            s_sum[0][q] = sq;
+            s_sum[1][q] = db4;
+        }
+        asm volatile("bar.sync 1, %0;" ::"r"(kTrEpiWarps * 32) : "memory");
+        if (et == 0 && rank == 0) {
+            sm[1024] = (s_sum[0][0] + s_sum[0][1]) + (s_sum[0][2] + s_sum[0][3]);
+            sm[1025] = (s_sum[1][0] + s_sum[1][1]) + (s_sum[1][2] + s_sum[1][3]);
+        }
+        if (sender) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    // after a wait that gave up, copies may still be on their way: let them land before either CTA leaves
+    if (s_fail)
+        for (int i = 0; i < 1000; i++) __nanosleep(1000);
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// ------------------------------------------------------------ weight gradients
+//
+// dW_l = dZ_l^T . H_{l-1}, summed over the batch's rows.  Both operands are
+// the row-major tiles the training kernel wrote, read as they are: a
+// [64 rows][64 columns] box in the 128-byte swizzle is an MN-major operand
+// whose K index is the row, so no transposed copies exist.  One CTA per
+// 128 x 128 output tile (128 x 64 for layer 1: ten tiles in all) and split of
+// the rows; partial sums go to global memory in the accumulator's own order
+// (whole 512-byte lines per warp) and are added by mlp_update.
+
+constexpr int kWgStages = 3;
+constexpr uint32_t kWgBox = 64 * kBK * 2;  // 64 rows x 64 columns: 8 KB
+constexpr size_t kWgSmem = 1024 + kWgStages * 4 * kWgBox + 128;
+constexpr int kWgTiles = 10;                             // 4 of dW3, 4 of dW2, 2 of dW1
+constexpr int kWgFloats = 8 * 128 * 128 + 2 * 128 * 64;  // partial sums of one split
+
+struct WgradMaps {
+    CUtensorMap dz[3], x0, h[2];  // boxes of 64 rows x 64 columns
+};
+
+// shared-memory matrix descriptor: MN-major, 128-byte swizzle; 64-element
+// blocks of the MN index lbo bytes apart, 8-row groups of K 1024 bytes apart
+__device__ __forceinline__ uint64_t umma_desc_mn(uint32_t saddr, uint32_t lbo) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
+    d |= (uint64_t)(lbo >> 4) << 16;
+    d |= (uint64_t)(1024 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+
+__global__ void __launch_bounds__(kThreads, 2)
+    mlp_wgrad(const __grid_constant__ WgradMaps mp, int kt_total, int kt_split, float *part, uint32_t *err) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + kWgStages * 4 * kWgBox);
+    uint64_t *empty = full + kWgStages;
+    uint64_t *done = empty + kWgStages;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
+    __shared__ volatile int s_fail;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tile = blockIdx.x;
+    const int layer = tile < 4 ? 2 : tile < 8 ? 1 : 0;
+    const int mi = layer ? (tile >> 1) & 1 : tile - 8, ni = layer ? tile & 1 : 0;
+    const int nb = layer ? 2 : 1;  // 64-column blocks of the B operand
+    const int kt0 = blockIdx.y * kt_split, nk = min(kt_total, kt0 + kt_split) - kt0;
+    if (threadIdx.x == 0) {
+        s_fail = 0;
+        for (int s = 0; s < kWgStages; s++) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(128));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0 && lane == 0) {
+        const CUtensorMap *ta = &mp.dz[layer], *tb = layer == 2 ? &mp.h[1] : layer == 1 ? &mp.h[0] : &mp.x0;
+        for (int i = 0; i < nk && !s_fail; i++) {
+            const int s = i % kWgStages;
+            if (i >= kWgStages && !mbar_wait(&empty[s], ((i / kWgStages) - 1) & 1)) {
+                atomicOr(err, 1u);
+                s_fail = 1;
+                break;
+            }
+            uint8_t *st = smem + s * 4 * kWgBox;
+            const int r = (kt0 + i) * 64;
+            mbar_expect_tx(&full[s], (2 + nb) * kWgBox);
+            tma_load_2d(st, ta, &full[s], mi * 128, r);
+            tma_load_2d(st + kWgBox, ta, &full[s], mi * 128 + 64, r);
+            tma_load_2d(st + 2 * kWgBox, tb, &full[s], ni * 128, r);
+            if (nb == 2) tma_load_2d(st + 3 * kWgBox, tb, &full[s], ni * 128 + 64, r);
+        }
+    } else if (warp == 1 && lane == 0) {
+        const uint32_t idesc = umma_idesc(nb * 64) | (1u << 15) | (1u << 16);  // A and B MN-major
+        for (int i = 0; i < nk && !s_fail; i++) {
+            const int s = i % kWgStages;
+            if (!mbar_wait(&full[s], (i / kWgStages) & 1)) {
+                atomicOr(err, 2u);
+                s_fail = 1;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t a0 = smem_u32(smem + s * 4 * kWgBox), b0 = a0 + 2 * kWgBox;
+#pragma unroll
+            for (int kk = 0; kk < 4; kk++)  // 16 rows per instruction: two 8-row groups
+                umma_f16(tmem, umma_desc_mn(a0 + kk * 2048, kWgBox), umma_desc_mn(b0 + kk * 2048, kWgBox), idesc,
+                         (i | kk) != 0);
+            umma_commit(&empty[s]);
+        }
+        umma_commit(done);
+    }
+    __syncwarp();
+    const bool ok = mbar_wait(done, 0);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (!ok) atomicOr(err, 4u);
+    const int q = warp & 3, ch = warp >> 2;
+    if (ok && !s_fail) {
+        float4 *out = reinterpret_cast<float4 *>(part + (size_t)blockIdx.y * kWgFloats +
+                                                 (layer ? tile * 16384 : 8 * 16384 + (tile - 8) * 8192));
+#pragma unroll 1
+        for (int c = 0; c < nb; c++) {
+            const int cb = ch * nb + c;  // 32-column block
+            uint32_t r[32];
+            tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cb * 32), r);
+#pragma unroll
+            for (int i = 0; i < 8; i++)
+                out[((cb * 4 + q) * 8 + i) * 32 + lane] =
+                    make_float4(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]), __uint_as_float(r[4 * i + 2]),
+                                __uint_as_float(r[4 * i + 3]));
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128));
+}
+
+// ------------------------------------------------------------------- update
+//
+// The gradients as sums of the partial sums (in a fixed order: the splits of
+// mlp_wgrad, the clusters of mlp_train_fused) and, with adam set, the Adam step
+// (Kingma and Ba 2015, Algorithm 1) on the f32 master weights and the BF16
+// copies of the new weights.  Parameters, moments and gradients are flat
+// arrays in the order W1 b1 W2 b2 W3 b3 W4 b4.
+
+__host__ __device__ constexpr int param_off(int t) {  // first element of tensor t (t = 8: their number)
+    return (t > 0 ? 64 * 256 : 0) + (t > 1 ? 256 : 0) + (t > 2 ? 256 * 256 : 0) + (t > 3 ? 256 : 0) +
+           (t > 4 ? 256 * 256 : 0) + (t > 5 ? 256 : 0) + (t > 6 ? 256 : 0) + (t > 7 ? 1 : 0);
+}
+constexpr int kUpdBlocks = kWgFloats / 4 / 256;  // four weights per thread
+constexpr int kUpdSmallBlocks = (kSmall + 255) / 256;
+
+struct UpdateArgs {
+    const float *part, *small;
+    int splits, clusters;
+    float *G;       // nullable
+    float *loss;    // sum of the squared errors (nullable)
+    float *P, *Mo, *Ve;
+    __nv_bfloat16 *Wb[3], *WbT[3];
+    int adam;
+    float lr, b1, b2, eps, c1, c2;
+};
+
+__device__ __forceinline__ float adam_one(const UpdateArgs &u, float gi, float &m, float &v, float p) {
+    m = u.b1 * m + (1.0f - u.b1) * gi;
+    v = u.b2 * v + (1.0f - u.b2) * gi * gi;
+    return p - u.lr * (m / u.c1) / (sqrtf(v / u.c2) + u.eps);
+}
+
+__global__ void __launch_bounds__(256) mlp_update(UpdateArgs u) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (blockIdx.x < kUpdBlocks) {
+        // four neighbouring weights of one row, in mlp_wgrad's order
+        const int i4 = blockIdx.x * 256 + threadIdx.x;
+        const int tile = i4 < 8 * 4096 ? i4 >> 12 : 8 + ((i4 - 8 * 4096) >> 11);
+        const int layer = tile < 4 ? 2 : tile < 8 ? 1 : 0;
+        const int mi = layer ? (tile >> 1) & 1 : tile - 8, ni = layer ? tile & 1 : 0;
+        const int in_tile = layer ? i4 & 4095 : i4 & 2047;
+        const int o = mi * 128 + ((in_tile >> 8) & 3) * 32 + (in_tile & 31);
+        const int k = ni * 128 + (in_tile >> 10) * 32 + ((in_tile >> 5) & 7) * 4;
+        const int n_in = layer ? 256 : 64;
+        const int flat = param_off(2 * layer) + o * n_in + k;
+        float4 gr = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        const float4 *pp = reinterpret_cast<const float4 *>(u.part) + i4;
+#pragma unroll 8
+        for (int s = 0; s < u.splits; s++) {
+            const float4 a = pp[(size_t)s * (kWgFloats / 4)];
+            gr.x += a.x;
+            gr.y += a.y;
+            gr.z += a.z;
+            gr.w += a.w;
+        }
+        if (u.G) *reinterpret_cast<float4 *>(u.G + flat) = gr;
+        if (u.adam) {
+            float4 p = *reinterpret_cast<const float4 *>(u.P + flat);
+            float4 m = *reinterpret_cast<const float4 *>(u.Mo + flat), v = *reinterpret_cast<const float4 *>(u.Ve + flat);
+            p.x = adam_one(u, gr.x, m.x, v.x, p.x);
+            p.y = adam_one(u, gr.y, m.y, v.y, p.y);
+            p.z = adam_one(u, gr.z, m.z, v.z, p.z);
+            p.w = adam_one(u, gr.w, m.w, v.w, p.w);
+            *reinterpret_cast<float4 *>(u.P + flat) = p;
+            *reinterpret_cast<float4 *>(u.Mo + flat) = m;
+            *reinterpret_cast<float4 *>(u.Ve + flat) = v;
+            const uint2 w = make_uint2(pack_bf16x2(p.x, p.y), pack_bf16x2(p.z, p.w));
+            *reinterpret_cast<uint2 *>(u.Wb[layer] + o * n_in + k) = w;
+            if (layer) {
+                __nv_bfloat16 *wt = u.WbT[layer] + k * 256 + o;
+                const float pv[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+                for (int j = 0; j < 4; j++) wt[j * 256] = __float2bfloat16_rn(pv[j]);
+            }
+        }
+        return;
+    }
+    const int i = (blockIdx.x - kUpdBlocks) * 256 + threadIdx.x;
+    if (i >= kSmall) return;
+    float gr = 0.0f;
+#pragma unroll 8
+    for (int c = 0; c < u.clusters; c++) gr += u.small[(size_t)c * kSmall + i];
+    if (i == 1024) {
+        if (u.loss) *u.loss = gr;
+        return;
+    }
+    const int t = i == 1025 ? 7 : i >= 768 ? 6 : 2 * (i >> 8) + 1;
+    const int flat = param_off(t) + (i == 1025 ? 0 : i & 255);
+    if (u.G) u.G[flat] = gr;
+    if (u.adam) {
+        float m = u.Mo[flat], v = u.Ve[flat];
+        u.P[flat] = adam_one(u, gr, m, v, u.P[flat]);
+        u.Mo[flat] = m;
+        u.Ve[flat] = v;
+    }
+}
+
+// the Adam step with the gradients in u.G (the BF16 copies follow separately)
+__global__ void adam_given(UpdateArgs u) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= param_off(8)) return;
+    float m = u.Mo[i], v = u.Ve[i];
+    u.P[i] = adam_one(u, u.G[i], m, v, u.P[i]);
+    u.Mo[i] = m;
+    u.Ve[i] = v;
 }
 
 // ------------------------------------------------------------- host side
@@ -969,26 +1430,31 @@ int make_map(CUtensorMap *map, const void *ptr, uint64_t rows, uint64_t cols, ui
     return LPSIM_OK;
 }
 
-template <int BN, int EPI>
-int launch_gemm(const CUtensorMap &a, const CUtensorMap &b, const GemmArgs &g_in, int splits, cudaStream_t st) {
-    // short K (the layer GEMMs, at most 4 slices): a 2-deep ring, so two CTAs
-    // share an SM and one's epilogue overlaps the other's loads; long K (the
-    // split weight-gradient GEMMs): the full ring
-    GemmArgs g = g_in;
-    g.stages = (BN == 256 && g.ktiles_per_split <= 4) ? 2 : kStages;
-    const size_t max_smem = 1024 + kStages * (size_t)(kBM * kBK * 2 + BN * kBK * 2) + (2 * kStages + 1) * 8 + 16;
-    const size_t smem = 1024 + g.stages * (size_t)(kBM * kBK * 2 + BN * kBK * 2) + (2 * g.stages + 1) * 8 + 16;
-    if ((size_t)g.stages * (kBM * kBK * 2 + BN * kBK * 2) < (size_t)kThreads / 32 * 2 * 32 * 33 * 4)
-        return fail(LPSIM_E_STATE, "GEMM epilogue staging does not fit in the operand ring");
-    static bool attr_set = false;
-    if (!attr_set) {
-        CU(cudaFuncSetAttribute(gemm_bf16_tn<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem));
-        attr_set = true;
-    }
+template <int BN>
+int launch_gemm(const CUtensorMap &a, const CUtensorMap &b, const GemmArgs &g, cudaStream_t st) {
+    const size_t smem = 1024 + kStages * (size_t)(kBM * kBK * 2 + BN * kBK * 2) + (2 * kStages + 1) * 8 + 16;
+    CU(cudaFuncSetAttribute(gemm_bf16_tn<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (g.M % kBM != 0 || g.N % BN != 0) return fail(LPSIM_E_INVALID_ARG, "GEMM shape not a multiple of the tile");
-    dim3 grid(g.M / kBM, g.N / BN, splits);
-    gemm_bf16_tn<BN, EPI><<<grid, kThreads, smem, st>>>(a, b, g);
+    gemm_bf16_tn<BN><<<dim3(g.M / kBM, g.N / BN), kThreads, smem, st>>>(a, b, g);
     CU(cudaGetLastError());
+    return LPSIM_OK;
+}
+
+// a launch that may start before the previous kernel of the stream has
+// finished (the kernel waits for it itself, griddepcontrol)
+template <class... P, class... A>
+int launch_dependent(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, const A &...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    CU(cudaLaunchKernelEx(&cfg, kernel, args...));
     return LPSIM_OK;
 }
 
@@ -1004,17 +1470,23 @@ struct lpsim_mlp {
     int nf = 9;       // real input features
     int B = 8192;     // rows per batch (multiple of 128)
     std::vector<void *> blocks;
-    // parameters: f32 master, Adam moments, gradients
-    float *P[8] = {}, *G[8] = {}, *Mo[8] = {}, *Ve[8] = {};
+    // parameters: f32 master, Adam moments, gradients; each one flat array in
+    // the order W1 b1 W2 b2 W3 b3 W4 b4, P[i] the tensors of the first.  The
+    // loss and the error word follow the gradients, so one copy brings all three
+    float *Pf = nullptr, *Gf = nullptr, *Mf = nullptr, *Vf = nullptr, *P[8] = {};
     int sz[8] = {};
     // bf16 weights (W1..W3) and transposes (W2^T, W3^T)
     __nv_bfloat16 *Wb[3] = {}, *WbT[3] = {};
-    // activations for one batch
-    __nv_bfloat16 *X0, *X0T, *H[3], *HT[3], *dZ[3], *dZT[3];
-    float *Gp[3];  // GELU'(Z_l) of the last training forward (f32)
-    float *y, *t, *dy, *Xf, *loss_acc, *colpart;
+    // one batch: inputs as given, inputs and hidden activations in bf16, the
+    // backward's dZ1..3
+    float *Xf, *t, *y;
+    __nv_bfloat16 *X0, *H[2], *dZ[3];
+    float *small, *part;  // partial sums of mlp_train_fused (per cluster) and mlp_wgrad (per split)
     uint32_t *err;
-    CUtensorMap mX0, mW[3], mH[3], mWT[3], mdZ[3], mdZT[3], mHT[3], mX0T;
+    CUtensorMap mX0, mW[3];
+    TrainMaps tmaps;
+    WgradMaps gmaps;
+    std::vector<float> h_flat;  // gradients or parameters on their way to the caller's tensors
     int adam_t = 0;
     uint64_t launches = 0;
     // training pool: samples kept on the device (grown by doubling), and the
@@ -1048,11 +1520,11 @@ namespace {
 
 const int kDims[5] = {64, 256, 256, 256, 1};
 
-int column_sums(const __nv_bfloat16 *A, int rows, int cols, const float *rowscale, float *out, float *part,
-                cudaStream_t st) {
-    column_partials<<<dim3(cols / 32, kSumBands), dim3(32, 8), 0, st>>>(A, rows, cols, rowscale, part);
-    reduce_bands<<<cols, 256, 0, st>>>(part, kSumBands, cols, out);
-    CU(cudaGetLastError());
+constexpr int kLossAt = (param_off(8) + 3) / 4 * 4, kErrAt = kLossAt + 1;  // in the gradients' flat array
+
+int err_status(uint32_t e) {
+    if (e & 64u) return fail(LPSIM_E_TIMEOUT, "training-pool permutation walk exceeded its bound");
+    if (e) return fail(LPSIM_E_TIMEOUT, "tensor-core GEMM wait gave up (code " + std::to_string(e) + ")");
     return LPSIM_OK;
 }
 
@@ -1060,9 +1532,7 @@ int mlp_check_err(lpsim_mlp *m) {
     uint32_t e = 0;
     CU(cudaMemcpyAsync(&e, m->err, 4, cudaMemcpyDeviceToHost, m->stream));
     CU(cudaStreamSynchronize(m->stream));
-    if (e & 64u) return fail(LPSIM_E_TIMEOUT, "training-pool permutation walk exceeded its bound");
-    if (e) return fail(LPSIM_E_TIMEOUT, "tensor-core GEMM wait gave up (code " + std::to_string(e) + ")");
-    return LPSIM_OK;
+    return err_status(e);
 }
 
 int refresh_weights(lpsim_mlp *m) {
@@ -1074,28 +1544,80 @@ int refresh_weights(lpsim_mlp *m) {
     return LPSIM_OK;
 }
 
-// One Adam step (Kingma and Ba 2015, Algorithm 1) with the gradients in G[]:
-// beta1 0.9, beta2 0.999, eps 1e-8 as FP32 constants; the bias corrections
-// 1 - beta^t are formed in double from those FP32 values and rounded once
-// (in float arithmetic 1 - beta2^t loses most of its digits to cancellation);
-// then the BF16 weight copies are refreshed.
-int adam_step(lpsim_mlp *m, float lr) {
+// The next Adam step's constants: beta1 0.9, beta2 0.999, eps 1e-8 as FP32
+// constants; the bias corrections 1 - beta^t are formed in double from those
+// FP32 values and rounded once (in float arithmetic 1 - beta2^t loses most of
+// its digits to cancellation).
+void adam_constants(lpsim_mlp *m, float lr, UpdateArgs &u) {
     m->adam_t++;
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float c1 = (float)(1.0 - std::pow((double)b1, (double)m->adam_t));
-    const float c2 = (float)(1.0 - std::pow((double)b2, (double)m->adam_t));
-    for (int i = 0; i < 8; i++) {
-        adam_update<<<(m->sz[i] + 255) / 256, 256, 0, m->stream>>>(m->P[i], m->G[i], m->Mo[i], m->Ve[i], m->sz[i], lr,
-                                                                  b1, b2, eps, c1, c2);
-        m->launches++;
-    }
-    CU(cudaGetLastError());
-    return refresh_weights(m);
+    u.adam = 1;
+    u.lr = lr;
+    u.b1 = 0.9f;
+    u.b2 = 0.999f;
+    u.eps = 1e-8f;
+    u.c1 = (float)(1.0 - std::pow((double)u.b1, (double)m->adam_t));
+    u.c2 = (float)(1.0 - std::pow((double)u.b2, (double)m->adam_t));
 }
 
-// forward of rows [0, B) already packed in X0; keep = training buffers
-// training keeps the pre-activations (for GELU') and transposed activations
-// (for the weight gradients); inference writes only the activations
+// Splits of mlp_wgrad's rows (kt slices of 64): two CTAs per SM at most (ten
+// tiles per split), and at least four slices each.  Measured, us per training
+// step with caps of 15 / 30 splits: 8192 rows 41.6 / 40.5, 32768 rows 126 /
+// 120, 155648 rows 455 / 440; with at least 2 / 4 / 16 slices: 1024 rows 34.9 /
+// 36.4 / 39.6, 8192 rows 40.6 / 40.5 / 42.7.
+int wgrad_splits(const lpsim_mlp *m, int kt) {
+    return std::max(1, std::min(kt / 4, 2 * m->n_sm / kWgTiles));
+}
+
+// forward and backward of n rows (X, t: the batch in order, or drawn from a
+// pool of pool_n rows from position pos0 of its shuffled passes on), leaving
+// the partial sums for mlp_update
+int train_core(lpsim_mlp *m, const float *X, const float *t, uint32_t n, uint64_t pool_n, uint32_t h, uint64_t seed,
+               uint64_t pos0, UpdateArgs &u) {
+    CU(cudaFuncSetAttribute(mlp_train_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrSmem));
+    CU(cudaFuncSetAttribute(mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem));
+    TrainArgs g{};
+    g.n_rows = (int)n;
+    g.n_tiles = (int)((n + kBM - 1) / kBM);
+    g.nf = m->nf;
+    g.l1_k16 = (m->nf + 15) / 16;
+    g.X = X;
+    g.t = t;
+    g.pool_n = pool_n;
+    g.seed = seed;
+    g.pos0 = pos0;
+    g.h = h;
+    g.b1 = m->P[1];
+    g.b2 = m->P[3];
+    g.b3 = m->P[5];
+    g.w4 = m->P[6];
+    g.b4 = m->P[7];
+    g.small = m->small;
+    g.err = m->err;
+    u.clusters = std::min(g.n_tiles, m->n_sm / 2);
+    TRY(launch_dependent(mlp_train_fused, dim3(2 * u.clusters), kTrThreads, kTrSmem, m->stream, m->tmaps, g));
+    const int kt = 2 * g.n_tiles, want = wgrad_splits(m, kt), per = (kt + want - 1) / want;
+    u.splits = (kt + per - 1) / per;
+    TRY(launch_dependent(mlp_wgrad, dim3(kWgTiles, u.splits), kThreads, kWgSmem, m->stream, m->gmaps, kt, per, m->part,
+                         m->err));
+    m->launches += 2;
+    u.part = m->part;
+    u.small = m->small;
+    u.P = m->Pf;
+    u.Mo = m->Mf;
+    u.Ve = m->Vf;
+    for (int l = 0; l < 3; l++) {
+        u.Wb[l] = m->Wb[l];
+        u.WbT[l] = m->WbT[l];
+    }
+    return LPSIM_OK;
+}
+
+int train_update(lpsim_mlp *m, const UpdateArgs &u) {
+    m->launches++;
+    return launch_dependent(mlp_update, dim3(kUpdBlocks + kUpdSmallBlocks), 256, 0, m->stream, u);
+}
+
+// inference forward of the rows packed in X0: every layer in one kernel, activations kept on chip
 int forward_fused(lpsim_mlp *m, float *y_out = nullptr) {
     static bool attr_set = false;
     if (!attr_set) {
@@ -1119,105 +1641,22 @@ int forward_fused(lpsim_mlp *m, float *y_out = nullptr) {
     return LPSIM_OK;
 }
 
-int forward_batch(lpsim_mlp *m, bool training = true) {
-    // inference: every layer in one kernel, activations kept on chip
-    if (!training) return forward_fused(m);
-    cudaStream_t st = m->stream;
-    for (int l = 0; l < 3; l++) {
-        GemmArgs g{};
-        g.M = m->B;
-        g.N = 256;
-        g.K = kDims[l];
-        g.ktiles_per_split = (g.K + kBK - 1) / kBK;
-        g.bias = m->P[2 * l + 1];
-        g.gout = training ? m->Gp[l] : nullptr;
-        g.hout = m->H[l];
-        g.htout = training ? m->HT[l] : nullptr;
-        g.err = m->err;
-        const CUtensorMap &a = l == 0 ? m->mX0 : m->mH[l - 1];
-        if (l < 2) {
-            TRY((launch_gemm<256, kEpiGelu>(a, m->mW[l], g, 1, st)));
-        } else {
-            g.w4 = m->P[6];
-            g.b4 = m->P[7];
-            g.yout = m->y;
-            if (!training) g.hout = nullptr;  // inference needs only y
-            TRY((launch_gemm<256, kEpiGeluHead>(a, m->mW[l], g, 1, st)));
-        }
-        m->launches++;
-    }
-    return LPSIM_OK;
-}
-
-// backward of the batch in the buffers (after forward_batch); fills G[]
-int backward_batch(lpsim_mlp *m, int n_real) {
-    cudaStream_t st = m->stream;
-    const int B = m->B;
-    for (int i = 0; i < 8; i++) CU(cudaMemsetAsync(m->G[i], 0, m->sz[i] * 4, st));
-    head_backward<<<dim3(B / 32, 256 / 32), dim3(32, 8), 0, st>>>(m->y, m->t, n_real, B, m->P[6], m->Gp[2], m->dZ[2],
-                                                                 m->dZT[2], m->dy, m->loss_acc);
-    // dW4 = sum_r dy[r] H3[r][:], db4 = sum dy
-    TRY(column_sums(m->H[2], B, 256, m->dy, m->G[6], m->colpart, st));
-    vector_partials<<<kSumBands, 256, 0, st>>>(m->dy, B, m->colpart);
-    reduce_bands<<<1, 256, 0, st>>>(m->colpart, kSumBands, 1, m->G[7]);
-    m->launches += 5;
-    for (int l = 2; l >= 0; l--) {
-        // dW_l = dZ_l^T . H_{l-1}   (A = dZ_l^T [256 x B], B = H_{l-1}^T [in x B])
-        GemmArgs g{};
-        g.M = 256;
-        g.N = kDims[l];
-        g.K = B;
-        const int kt = B / kBK;
-        const int splits = kt >= 64 ? 64 : kt;
-        g.ktiles_per_split = (kt + splits - 1) / splits;
-        g.fout = m->G[2 * l];
-        g.err = m->err;
-        const CUtensorMap &bT = l == 0 ? m->mX0T : m->mHT[l - 1];
-        if (g.N == 256) {
-            TRY((launch_gemm<256, kEpiAtomic>(m->mdZT[l], bT, g, splits, st)));
-        } else {
-            TRY((launch_gemm<64, kEpiAtomic>(m->mdZT[l], bT, g, splits, st)));
-        }
-        if (l == 2) {
-            // db3 = column sums of dZ3 (db2, db1 come from the GELU' epilogues below)
-            TRY(column_sums(m->dZ[l], B, 256, nullptr, m->G[2 * l + 1], m->colpart, st));
-            m->launches += 2;
-        }
-        m->launches += 1;
-        if (l > 0) {
-            // dZ_{l-1} = (dZ_l . W_l) * GELU'(Z_{l-1})   (B operand = W_l^T [in x out])
-            GemmArgs h{};
-            h.M = B;
-            h.N = 256;
-            h.K = 256;
-            h.ktiles_per_split = 4;
-            h.gprev = m->Gp[l - 1];
-            h.colpart = m->colpart;
-            h.hout = m->dZ[l - 1];
-            h.htout = m->dZT[l - 1];
-            h.err = m->err;
-            TRY((launch_gemm<256, kEpiDgelu>(m->mdZ[l], m->mWT[l], h, 1, st)));
-            // db_{l-1} = column sums of dZ_{l-1}: the per-row-tile sums of the epilogue, added in order
-            reduce_bands<<<256, 256, 0, st>>>(m->colpart, B / kBM, 256, m->G[2 * (l - 1) + 1]);
-            m->launches += 2;
-        }
-    }
-    CU(cudaGetLastError());
-    return LPSIM_OK;
-}
-
-// transposed: also the transposed input copy the weight gradients read (training only)
-int pack_batch(lpsim_mlp *m, const float *X_host, const float *t_host, uint64_t n, bool transposed = true) {
-    cudaStream_t st = m->stream;
-    CU(cudaMemcpyAsync(m->Xf, X_host, n * m->nf * 4, cudaMemcpyHostToDevice, st));
-    if (t_host) {
-        CU(cudaMemsetAsync(m->t, 0, m->B * 4, st));
-        CU(cudaMemcpyAsync(m->t, t_host, n * 4, cudaMemcpyHostToDevice, st));
-    }
-    pack_inputs<<<dim3(m->B / 32, 2), dim3(32, 8), 0, st>>>(m->Xf, (int)n, m->nf, m->B, m->X0,
-                                                           transposed ? m->X0T : nullptr);
+int pack_batch(lpsim_mlp *m, const float *X_host, uint64_t n) {
+    CU(cudaMemcpyAsync(m->Xf, X_host, n * m->nf * 4, cudaMemcpyHostToDevice, m->stream));
+    pack_inputs<<<dim3(m->B / 32, 2), dim3(32, 8), 0, m->stream>>>(m->Xf, (int)n, m->nf, m->X0);
     m->launches++;
     CU(cudaGetLastError());
+    return LPSIM_OK;
+}
+
+// a flat parameter-shaped device array into the caller's tensors (each
+// nullable): one copy, then host copies
+int flat_to_tensors(lpsim_mlp *m, const float *flat, float *const *tensors) {
+    m->h_flat.resize(kErrAt + 1);
+    CU(cudaMemcpyAsync(m->h_flat.data(), flat, (kErrAt + 1) * 4, cudaMemcpyDeviceToHost, m->stream));
+    CU(cudaStreamSynchronize(m->stream));
+    for (int i = 0; i < 8 && tensors; i++)
+        if (tensors[i]) std::memcpy(tensors[i], m->h_flat.data() + param_off(i), (size_t)m->sz[i] * 4);
     return LPSIM_OK;
 }
 
@@ -1252,41 +1691,46 @@ int lpsim_mlp_create(lpsim_mlp **out, uint32_t n_features, uint32_t batch, uint6
         m->sz[2 * l] = kDims[l + 1] * kDims[l];
         m->sz[2 * l + 1] = kDims[l + 1];
     }
-    for (int i = 0; i < 8; i++) {
-        m->P[i] = (float *)m->alloc(m->sz[i] * 4);
-        m->G[i] = (float *)m->alloc(m->sz[i] * 4);
-        m->Mo[i] = (float *)m->alloc(m->sz[i] * 4);
-        m->Ve[i] = (float *)m->alloc(m->sz[i] * 4);
-        if (!m->P[i] || !m->G[i] || !m->Mo[i] || !m->Ve[i]) return bail(fail(LPSIM_E_OOM, "device allocation failed"));
-    }
+    const size_t flat = (size_t)(kErrAt + 1) * 4;
+    m->Pf = (float *)m->alloc(flat);
+    m->Gf = (float *)m->alloc(flat);
+    m->Mf = (float *)m->alloc(flat);
+    m->Vf = (float *)m->alloc(flat);
+    const int max_kt = 2 * (B / kBM);
+    m->small = (float *)m->alloc((size_t)std::max(1, std::min(B / kBM, m->n_sm / 2)) * kSmall * 4);
+    m->part = (float *)m->alloc((size_t)wgrad_splits(m, max_kt) * kWgFloats * 4);
+    if (!m->Pf || !m->Gf || !m->Mf || !m->Vf || !m->small || !m->part)
+        return bail(fail(LPSIM_E_OOM, "device allocation failed"));
+    for (int i = 0; i < 8; i++) m->P[i] = m->Pf + param_off(i);
+    m->err = reinterpret_cast<uint32_t *>(m->Gf + kErrAt);
     for (int l = 0; l < 3; l++) {
         m->Wb[l] = (__nv_bfloat16 *)m->alloc(kDims[l + 1] * kDims[l] * 2);
-        m->WbT[l] = (__nv_bfloat16 *)m->alloc(kDims[l + 1] * kDims[l] * 2);
-        m->H[l] = (__nv_bfloat16 *)m->alloc((size_t)B * 256 * 2);
-        m->HT[l] = (__nv_bfloat16 *)m->alloc((size_t)B * 256 * 2);
+        if (l > 0) m->WbT[l] = (__nv_bfloat16 *)m->alloc(kDims[l + 1] * kDims[l] * 2);
+        if (l < 2) m->H[l] = (__nv_bfloat16 *)m->alloc((size_t)B * 256 * 2);
         m->dZ[l] = (__nv_bfloat16 *)m->alloc((size_t)B * 256 * 2);
-        m->dZT[l] = (__nv_bfloat16 *)m->alloc((size_t)B * 256 * 2);
-        m->Gp[l] = (float *)m->alloc((size_t)B * 256 * 4);
+        if (!m->Wb[l] || (l > 0 && !m->WbT[l]) || (l < 2 && !m->H[l]) || !m->dZ[l])
+            return bail(fail(LPSIM_E_OOM, "device allocation failed"));
     }
     m->X0 = (__nv_bfloat16 *)m->alloc((size_t)B * 64 * 2);
-    m->X0T = (__nv_bfloat16 *)m->alloc((size_t)B * 64 * 2);
-    m->Xf = (float *)m->alloc((size_t)B * 64 * 4);
+    m->Xf = (float *)m->alloc((size_t)B * n_features * 4);
     m->y = (float *)m->alloc((size_t)B * 4);
     m->t = (float *)m->alloc((size_t)B * 4);
-    m->dy = (float *)m->alloc((size_t)B * 4);
-    m->loss_acc = (float *)m->alloc(16);
-    m->colpart = (float *)m->alloc((size_t)std::max(kSumBands, B / kBM) * 256 * 4);
-    m->err = (uint32_t *)m->alloc(16);
-    if (!m->err || !m->X0 || !m->Xf) return bail(fail(LPSIM_E_OOM, "device allocation failed"));
-    if (cudaMemsetAsync(m->err, 0, 16, m->stream) != cudaSuccess) return bail(fail(LPSIM_E_CUDA, "memset"));
-    // tensor maps of every GEMM operand
+    if (!m->X0 || !m->Xf || !m->y || !m->t) return bail(fail(LPSIM_E_OOM, "device allocation failed"));
+    if (cudaMemsetAsync(m->err, 0, 4, m->stream) != cudaSuccess) return bail(fail(LPSIM_E_CUDA, "memset"));
+    // tensor maps of every operand
     int rc;
-    if ((rc = make_map(&m->mX0, m->X0, B, 64, kBM)) || (rc = make_map(&m->mX0T, m->X0T, 64, B, 64))) return bail(rc);
+    TrainMaps &tm = m->tmaps;
+    WgradMaps &gm = m->gmaps;
+    const __nv_bfloat16 *wsrc[5] = {m->Wb[0], m->Wb[1], m->Wb[2], m->WbT[2], m->WbT[1]};
+    if ((rc = make_map(&m->mX0, m->X0, B, 64, kBM)) || (rc = make_map(&gm.x0, m->X0, B, 64, 64))) return bail(rc);
+    tm.x0 = m->mX0;
+    for (int s = 0; s < 5; s++)
+        if ((rc = make_map(&tm.w[s], wsrc[s], 256, s == 0 ? 64 : 256, 128))) return bail(rc);
     for (int l = 0; l < 3; l++) {
         if ((rc = make_map(&m->mW[l], m->Wb[l], 256, kDims[l], 256)) ||
-            (rc = make_map(&m->mWT[l], m->WbT[l], kDims[l], 256, kDims[l] == 64 ? 64 : 256)) ||
-            (rc = make_map(&m->mH[l], m->H[l], B, 256, kBM)) || (rc = make_map(&m->mHT[l], m->HT[l], 256, B, 256)) ||
-            (rc = make_map(&m->mdZ[l], m->dZ[l], B, 256, kBM)) || (rc = make_map(&m->mdZT[l], m->dZT[l], 256, B, kBM)))
+            (rc = make_map(&tm.dz[l], m->dZ[l], B, 256, 32)) || (rc = make_map(&gm.dz[l], m->dZ[l], B, 256, 64)))
+            return bail(rc);
+        if (l < 2 && ((rc = make_map(&tm.h[l], m->H[l], B, 256, 32)) || (rc = make_map(&gm.h[l], m->H[l], B, 256, 64))))
             return bail(rc);
     }
     // He initialisation (host, seeded), then upload
@@ -1303,10 +1747,8 @@ int lpsim_mlp_create(lpsim_mlp **out, uint32_t n_features, uint32_t batch, uint6
             cudaMemcpy(m->P[2 * l + 1], b.data(), b.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess)
             return bail(fail(LPSIM_E_CUDA, "parameter upload failed"));
     }
-    for (int i = 0; i < 8; i++) {
-        cudaMemsetAsync(m->Mo[i], 0, m->sz[i] * 4, m->stream);
-        cudaMemsetAsync(m->Ve[i], 0, m->sz[i] * 4, m->stream);
-    }
+    cudaMemsetAsync(m->Mf, 0, flat, m->stream);
+    cudaMemsetAsync(m->Vf, 0, flat, m->stream);
     if ((rc = refresh_weights(m))) return bail(rc);
     if (cudaStreamSynchronize(m->stream) != cudaSuccess) return bail(fail(LPSIM_E_CUDA, "init failed"));
     *out = m;
@@ -1318,9 +1760,9 @@ int lpsim_mlp_set_params(lpsim_mlp *m, const float *const *tensors) {
     for (int i = 0; i < 8; i++) {
         if (!tensors[i]) return fail(LPSIM_E_INVALID_ARG, "parameter tensor is NULL");
         CU(cudaMemcpyAsync(m->P[i], tensors[i], m->sz[i] * 4, cudaMemcpyHostToDevice, m->stream));
-        CU(cudaMemsetAsync(m->Mo[i], 0, m->sz[i] * 4, m->stream));
-        CU(cudaMemsetAsync(m->Ve[i], 0, m->sz[i] * 4, m->stream));
     }
+    CU(cudaMemsetAsync(m->Mf, 0, param_off(8) * 4, m->stream));
+    CU(cudaMemsetAsync(m->Vf, 0, param_off(8) * 4, m->stream));
     m->adam_t = 0;
     TRY(refresh_weights(m));
     CU(cudaStreamSynchronize(m->stream));
@@ -1329,10 +1771,7 @@ int lpsim_mlp_set_params(lpsim_mlp *m, const float *const *tensors) {
 
 int lpsim_mlp_get_params(lpsim_mlp *m, float *const *tensors) {
     if (!m || !tensors) return fail(LPSIM_E_INVALID_ARG, "NULL argument");
-    CU(cudaStreamSynchronize(m->stream));
-    for (int i = 0; i < 8; i++)
-        if (tensors[i]) CU(cudaMemcpy(tensors[i], m->P[i], m->sz[i] * 4, cudaMemcpyDeviceToHost));
-    return LPSIM_OK;
+    return flat_to_tensors(m, m->Pf, tensors);
 }
 
 int lpsim_mlp_forward(lpsim_mlp *m, uint64_t n, const float *X, float *y) {
@@ -1357,11 +1796,11 @@ int lpsim_mlp_forward(lpsim_mlp *m, uint64_t n, const float *X, float *y) {
     }
     for (uint64_t r0 = 0; r0 < n; r0 += B) {
         const uint64_t nb = std::min<uint64_t>(B, n - r0);
-        TRY(pack_batch(m, X + r0 * m->nf, nullptr, nb, false));
+        TRY(pack_batch(m, X + r0 * m->nf, nb));
         if (n > B) {
             TRY(forward_fused(m, m->y_all + r0));
         } else {
-            TRY(forward_batch(m, false));
+            TRY(forward_fused(m));
             CU(cudaMemcpyAsync(y + r0, m->y, nb * 4, cudaMemcpyDeviceToHost, m->stream));
         }
     }
@@ -1373,20 +1812,18 @@ int lpsim_mlp_forward(lpsim_mlp *m, uint64_t n, const float *X, float *y) {
 int lpsim_mlp_grad(lpsim_mlp *m, uint64_t n, const float *X, const float *t, float *loss, float *const *grads) {
     if (!m || !X || !t) return fail(LPSIM_E_INVALID_ARG, "NULL argument");
     if (n == 0 || n > (uint64_t)m->B) return fail(LPSIM_E_INVALID_ARG, "n must be 1..batch");
-    TRY(pack_batch(m, X, t, n));
-    TRY(forward_batch(m));
-    CU(cudaMemsetAsync(m->loss_acc, 0, 4, m->stream));
-    TRY(backward_batch(m, (int)n));
-    CU(cudaStreamSynchronize(m->stream));
-    TRY(mlp_check_err(m));
-    if (loss) {
-        float s = 0.0f;
-        CU(cudaMemcpy(&s, m->loss_acc, 4, cudaMemcpyDeviceToHost));
-        *loss = s / (float)n;
-    }
-    if (grads)
-        for (int i = 0; i < 8; i++)
-            if (grads[i]) CU(cudaMemcpy(grads[i], m->G[i], m->sz[i] * 4, cudaMemcpyDeviceToHost));
+    CU(cudaMemcpyAsync(m->Xf, X, n * m->nf * 4, cudaMemcpyHostToDevice, m->stream));
+    CU(cudaMemcpyAsync(m->t, t, n * 4, cudaMemcpyHostToDevice, m->stream));
+    UpdateArgs u{};
+    TRY(train_core(m, m->Xf, m->t, (uint32_t)n, 0, 0, 0, 0, u));
+    u.G = m->Gf;
+    u.loss = m->Gf + kLossAt;
+    TRY(train_update(m, u));
+    TRY(flat_to_tensors(m, m->Gf, grads));
+    uint32_t e;
+    std::memcpy(&e, &m->h_flat[kErrAt], 4);
+    TRY(err_status(e));
+    if (loss) *loss = m->h_flat[kLossAt] / (float)n;
     return LPSIM_OK;
 }
 
@@ -1445,18 +1882,13 @@ int lpsim_mlp_train_pool(lpsim_mlp *m, uint32_t steps, float lr, uint64_t shuffl
     while ((1ull << (2 * h)) < n) h++;
     const uint32_t nb = (uint32_t)std::min<uint64_t>(m->B, n);
     cudaStream_t st = m->stream;
-    CU(cudaMemsetAsync(m->t, 0, m->B * 4, st));
     for (uint32_t s = 0; s < steps; s++) {
-        // the next minibatch of the shuffled passes, gathered on the device
-        gather_batch<<<(nb + 255) / 256, 256, 0, st>>>(m->pool_X, m->pool_t, n, m->nf, h, shuffle_seed,
-                                                       (uint64_t)s * nb, nb, m->Xf, m->t, m->err);
-        pack_inputs<<<dim3(m->B / 32, 2), dim3(32, 8), 0, st>>>(m->Xf, (int)nb, m->nf, m->B, m->X0, m->X0T);
-        m->launches += 2;
-        TRY(forward_batch(m));
-        CU(cudaMemsetAsync(m->loss_acc, 0, 4, st));
-        TRY(backward_batch(m, (int)nb));
-        TRY(adam_step(m, lr));
-        CU(cudaMemcpyAsync(m->loss_hist + s, m->loss_acc, 4, cudaMemcpyDeviceToDevice, st));
+        // the next minibatch of the shuffled passes, drawn by the training kernel
+        UpdateArgs u{};
+        TRY(train_core(m, m->pool_X, m->pool_t, nb, n, h, shuffle_seed, (uint64_t)s * nb, u));
+        adam_constants(m, lr, u);
+        u.loss = m->loss_hist + s;
+        TRY(train_update(m, u));
     }
     CU(cudaGetLastError());
     if (losses && steps) {
@@ -1483,8 +1915,18 @@ int lpsim_mlp_apply_grads(lpsim_mlp *m, const float *const *grads, float lr) {
     for (int i = 0; i < 8; i++)
         if (!grads[i]) return fail(LPSIM_E_INVALID_ARG, "gradient tensor is NULL");
     CU(cudaStreamSynchronize(m->stream));
-    for (int i = 0; i < 8; i++) CU(cudaMemcpyAsync(m->G[i], grads[i], m->sz[i] * 4, cudaMemcpyHostToDevice, m->stream));
-    TRY(adam_step(m, lr));
+    for (int i = 0; i < 8; i++)
+        CU(cudaMemcpyAsync(m->Gf + param_off(i), grads[i], m->sz[i] * 4, cudaMemcpyHostToDevice, m->stream));
+    UpdateArgs u{};
+    u.G = m->Gf;
+    u.P = m->Pf;
+    u.Mo = m->Mf;
+    u.Ve = m->Vf;
+    adam_constants(m, lr, u);
+    adam_given<<<(param_off(8) + 255) / 256, 256, 0, m->stream>>>(u);
+    m->launches++;
+    CU(cudaGetLastError());
+    TRY(refresh_weights(m));
     CU(cudaStreamSynchronize(m->stream));
     return LPSIM_OK;
 }
@@ -1513,10 +1955,9 @@ int lpsim_mlp_gemm_test(uint32_t M, uint32_t N, uint32_t K, const uint16_t *A, c
         g.M = (int)M;
         g.N = (int)N;
         g.K = (int)K;
-        g.ktiles_per_split = (int)(K / kBK);
         g.fout = (float *)dD;
         g.err = (uint32_t *)dE;
-        rc = N == 64 ? launch_gemm<64, kEpiStore>(ma, mb, g, 1, st) : launch_gemm<256, kEpiStore>(ma, mb, g, 1, st);
+        rc = N == 64 ? launch_gemm<64>(ma, mb, g, st) : launch_gemm<256>(ma, mb, g, st);
     }
     if (!rc) {
         uint32_t e = 0;
@@ -1540,20 +1981,22 @@ int lpsim_mlp_time(lpsim_mlp *m, uint32_t iters, double *fwd_ms, double *train_m
     CU(cudaEventCreate(&e0));
     CU(cudaEventCreate(&e1));
     // whatever the batch buffers hold is a valid input; warm up once
-    TRY(forward_batch(m, false));
+    TRY(forward_fused(m));
     CU(cudaEventRecord(e0, m->stream));
-    for (uint32_t i = 0; i < iters; i++) TRY(forward_batch(m, false));
+    for (uint32_t i = 0; i < iters; i++) TRY(forward_fused(m));
     CU(cudaEventRecord(e1, m->stream));
     CU(cudaEventSynchronize(e1));
     float ms = 0.0f;
     CU(cudaEventElapsedTime(&ms, e0, e1));
     if (fwd_ms) *fwd_ms = ms / iters;
     if (train_ms) {
-        CU(cudaMemsetAsync(m->loss_acc, 0, 4, m->stream));
         CU(cudaEventRecord(e0, m->stream));
         for (uint32_t i = 0; i < iters; i++) {
-            TRY(forward_batch(m, true));
-            TRY(backward_batch(m, m->B));
+            UpdateArgs u{};
+            TRY(train_core(m, m->Xf, m->t, (uint32_t)m->B, 0, 0, 0, 0, u));
+            u.G = m->Gf;
+            u.loss = m->Gf + kLossAt;
+            TRY(train_update(m, u));
         }
         CU(cudaEventRecord(e1, m->stream));
         CU(cudaEventSynchronize(e1));

@@ -168,6 +168,39 @@ def test_gradients_match_oracle():
     assert np.all(g["W1"].reshape(256, 64)[:, 9:] == 0)
 
 
+@pytest.mark.parametrize("batch,n,nf", [(128, 1, 11), (128, 128, 1), (256, 129, 16), (256, 127, 17), (9856, 9729, 11),
+                                        (20480, 20353, 64)])
+def test_gradients_at_tile_edges(batch, n, nf):
+    """One row, whole and ragged 128-row tiles, every padding of the inputs'
+    16-wide steps, and more tiles than there are CTA pairs (76 on 152 SMs), so
+    that a pair walks over several.  Tolerances as above: BF16 rounding of the
+    activations and of dZ, 2^-9 of each term."""
+    from paper_2406_08496_gb300 import Surrogate
+    p = _params(31)
+    p["W1"] = np.random.default_rng(32).standard_normal((256, 64)) * np.sqrt(2.0 / nf)
+    p["W1"][:, nf:] = 0.0
+    s = Surrogate(n_features=nf, batch=batch, seed=0)
+    s.set_params(p)
+    X, Xp = _inputs(n, 33, nf)
+    t = np.random.default_rng(34).standard_normal(n).astype(np.float32)
+    loss, g = s.grad(X, t)
+    q = _bf16_params(p)
+    ref_loss = float(np.mean((M.forward(q, Xp, act_round=M.bf16_round) - t) ** 2))
+    assert abs(loss - ref_loss) <= 1e-2 * ref_loss
+    gr = M.backward(q, Xp, t.astype(np.float64), act_round=M.bf16_round)
+    for k in gr:
+        a, b = g[k].astype(np.float64).reshape(gr[k].shape), gr[k]
+        if k == "W1":
+            assert np.all(a[:, nf:] == 0)
+            a, b = a[:, :nf], b[:, :nf]
+        assert np.linalg.norm(a - b) < 3e-2 * np.linalg.norm(b) + 1e-12, k
+        tol = 2 ** -7 * np.sqrt(256) * (np.abs(b) + np.sqrt(np.mean(b * b)))
+        assert np.all(np.abs(a - b) <= tol), (k, float(np.max(np.abs(a - b) / tol)))
+    loss2, g2 = s.grad(X, t)  # no sum depends on the order of arrival
+    assert loss2 == loss and all(np.array_equal(g[k], g2[k]) for k in g)
+    s.close()
+
+
 F32 = np.float32
 ADAM_B1, ADAM_B2, ADAM_EPS = float(F32(0.9)), float(F32(0.999)), float(F32(1e-8))
 
