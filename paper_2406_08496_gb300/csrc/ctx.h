@@ -13,6 +13,10 @@
 // record `msg` as the calling thread's lpsim_last_error() and return `code`
 int lpsim_fail(int code, const std::string &msg);
 
+// the run counters' array: [0..7] counters, then, on another cache line, the
+// error word and the slot count, so that one copy brings a status to the host
+constexpr int kCtrErr = 16, kCtrSlots = 17, kCtrWords = 18;
+
 struct lpsim_ctx {
     int device = 0;
     int n_sm = 0;
@@ -43,7 +47,7 @@ struct lpsim_ctx {
     int grid = 0, block = 256;
     bool sort = true;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
-    unsigned long long *h_ctr = nullptr;  // pinned: ctr[0..7], err, n_slots, ...
+    unsigned long long *h_ctr = nullptr;  // pinned: kCtrWords words of ctr
     uint32_t *d_tmp = nullptr;
     lpsim::QRec *org_hd0 = nullptr;  // first trip of each origin queue (reset)
     uint64_t launches = 0;

@@ -288,6 +288,35 @@ def test_light_load_chunks_match_oracle(grid_day, flags):
     assert co["lane_changes"] == cg["lane_changes"]
 
 
+@pytest.mark.parametrize("flags,light_trips", [(0, 0), (4, 0), (0, 400)])
+def test_uneven_pieces_match_oracle(grid_day, flags, light_trips):
+    """Step counts that are no whole chunks: pieces too short for the
+    light-load kernel, pieces inside a sort period, over one and over
+    several, up to a chunk's end and past it, in the light-load kernel
+    (flags 0), in the grid-wide kernels (flags 4) and in both by turns (at
+    most 400 trips for the light-load kernel); every output matches the
+    oracle after every piece."""
+    import oracle as O
+    import workloads as Wk
+    from paper_2406_08496_gb300 import Simulation
+    net, dem = grid_day
+    keep = np.zeros(len(dem["depart_step"]), bool)
+    keep[::3] = True
+    sub = Wk.subset_trips(dem, keep)
+    params = dict(bin_steps=300, n_bins=16, eps_amp=1.0, dlc_prob=0.3, dlc_gain=3.0)
+    o = O.Oracle(net, params)
+    o.load_demand(sub)
+    g = Simulation(net, dict(params, flags=flags | 2, light_trips=light_trips))
+    g.load_demand(sub)
+    for n in (1, 2, 3, 37, 212, 1, 256, 255, 700, 68, 1, 1537, 1536, 5, 530, 4):
+        o.step(n)
+        g.step(n)
+        assert_outputs_equal(o, g, n_bins=16, where=f"step {o.counters()['k']}")
+    co, cg = o.counters(), g.counters()
+    for key in ("k", "veh_steps", "arrived", "active", "waiting", "lane_changes"):
+        assert co[key] == cg[key], (key, co[key], cg[key])
+
+
 def test_light_and_grid_wide_chunks_alternate():
     """8,000 trips on a 12x12 grid: the chunks switch between the grid-wide
     kernels and the light-load block as the network fills and drains; every
