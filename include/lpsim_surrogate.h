@@ -30,16 +30,18 @@ extern "C" {
 typedef struct lpsim_mlp lpsim_mlp;
 
 /* New model with He-initialised weights from `seed`; batch = rows per
- * training step and per forward chunk (multiple of 128); stream as in
+ * training step (multiple of 128); stream as in
  * lpsim_load_network (NULL: the model creates its own). */
 int lpsim_mlp_create(lpsim_mlp **out, uint32_t n_features, uint32_t batch, uint64_t seed, void *stream);
 int lpsim_mlp_set_params(lpsim_mlp *m, const float *const *tensors);
 int lpsim_mlp_get_params(lpsim_mlp *m, float *const *tensors);
 
 /* y[i] = MLP(X[i, :]) for n rows of n_features f32 values (BF16 inside).
- * With more than `batch` rows the outputs gather on the device (4 bytes per
- * row, in whole batches; allocated at the first such call and kept until
- * lpsim_mlp_destroy, LPSIM_E_OOM if it cannot be) and cross back once. */
+ * With more than `batch` rows the rows pass through the device in pieces (two
+ * of 512 rows per SM, one copied in while the other is computed) and the
+ * outputs gather there (4 bytes per row) and cross back once; both are
+ * allocated at the first such call and kept until lpsim_mlp_destroy
+ * (LPSIM_E_OOM if they cannot be). */
 int lpsim_mlp_forward(lpsim_mlp *m, uint64_t n, const float *X, float *y);
 
 /* Forward and backward of one batch (n <= batch rows): mean squared error

@@ -341,15 +341,17 @@ __global__ void __launch_bounds__(kThreads)
 // ------------------------------------------------ fused inference forward
 //
 // All three hidden layers and the head of the inference forward in one
-// persistent kernel.  Per 128-row tile the input slice arrives by TMA; each
+// persistent kernel.  Per 128-row tile two warps read the f32 inputs, round
+// them and write the 128-byte-swizzled slice the first MMA reads (a packing
+// pass before the kernel moved another 128 B per row out and back in); each
 // layer's accumulator (128 x 256 f32) lives in tensor memory; the epilogue
 // writes the layer's BF16 activations straight into shared memory in the
 // 128-byte-swizzled K-major layout that the next layer's MMA reads, so the
 // hidden activations never leave the SM and the forward moves only the
-// inputs (128 B per row) and the outputs (4 B per row) through HBM.  Weights
-// stream from L2 through a ring of 256 x 64 slices.  Roles: warp 0 lane 0
-// loads, warp 1 lane 0 issues the MMAs, warps 2-17 run the epilogues (four per
-// tensor-memory lane quarter, each a quarter of the 256 columns).
+// inputs and the outputs (4 B per row) through HBM.  Weights stream from L2
+// through a ring of 256 x 64 slices.  Roles: warp 0 lane 0 loads them, warp 1
+// lane 0 issues the MMAs, warps 2-17 run the epilogues (four per tensor-memory
+// lane quarter, each a quarter of the 256 columns), warps 18-19 the inputs.
 //
 // Two tiles are in flight per CTA, each with its own accumulator (the two
 // fill the 512 tensor-memory columns) and its own activation buffer (the
@@ -358,7 +360,8 @@ __global__ void __launch_bounds__(kThreads)
 // one tile's layer run while the epilogue warps work on the other tile's.
 
 constexpr int kFwdEpiWarps = 16;
-constexpr int kFwdThreads = (2 + kFwdEpiWarps) * 32;
+constexpr int kFwdInWarps = 2;
+constexpr int kFwdThreads = (2 + kFwdEpiWarps + kFwdInWarps) * 32;
 constexpr int kFwdBStages = 3;
 constexpr uint32_t kSliceA = kBM * kBK * 2;  // one 64-wide K slice of a 128-row operand: 16 KB
 constexpr uint32_t kSliceB = 256 * kBK * 2;  // one 64-wide K slice of a weight matrix: 32 KB
@@ -368,7 +371,8 @@ constexpr size_t kFwdSmem = 1024 + 2 * kFwdBuf + kFwdBStages * kSliceB + 128;
 static_assert(kFwdSmem <= 232448, "fused forward exceeds the shared memory of a CTA");
 
 struct FwdArgs {
-    int n_tiles;
+    int n_tiles, n_rows, nf;
+    const float *X;  // n_rows x nf
     int l1_k16;  // 16-wide K steps of layer 1 that hold real inputs (the rest of the 64 columns is zero padding)
     const float *b1, *b2, *b3, *w4, *b4;
     float *y;
@@ -376,8 +380,8 @@ struct FwdArgs {
 };
 
 __global__ void __launch_bounds__(kFwdThreads, 1)
-    mlp_forward_fused(const __grid_constant__ CUtensorMap tX, const __grid_constant__ CUtensorMap tW1,
-                      const __grid_constant__ CUtensorMap tW2, const __grid_constant__ CUtensorMap tW3, FwdArgs g) {
+    mlp_forward_fused(const __grid_constant__ CUtensorMap tW1, const __grid_constant__ CUtensorMap tW2,
+                      const __grid_constant__ CUtensorMap tW3, FwdArgs g) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *sA = smem;                  // two tiles' activation buffers (kFwdBuf each)
@@ -402,7 +406,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
             mbar_init(&b_empty[s], 1);
         }
         for (int p = 0; p < 2; p++) {
-            mbar_init(&x_full[p], 1);
+            mbar_init(&x_full[p], kFwdInWarps);
             mbar_init(&a_free[p], 1);
             mbar_init(&acc_full[p], 1);
             mbar_init(&ep_done[p], kFwdEpiWarps);
@@ -428,16 +432,6 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                     for (int p = 0; p < 2; p++) {
                         const int j = 2 * P + p;
                         if (j >= nt || s_fail) continue;
-                        if (l == 0) {
-                            // the buffer's previous tile has finished its last layer
-                            if (P > 0 && !mbar_wait(&a_free[p], (P - 1) & 1)) {
-                                atomicOr(g.err, 8u);
-                                s_fail = 1;
-                                continue;
-                            }
-                            mbar_expect_tx(&x_full[p], kSliceA);
-                            tma_load_2d(sA + p * kFwdBuf, &tX, &x_full[p], 0, ((int)blockIdx.x + j * (int)gridDim.x) * kBM);
-                        }
                         const CUtensorMap *tw = l == 0 ? &tW1 : l == 1 ? &tW2 : &tW3;
                         const int nks = l == 0 ? 1 : 4;
                         for (int ks = 0; ks < nks; ks++, bi++) {
@@ -501,6 +495,44 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                     }
                 }
             }
+        }
+    } else if (warp >= 2 + kFwdEpiWarps) {
+        // inputs: two rows per thread, eight columns (one 16-byte chunk) at a time; the first 16 columns are on
+        // their way while the buffer's previous tile finishes
+        const int t0 = (int)threadIdx.x - (2 + kFwdEpiWarps) * 32;
+        const int nch = 2 * g.l1_k16;
+        for (int j = 0; j < nt; j++) {
+            const int p = j & 1;
+            const int r0 = ((int)blockIdx.x + j * (int)gridDim.x) * kBM;
+            auto chunk = [&](int row, int ch) {
+                const float *xp = g.X + (size_t)(r0 + row) * g.nf + ch * 8;
+                float v[8];
+#pragma unroll
+                for (int i = 0; i < 8; i++) v[i] = r0 + row < g.n_rows && ch * 8 + i < g.nf ? xp[i] : 0.0f;
+                return make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]),
+                                  pack_bf16x2(v[6], v[7]));
+            };
+            uint8_t *xs = sA + p * kFwdBuf;
+            auto put = [&](int row, int ch, uint4 v) {
+                *reinterpret_cast<uint4 *>(xs + (row >> 3) * 1024 + (row & 7) * 128 + ((ch ^ (row & 7)) << 4)) = v;
+            };
+            uint4 first[2][2];
+#pragma unroll
+            for (int i = 0; i < 4; i++) first[i >> 1][i & 1] = chunk(t0 + 64 * (i >> 1), i & 1);
+            // the buffer's previous tile has finished its last layer
+            if (j >= 2 && !s_fail && !mbar_wait(&a_free[p], ((j >> 1) - 1) & 1)) {
+                atomicOr(g.err, 8u);
+                s_fail = 1;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; i++) put(t0 + 64 * (i >> 1), i & 1, first[i >> 1][i & 1]);
+            for (int ch = 2; ch < nch; ch++) {
+                put(t0, ch, chunk(t0, ch));
+                put(t0 + 64, ch, chunk(t0 + 64, ch));
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&x_full[p]);
         }
     } else {
         // epilogue warps: rows q*32 + lane of the tile, columns [64 cq, 64 cq + 64)
@@ -578,7 +610,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                         f2_unpack(head2, he, ho);
                         s_head[cq * kBM + row] = he + ho;
                         asm volatile("bar.sync 1, %0;" ::"r"(kFwdEpiWarps * 32) : "memory");
-                        if (cq == 0 && !s_fail)
+                        if (cq == 0 && !s_fail && ((int)blockIdx.x + j * (int)gridDim.x) * kBM + row < g.n_rows)
                             g.y[((int)blockIdx.x + j * (int)gridDim.x) * kBM + row] =
                                 (((s_head[row] + s_head[kBM + row]) + s_head[2 * kBM + row]) + s_head[3 * kBM + row]) +
                                 *g.b4;
@@ -601,16 +633,6 @@ __global__ void gelu_eval(const float *z, uint64_t n, float *gelu, float *dgelu)
         const float cdf = norm_cdf(z[i]);
         gelu[i] = z[i] * cdf;
         dgelu[i] = cdf + z[i] * norm_pdf(z[i]);
-    }
-}
-
-// X (n x nf f32, host layout) -> Xb (n_pad x 64 bf16, zero padded); block
-// (32, 8) handles a 32-row x 32-column tile
-__global__ void pack_inputs(const float *X, int n, int nf, __nv_bfloat16 *Xb) {
-    const int r0 = blockIdx.x * 32, c = blockIdx.y * 32 + threadIdx.x;
-    for (int rr = threadIdx.y; rr < 32; rr += 8) {
-        const int r = r0 + rr;
-        Xb[(size_t)r * 64 + c] = __float2bfloat16_rn((r < n && c < nf) ? X[(size_t)r * nf + c] : 0.0f);
     }
 }
 
@@ -1483,7 +1505,7 @@ struct lpsim_mlp {
     __nv_bfloat16 *X0, *H[2], *dZ[3];
     float *small, *part;  // partial sums of mlp_train_fused (per cluster) and mlp_wgrad (per split)
     uint32_t *err;
-    CUtensorMap mX0, mW[3];
+    CUtensorMap mW[3];
     TrainMaps tmaps;
     WgradMaps gmaps;
     std::vector<float> h_flat;  // gradients or parameters on their way to the caller's tensors
@@ -1495,9 +1517,13 @@ struct lpsim_mlp {
     uint64_t pool_n = 0, pool_cap = 0;
     float *loss_hist = nullptr;
     uint32_t loss_cap = 0;
-    // outputs of a many-batch inference call, gathered on the device
+    // an inference call of more than a batch: outputs gathered on the device,
+    // two pieces of inputs and the stream that copies them in
     float *y_all = nullptr;
     uint64_t y_all_cap = 0;
+    float *in[2] = {};
+    cudaStream_t in_stream = nullptr;
+    cudaEvent_t in_here[2] = {}, in_used[2] = {};
 
     void *alloc(size_t bytes) {
         void *p = nullptr;
@@ -1512,6 +1538,12 @@ struct lpsim_mlp {
         cudaFree(pool_t);
         cudaFree(loss_hist);
         cudaFree(y_all);
+        if (in_stream) cudaStreamDestroy(in_stream);
+        for (int b = 0; b < 2; b++) {
+            cudaFree(in[b]);
+            if (in_here[b]) cudaEventDestroy(in_here[b]);
+            if (in_used[b]) cudaEventDestroy(in_used[b]);
+        }
         if (own_stream) cudaStreamDestroy(stream);
     }
 };
@@ -1617,35 +1649,52 @@ int train_update(lpsim_mlp *m, const UpdateArgs &u) {
     return launch_dependent(mlp_update, dim3(kUpdBlocks + kUpdSmallBlocks), 256, 0, m->stream, u);
 }
 
-// inference forward of the rows packed in X0: every layer in one kernel, activations kept on chip
-int forward_fused(lpsim_mlp *m, float *y_out = nullptr) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        CU(cudaFuncSetAttribute(mlp_forward_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem));
-        attr_set = true;
-    }
+// inference forward of n rows of m->nf inputs (device) into y
+int forward_fused(lpsim_mlp *m, const float *X, uint64_t n, float *y) {
+    CU(cudaFuncSetAttribute(mlp_forward_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem));
     FwdArgs g{};
-    g.n_tiles = m->B / kBM;
+    g.n_rows = (int)n;
+    g.n_tiles = (int)((n + kBM - 1) / kBM);
+    g.nf = m->nf;
+    g.X = X;
     g.l1_k16 = (m->nf + 15) / 16;
     g.b1 = m->P[1];
     g.b2 = m->P[3];
     g.b3 = m->P[5];
     g.w4 = m->P[6];
     g.b4 = m->P[7];
-    g.y = y_out ? y_out : m->y;
+    g.y = y;
     g.err = m->err;
     const int grid = std::min(g.n_tiles, m->n_sm);
-    mlp_forward_fused<<<grid, kFwdThreads, kFwdSmem, m->stream>>>(m->mX0, m->mW[0], m->mW[1], m->mW[2], g);
+    mlp_forward_fused<<<grid, kFwdThreads, kFwdSmem, m->stream>>>(m->mW[0], m->mW[1], m->mW[2], g);
     m->launches++;
     CU(cudaGetLastError());
     return LPSIM_OK;
 }
 
-int pack_batch(lpsim_mlp *m, const float *X_host, uint64_t n) {
-    CU(cudaMemcpyAsync(m->Xf, X_host, n * m->nf * 4, cudaMemcpyHostToDevice, m->stream));
-    pack_inputs<<<dim3(m->B / 32, 2), dim3(32, 8), 0, m->stream>>>(m->Xf, (int)n, m->nf, m->X0);
-    m->launches++;
-    CU(cudaGetLastError());
+// Rows per launch of a long inference call: four tiles per SM, whole waves, for
+// which the kernel takes 35.5 us and the copy in 22 us.  (One launch per batch
+// of 8192 rows kept 64 of the 152 SMs busy for 14.9 us each and the host with
+// 735 calls: 2,000,003 rows 9.9 ms, now 1.08 ms, 0.92 ms of it the kernel.)
+// Every tile's result is its own, so the split does not show in the outputs.
+uint64_t forward_piece(const lpsim_mlp *m) { return 4ull * m->n_sm * kBM; }
+
+// A long inference call: pieces of the rows, two on the device at once, so that
+// one is copied in (on a stream of the model's own) while the other is computed.
+// The copy stream is waited for before the caller's rows may go away.
+int forward_pieces(lpsim_mlp *m, uint64_t n, const float *X, float *y) {
+    const uint64_t piece = forward_piece(m);
+    for (uint64_t r0 = 0, i = 0; r0 < n; r0 += piece, i++) {
+        const uint64_t nb = std::min(piece, n - r0);
+        const int b = (int)(i & 1);
+        if (i >= 2) CU(cudaStreamWaitEvent(m->in_stream, m->in_used[b], 0));
+        CU(cudaMemcpyAsync(m->in[b], X + r0 * m->nf, nb * m->nf * 4, cudaMemcpyHostToDevice, m->in_stream));
+        CU(cudaEventRecord(m->in_here[b], m->in_stream));
+        CU(cudaStreamWaitEvent(m->stream, m->in_here[b], 0));
+        TRY(forward_fused(m, m->in[b], nb, m->y_all + r0));
+        CU(cudaEventRecord(m->in_used[b], m->stream));
+    }
+    CU(cudaMemcpyAsync(y, m->y_all, n * 4, cudaMemcpyDeviceToHost, m->stream));
     return LPSIM_OK;
 }
 
@@ -1722,8 +1771,7 @@ int lpsim_mlp_create(lpsim_mlp **out, uint32_t n_features, uint32_t batch, uint6
     TrainMaps &tm = m->tmaps;
     WgradMaps &gm = m->gmaps;
     const __nv_bfloat16 *wsrc[5] = {m->Wb[0], m->Wb[1], m->Wb[2], m->WbT[2], m->WbT[1]};
-    if ((rc = make_map(&m->mX0, m->X0, B, 64, kBM)) || (rc = make_map(&gm.x0, m->X0, B, 64, 64))) return bail(rc);
-    tm.x0 = m->mX0;
+    if ((rc = make_map(&tm.x0, m->X0, B, 64, kBM)) || (rc = make_map(&gm.x0, m->X0, B, 64, 64))) return bail(rc);
     for (int s = 0; s < 5; s++)
         if ((rc = make_map(&tm.w[s], wsrc[s], 256, s == 0 ? 64 : 256, 128))) return bail(rc);
     for (int l = 0; l < 3; l++) {
@@ -1776,37 +1824,42 @@ int lpsim_mlp_get_params(lpsim_mlp *m, float *const *tensors) {
 
 int lpsim_mlp_forward(lpsim_mlp *m, uint64_t n, const float *X, float *y) {
     if (!m || !X || !y) return fail(LPSIM_E_INVALID_ARG, "NULL argument");
-    const uint64_t B = (uint64_t)m->B;
-    if (n > B) {
-        // many batches: each batch's outputs land in one device array (every
-        // tile of a batch writes its 128 rows, so it is sized in whole
-        // batches) that crosses back once, not one small copy per batch
-        const uint64_t rows = (n + B - 1) / B * B;
-        if (rows > m->y_all_cap) {
-            CU(cudaStreamSynchronize(m->stream));
-            cudaFree(m->y_all);
+    if (n <= (uint64_t)m->B) {
+        if (n == 0) return mlp_check_err(m);
+        CU(cudaMemcpyAsync(m->Xf, X, n * m->nf * 4, cudaMemcpyHostToDevice, m->stream));
+        TRY(forward_fused(m, m->Xf, n, m->y));
+        CU(cudaMemcpyAsync(y, m->y, n * 4, cudaMemcpyDeviceToHost, m->stream));
+        return mlp_check_err(m);
+    }
+    if (n > m->y_all_cap) {
+        CU(cudaStreamSynchronize(m->stream));
+        cudaFree(m->y_all);
+        m->y_all = nullptr;
+        m->y_all_cap = 0;
+        if (cudaMalloc(&m->y_all, n * 4) != cudaSuccess) {
             m->y_all = nullptr;
-            m->y_all_cap = 0;
-            if (cudaMalloc(&m->y_all, rows * 4) != cudaSuccess) {
-                m->y_all = nullptr;
-                return fail(LPSIM_E_OOM, "device allocation of the outputs failed");
+            return fail(LPSIM_E_OOM, "device allocation of the outputs failed");
+        }
+        m->y_all_cap = n;
+    }
+    if (!m->in_stream) {
+        const size_t bytes = forward_piece(m) * m->nf * 4;
+        for (int b = 0; b < 2; b++) {
+            if (!m->in[b] && cudaMalloc(&m->in[b], bytes) != cudaSuccess) {
+                m->in[b] = nullptr;
+                return fail(LPSIM_E_OOM, "device allocation of the input pieces failed");
             }
-            m->y_all_cap = rows;
+            if (!m->in_here[b]) CU(cudaEventCreateWithFlags(&m->in_here[b], cudaEventDisableTiming));
+            if (!m->in_used[b]) CU(cudaEventCreateWithFlags(&m->in_used[b], cudaEventDisableTiming));
         }
+        CU(cudaStreamCreateWithFlags(&m->in_stream, cudaStreamNonBlocking));
     }
-    for (uint64_t r0 = 0; r0 < n; r0 += B) {
-        const uint64_t nb = std::min<uint64_t>(B, n - r0);
-        TRY(pack_batch(m, X + r0 * m->nf, nb));
-        if (n > B) {
-            TRY(forward_fused(m, m->y_all + r0));
-        } else {
-            TRY(forward_fused(m));
-            CU(cudaMemcpyAsync(y + r0, m->y, nb * 4, cudaMemcpyDeviceToHost, m->stream));
-        }
-    }
-    if (n > B) CU(cudaMemcpyAsync(y, m->y_all, n * 4, cudaMemcpyDeviceToHost, m->stream));
-    CU(cudaStreamSynchronize(m->stream));
-    return mlp_check_err(m);
+    const int rc = forward_pieces(m, n, X, y);
+    const cudaError_t e = cudaStreamSynchronize(m->in_stream);
+    const int rc2 = mlp_check_err(m);
+    if (rc) return rc;
+    if (e != cudaSuccess) return fail(LPSIM_E_CUDA, std::string("input copies: ") + cudaGetErrorString(e));
+    return rc2;
 }
 
 int lpsim_mlp_grad(lpsim_mlp *m, uint64_t n, const float *X, const float *t, float *loss, float *const *grads) {
@@ -1981,9 +2034,9 @@ int lpsim_mlp_time(lpsim_mlp *m, uint32_t iters, double *fwd_ms, double *train_m
     CU(cudaEventCreate(&e0));
     CU(cudaEventCreate(&e1));
     // whatever the batch buffers hold is a valid input; warm up once
-    TRY(forward_fused(m));
+    TRY(forward_fused(m, m->Xf, (uint64_t)m->B, m->y));
     CU(cudaEventRecord(e0, m->stream));
-    for (uint32_t i = 0; i < iters; i++) TRY(forward_fused(m));
+    for (uint32_t i = 0; i < iters; i++) TRY(forward_fused(m, m->Xf, (uint64_t)m->B, m->y));
     CU(cudaEventRecord(e1, m->stream));
     CU(cudaEventSynchronize(e1));
     float ms = 0.0f;

@@ -143,6 +143,30 @@ def test_forward_production_size_matches_oracle():
     assert np.array_equal(ys.view(np.uint32), y[pick].view(np.uint32))
 
 
+@pytest.mark.parametrize("n,nf", [(129, 11), (77823, 9), (77824, 1), (77825, 17), (2 * 77824 + 1, 8), (300000, 64)])
+def test_forward_in_pieces_equals_one_batch(n, nf):
+    """A call of more than a batch passes through the device in pieces of 512
+    rows per SM (77,824 on 152 SMs): row counts around the pieces' ends and
+    every padding of the inputs' 16-wide steps, bit for bit equal to the same
+    rows in one batch, and the first rows within the derived bound."""
+    from paper_2406_08496_gb300 import Surrogate
+    p = _params(41)
+    p["W1"] = np.random.default_rng(42).standard_normal((256, 64)) * np.sqrt(2.0 / nf)
+    p["W1"][:, nf:] = 0.0
+    X, Xp = _inputs(n, 43, nf=nf)
+    s = Surrogate(n_features=nf, batch=128, seed=0)
+    s.set_params(p)
+    y = s.forward(X)
+    assert np.array_equal(s.forward(X).view(np.uint32), y.view(np.uint32))
+    s.close()
+    one = Surrogate(n_features=nf, batch=(n + 127) // 128 * 128, seed=0)
+    one.set_params(p)
+    assert np.array_equal(one.forward(X).view(np.uint32), y.view(np.uint32))
+    one.close()
+    ref, bound = forward_bound(_bf16_params(p), Xp[:1000])
+    assert np.all(np.abs(y[:1000] - ref) <= bound)
+
+
 def test_gradients_match_oracle():
     from paper_2406_08496_gb300 import Surrogate
     p = _params(5)
