@@ -65,50 +65,92 @@ __device__ __forceinline__ uint8_t speed_byte(float v) {
     return (uint8_t)(uint32_t)t;
 }
 
-// 16-bit mask of the occupied bytes of a 16-byte chunk.
-__device__ __forceinline__ uint32_t occ_mask16(uint4 q) {
-    uint32_t w[4] = {q.x, q.y, q.z, q.w};
-    uint32_t m = 0;
+// Searches of a 16-byte aligned lane row for the nearest occupied cell.  Cells
+// are bytes, 0xFF when empty, so a word's complement has a nonzero byte per
+// occupied cell: the search picks the first (or last) nonzero word of the
+// window, the cells before the window's start masked off its first chunk, and
+// the byte within it; a find past the window's end is none.  (A 16-bit mask
+// built per chunk from byte compares took four times the instructions.)
+
+// the complements of chunks c_first, c_first + step, ... (N of them, loaded
+// together: one memory round trip), zero where `in` says the window has ended
+template <int N, class In>
+__device__ __forceinline__ void load_cells(const uint8_t *row, uint32_t c_first, int step, In in,
+                                           uint32_t (&w)[4 * N]) {
+    uint4 q[N];
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-        uint32_t b = __vcmpne4(w[j], 0xFFFFFFFFu);  // 0xFF per occupied byte
-        uint32_t bits = ((b >> 7) & 1u) | ((b >> 14) & 2u) | ((b >> 21) & 4u) | ((b >> 28) & 8u);
-        m |= bits << (4 * j);
+    for (int j = 0; j < N; j++) {
+        const uint32_t c = c_first + (uint32_t)(step * j);
+        q[j] = in(c, j) ? *reinterpret_cast<const uint4 *>(row + c) : make_uint4(~0u, ~0u, ~0u, ~0u);
     }
-    return m;
+#pragma unroll
+    for (int j = 0; j < N; j++) {
+        w[4 * j] = ~q[j].x;
+        w[4 * j + 1] = ~q[j].y;
+        w[4 * j + 2] = ~q[j].z;
+        w[4 * j + 3] = ~q[j].w;
+    }
 }
 
-__device__ __forceinline__ uint32_t range_mask16(uint32_t c, uint32_t lo, uint32_t hi) {
-    // bits of chunk [c, c+16) that fall in [lo, hi]
-    uint32_t a = lo > c ? lo - c : 0u;
-    uint32_t b = hi < c + 15u ? hi - c : 15u;
-    return ((0xFFFFu << a) & (0xFFFFu >> (15u - b))) & 0xFFFFu;
+// chunks of [lo, hi] from lo's on, the cells before lo dropped
+template <int N>
+__device__ __forceinline__ void load_ahead(const uint8_t *row, uint32_t lo, uint32_t hi, uint32_t (&w)[4 * N]) {
+    load_cells<N>(row, lo & ~15u, 16, [hi](uint32_t c, int) { return c <= hi; }, w);
+#pragma unroll
+    for (int j = 0; j < 4; j++) w[j] &= __funnelshift_lc(0u, ~0u, max((int)(8u * (lo & 15u)) - 32 * j, 0));
 }
 
-// first occupied cell in [lo, hi] of a 16-byte aligned row, or kNone; the
-// first four 16-byte chunks of the window are loaded together, so a window of
-// up to 49 cells costs one memory round trip
+// first occupied cell at or after lo in the loaded chunks, or kNone
+template <int N>
+__device__ __forceinline__ uint32_t find_first(const uint32_t (&w)[4 * N], uint32_t lo) {
+    uint32_t t = 0, at = 0;
+#pragma unroll
+    for (int j = 4 * N - 1; j >= 0; j--)
+        if (w[j]) {
+            t = w[j];
+            at = 4u * j;
+        }
+    return t ? (lo & ~15u) + at + ((uint32_t)(__ffs((int)t) - 1) >> 3) : kNone;
+}
+
+// chunks of [lo, hi] from hi's down, the cells after hi dropped
+template <int N>
+__device__ __forceinline__ void load_behind(const uint8_t *row, uint32_t lo, uint32_t hi, uint32_t (&w)[4 * N]) {
+    const uint32_t n = (hi >> 4) - (lo >> 4);  // chunks of the window after the first
+    load_cells<N>(row, hi & ~15u, -16, [n](uint32_t, int j) { return (uint32_t)j <= n; }, w);
+#pragma unroll
+    for (int j = 0; j < 4; j++) w[j] &= __funnelshift_rc(~0u, 0u, max(32 * (j + 1) - 8 * (int)((hi & 15u) + 1u), 0));
+}
+
+// last occupied cell at or before hi in the loaded chunks, or kNone
+template <int N>
+__device__ __forceinline__ uint32_t find_last(const uint32_t (&w)[4 * N], uint32_t hi) {
+    uint32_t t = 0, at = 0;
+#pragma unroll
+    for (int j = N - 1; j >= 0; j--)
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+            if (w[4 * j + i]) {
+                t = w[4 * j + i];
+                at = 16u * j - 4u * i;
+            }
+    return t ? (hi & ~15u) - at + ((uint32_t)(31 - __clz((int)t)) >> 3) : kNone;
+}
+
+// first occupied cell in [lo, hi], or kNone; the first four 16-byte chunks of
+// the window are loaded together, so a window of up to 49 cells costs one
+// memory round trip
 __device__ __forceinline__ uint32_t first_occupied_wide(const uint8_t *row, uint32_t lo, uint32_t hi) {
     if (lo > hi) return kNone;
-    const uint32_t c0 = lo & ~15u;
-    uint4 q[4];
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-        const uint32_t c = c0 + 16u * j;
-        q[j] = c <= hi ? *reinterpret_cast<const uint4 *>(row + c) : make_uint4(~0u, ~0u, ~0u, ~0u);
+    uint32_t w[16];
+    load_ahead<4>(row, lo, hi, w);
+    uint32_t f = find_first<4>(w, lo);
+    for (uint32_t c = (lo & ~15u) + 64u; f == kNone && c <= hi; c += 16u) {
+        uint32_t u[4];
+        load_ahead<1>(row, c, hi, u);
+        f = find_first<1>(u, c);
     }
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-        const uint32_t c = c0 + 16u * j;
-        if (c > hi) break;
-        const uint32_t mk = occ_mask16(q[j]) & range_mask16(c, lo, hi);
-        if (mk) return c + (uint32_t)(__ffs((int)mk) - 1);
-    }
-    for (uint32_t c = c0 + 64u; c <= hi; c += 16u) {
-        const uint32_t mk = occ_mask16(*reinterpret_cast<const uint4 *>(row + c)) & range_mask16(c, lo, hi);
-        if (mk) return c + (uint32_t)(__ffs((int)mk) - 1);
-    }
-    return kNone;
+    return f <= hi ? f : kNone;
 }
 
 // car-following parameters of one vehicle (its type's, or the run's)
@@ -746,20 +788,6 @@ __device__ __forceinline__ void p2_dep(const Dev &d, const StepView &w, const De
 
 // ----------------------------------------------------------------------- P3
 
-// occupancy masks of the 5 chunks covering [c0 - 64, c0 + 63] around an
-// aligned base (loaded together)
-template <int N>
-__device__ __forceinline__ void load_chunks(const uint8_t *row, uint32_t c_first, uint32_t c_last, uint32_t (&mk)[N]) {
-    uint4 q[N];
-#pragma unroll
-    for (int j = 0; j < N; j++) {
-        const uint32_t c = c_first + 16u * j;
-        q[j] = c <= c_last ? *reinterpret_cast<const uint4 *>(row + c) : make_uint4(~0u, ~0u, ~0u, ~0u);
-    }
-#pragma unroll
-    for (int j = 0; j < N; j++) mk[j] = occ_mask16(q[j]);
-}
-
 // Lane-change intender ir: gap acceptance against the step-k map and the
 // reservations of the next map; the accepted move their byte sideways.  With
 // `late` (the intent aims at cell len - 1 and runs alongside the crossing
@@ -784,27 +812,21 @@ __device__ __forceinline__ void lane_change(const Dev &d, const StepView &w, con
     // window [c0 - 64, c0 + 63] of the target lane, clipped to the row
     const uint32_t lo = c0 > 64u ? c0 - 64u : 0u;
     const uint32_t hi = c0 + 63u < len - 1 ? c0 + 63u : len - 1;
-    const uint32_t cfirst = lo & ~15u;
-    uint32_t mk[9];
-    load_chunks<9>(row2, cfirst, hi, mk);
+    // at most five chunks on either side of c0; without cells behind c0 the
+    // window behind is cell 0 with nothing in it that counts
+    uint32_t wa[20], wb[20];
+    load_ahead<5>(row2, c0, hi, wa);
+    load_behind<5>(row2, lo, c0 > 0 ? c0 - 1 : 0u, wb);
     const uint32_t tgt = base2 + cn;
     const uint8_t tgt_map = Mn[tgt], tgt_mark = Iw[tgt];
     const uint4 xr = late ? d.xreq[base2 >> 4] : make_uint4(kNone, 0u, 0u, 0u);
     uint64_t h = 0;
     if (m.eps_amp > 0.0f) h = splitmix64_mix(ir.hk ^ ((uint64_t)k * 0xD1B54A32D192ED03ull));
     // lead: first occupied cell in [c0, hi]; lag: last in [lo, c0 - 1]
-    uint32_t ca = kNone, cb = kNone;
-#pragma unroll
-    for (int j = 0; j < 9; j++) {
-        const uint32_t c = cfirst + 16u * j;
-        if (c > hi) break;
-        const uint32_t a = mk[j] & range_mask16(c, c0, hi);
-        if (ca == kNone && a) ca = c + (uint32_t)(__ffs((int)a) - 1);
-        if (c0 > 0 && c <= c0 - 1) {
-            const uint32_t b = mk[j] & range_mask16(c, lo, c0 - 1);
-            if (b) cb = c + (31u - (uint32_t)__clz((int)b));
-        }
-    }
+    uint32_t ca = find_first<5>(wa, c0);
+    if (ca > hi) ca = kNone;
+    uint32_t cb = c0 > 0 ? find_last<5>(wb, c0 - 1) : kNone;
+    if (cb != kNone && cb < lo) cb = kNone;
     float eps_a = 0.0f, eps_b = 0.0f;
     if (m.eps_amp > 0.0f) {
         eps_a = m.eps_amp * (2.0f * unit24(splitmix64_mix(h ^ 0x632BE59BD9B4E019ull)) - 1.0f);
