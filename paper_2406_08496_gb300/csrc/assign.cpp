@@ -120,6 +120,36 @@ void td_dijkstra(const TD &td, uint32_t s, uint64_t t0, std::vector<uint64_t> &a
     }
 }
 
+// the candidate path becomes the route of the trips listed (ascending): the
+// flat routes are written anew, on the host's threads
+int take_candidates(lpsim_assign *a, const std::vector<uint64_t> &trips) {
+    if (trips.empty()) return LPSIM_OK;
+    std::vector<uint64_t> off(a->n + 1);
+    uint64_t o = 0;
+    size_t q = 0;
+    for (uint64_t j = 0; j < a->n; j++) {
+        off[j] = o;
+        const bool moved = q < trips.size() && trips[q] == j;
+        o += moved ? a->clen[j] : a->route_len(j);
+        q += moved;
+    }
+    off[a->n] = o;
+    if (!a->redge_next.reserve(o)) return fail(LPSIM_E_OOM, "host allocation of the routes failed");
+    uint32_t *edges = a->redge_next.p.get();
+    parallel_pieces(a->n, [&](uint64_t j0, uint64_t j1, uint64_t) {
+        size_t p = (size_t)(std::lower_bound(trips.begin(), trips.end(), j0) - trips.begin());
+        for (uint64_t j = j0; j < j1; j++) {
+            const bool moved = p < trips.size() && trips[p] == j;
+            std::memcpy(edges + off[j], moved ? a->cand(j) : a->route(j), (off[j + 1] - off[j]) * 4);
+            p += moved;
+        }
+    });
+    a->roff = std::move(off);
+    std::swap(a->redge, a->redge_next);
+    a->routes_version++;
+    return LPSIM_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -157,8 +187,8 @@ int lpsim_assign_create(lpsim_assign **out, uint32_t n_nodes, uint32_t n_edges, 
     a->orig.assign(orig, orig + n_trips);
     a->dest.assign(dest, dest + n_trips);
     a->dep.assign(depart_step, depart_step + n_trips);
-    a->route.resize(n_trips);
-    a->cand.resize(n_trips);
+    a->coff.assign(n_trips, 0);
+    a->clen.assign(n_trips, 0);
     a->tsp.assign(n_trips, 0.0f);
     a->excess.assign(n_trips, 0.0f);
     for (uint64_t j = 0; j < n_trips; j++) {
@@ -166,7 +196,21 @@ int lpsim_assign_create(lpsim_assign **out, uint32_t n_nodes, uint32_t n_edges, 
             delete a;
             return fail(LPSIM_E_INVALID_ARG, "trip " + std::to_string(j) + ": empty route or bad node");
         }
-        a->route[j].assign(route_edges + route_off[j], route_edges + route_off[j + 1]);
+    }
+    if (n_trips) {
+        a->roff.resize(n_trips + 1);
+        for (uint64_t j = 0; j <= n_trips; j++) a->roff[j] = route_off[j] - route_off[0];
+        const uint64_t n_edge_ids = a->roff[n_trips];
+        if (!a->redge.reserve(n_edge_ids)) {
+            delete a;
+            return fail(LPSIM_E_OOM, "host allocation of the routes failed");
+        }
+        const uint32_t *from = route_edges + route_off[0];
+        parallel_pieces(n_edge_ids, [&](uint64_t q0, uint64_t q1, uint64_t) {
+            std::memcpy(a->redge.p.get() + q0, from + q0, (q1 - q0) * 4);
+        });
+    } else {
+        a->roff.assign(1, 0);
     }
     a->dt = dt;
     a->seed = seed;
@@ -185,7 +229,13 @@ int lpsim_assign_shortest_paths(lpsim_assign *a, const float *tt, uint32_t n_bin
     const uint64_t ng = gstart.size() - 1;
     std::atomic<uint64_t> next{0};
     std::atomic<int> bad{0};
-    auto worker = [&]() {
+    const uint32_t nt = std::max<uint32_t>(1, std::min<uint32_t>(n_threads ? n_threads : 1, 256));
+    // each thread's paths; of each trip the thread, the position among its paths and the length
+    std::vector<std::vector<uint32_t>> paths(nt);
+    std::vector<uint32_t> by(a->n), plen(a->n, 0);
+    std::vector<uint64_t> pos(a->n);
+    auto worker = [&](uint32_t me) {
+        std::vector<uint32_t> &out = paths[me];
         std::vector<uint64_t> arr(a->n_nodes);
         std::vector<uint32_t> pred(a->n_nodes);
         std::vector<uint8_t> done(a->n_nodes);
@@ -224,21 +274,31 @@ int lpsim_assign_shortest_paths(lpsim_assign *a, const float *tt, uint32_t n_bin
                     tmp.push_back(e);
                     v = a->src[e];
                 }
-                a->cand[j].assign(tmp.rbegin(), tmp.rend());
+                by[j] = me;
+                pos[j] = out.size();
+                plen[j] = (uint32_t)tmp.size();
+                out.insert(out.end(), tmp.rbegin(), tmp.rend());
                 // the tree's path, timed from the trip's own departure (the
                 // same start as its experienced time)
                 const uint64_t tj = to_ms((double)a->dep[j] * a->dt);
                 uint64_t tt_j = tj;
-                for (uint32_t e : a->cand[j]) tt_j = td.arrive(e, tt_j);
+                for (size_t q = tmp.size(); q-- > 0;) tt_j = td.arrive(tmp[q], tt_j);
                 a->tsp[j] = (float)((double)(tt_j - tj) / 1000.0);
             }
         }
     };
-    const uint32_t nt = std::max<uint32_t>(1, std::min<uint32_t>(n_threads ? n_threads : 1, 256));
     std::vector<std::thread> th;
-    for (uint32_t i = 0; i < nt; i++) th.emplace_back(worker);
+    for (uint32_t i = 0; i < nt; i++) th.emplace_back(worker, i);
     for (auto &t : th) t.join();
     if (bad) return fail(LPSIM_E_INVALID_ARG, "a destination is unreachable from its origin");
+    std::vector<uint64_t> first(nt + 1, 0);
+    for (uint32_t i = 0; i < nt; i++) first[i + 1] = first[i] + paths[i].size();
+    std::fill(a->clen.begin(), a->clen.end(), 0u);
+    if (!a->cedge.reserve(first[nt])) return fail(LPSIM_E_OOM, "host allocation of the paths failed");
+    for (uint32_t i = 0; i < nt; i++)
+        if (!paths[i].empty()) std::memcpy(a->cedge.p.get() + first[i], paths[i].data(), paths[i].size() * 4);
+    for (uint64_t j = 0; j < a->n; j++) a->coff[j] = first[by[j]] + pos[j];
+    a->clen = std::move(plen);
     if (t_sp) std::memcpy(t_sp, a->tsp.data(), a->n * 4);
     return LPSIM_OK;
 }
@@ -277,15 +337,13 @@ int lpsim_assign_reroute(lpsim_assign *a, double fraction, uint32_t iteration, u
     if (!a || !(fraction >= 0.0 && fraction <= 1.0)) return fail(LPSIM_E_INVALID_ARG, "bad argument");
     std::mt19937_64 gen(a->seed * 1000003ull + iteration);
     std::uniform_real_distribution<double> u(0.0, 1.0);
-    uint64_t changed = 0;
+    std::vector<uint64_t> moved;
     for (uint64_t j = 0; j < a->n; j++) {
-        if (u(gen) >= fraction || a->cand[j].empty()) continue;
-        if (a->cand[j] != a->route[j]) {
-            a->route[j] = a->cand[j];
-            changed++;
-        }
+        if (u(gen) >= fraction || a->clen[j] == 0) continue;
+        if (a->cand_differs(j)) moved.push_back(j);
     }
-    if (n_changed) *n_changed = changed;
+    if (const int rc = take_candidates(a, moved)) return rc;
+    if (n_changed) *n_changed = moved.size();
     return LPSIM_OK;
 }
 
@@ -296,7 +354,7 @@ int lpsim_assign_route_excess(lpsim_assign *a, const float *tt, uint32_t n_bins,
         for (uint64_t j = j0; j < j1; j++) {
             const uint64_t t0 = to_ms((double)a->dep[j] * a->dt);
             uint64_t t = t0;
-            for (uint32_t e : a->route[j]) t = td.arrive(e, t);
+            for (uint64_t q = a->roff[j]; q < a->roff[j + 1]; q++) t = td.arrive(a->redge.p[q], t);
             a->excess[j] = (float)((double)(t - t0) / 1000.0 - a->tsp[j]);
         }
     });
@@ -312,35 +370,32 @@ int lpsim_assign_reroute_worst(lpsim_assign *a, double fraction, double min_rel_
     // ties to the lower index)
     std::vector<uint64_t> pick;
     for (uint64_t j = 0; j < a->n; j++)
-        if (!a->cand[j].empty() && a->excess[j] > 0.0f && rel(j) > min_rel_excess && a->cand[j] != a->route[j])
+        if (a->clen[j] != 0 && a->excess[j] > 0.0f && rel(j) > min_rel_excess && a->cand_differs(j))
             pick.push_back(j);
     const uint64_t want = std::min<uint64_t>(pick.size(), (uint64_t)std::llround(fraction * (double)a->n));
     std::partial_sort(pick.begin(), pick.begin() + want, pick.end(), [&](uint64_t x, uint64_t y) {
         const double rx = rel(x), ry = rel(y);
         return rx != ry ? rx > ry : x < y;
     });
-    for (uint64_t i = 0; i < want; i++) a->route[pick[i]] = a->cand[pick[i]];
+    pick.resize(want);
+    std::sort(pick.begin(), pick.end());
+    if (const int rc = take_candidates(a, pick)) return rc;
     if (n_changed) *n_changed = want;
     return LPSIM_OK;
 }
 
 uint64_t lpsim_assign_route_length(const lpsim_assign *a) {
     if (!a) return 0;
-    uint64_t t = 0;
-    for (auto &r : a->route) t += r.size();
-    return t;
+    return a->roff[a->n];
 }
 
 int lpsim_assign_get_routes(const lpsim_assign *a, uint64_t *route_off, uint32_t *route_edges, uint64_t capacity) {
     if (!a || !route_off || !route_edges) return fail(LPSIM_E_INVALID_ARG, "NULL argument");
     if (capacity < lpsim_assign_route_length(a)) return fail(LPSIM_E_INVALID_ARG, "route buffer too small");
-    uint64_t o = 0;
-    for (uint64_t j = 0; j < a->n; j++) {
-        route_off[j] = o;
-        std::memcpy(route_edges + o, a->route[j].data(), a->route[j].size() * 4);
-        o += a->route[j].size();
-    }
-    route_off[a->n] = o;
+    std::memcpy(route_off, a->roff.data(), (a->n + 1) * sizeof(uint64_t));
+    parallel_pieces(a->roff[a->n], [&](uint64_t q0, uint64_t q1, uint64_t) {
+        std::memcpy(route_edges + q0, a->redge.p.get() + q0, (q1 - q0) * 4);
+    });
     return LPSIM_OK;
 }
 
@@ -351,7 +406,8 @@ int lpsim_assign_load(const lpsim_assign *a, const float *tt, uint32_t n_bins, u
     parallel_pieces(a->n, [&](uint64_t j0, uint64_t j1, uint64_t) {
         for (uint64_t j = j0; j < j1; j++) {
             uint64_t t = to_ms((double)a->dep[j] * a->dt);
-            for (uint32_t e : a->route[j]) {
+            for (uint64_t q = a->roff[j]; q < a->roff[j + 1]; q++) {
+                const uint32_t e = a->redge.p[q];
                 const uint64_t b = t / td.bin_ms;
                 if (b < n_bins) __atomic_fetch_add(&inflow[(size_t)e * n_bins + b], 1u, __ATOMIC_RELAXED);
                 t = td.arrive(e, t);

@@ -9,7 +9,9 @@
 // of the period; at the regional scale that is some 10^5 trees per iteration
 // on a 224k-node graph, far more than the host's threads finish in seconds.
 //
-// Here every tree is searched by one warp, thousands of warps at a time (a
+// Networks of up to some 55 thousand nodes are searched with a tree's labels in
+// a block's shared memory (td_trees_shared, below).  Beyond that every tree is
+// searched by one warp (td_trees), thousands of warps at a time (a
 // tree's frontier is a wave of a few hundred nodes; many trees in flight
 // hide the memory latency each relaxation pays: on the 2.82M-trip day, 16
 // trees per SM took 2.7 s per pass, 32 took 1.85 s, 64 took 1.78 s; the
@@ -108,8 +110,16 @@ struct TreeArgs {
     uint32_t n_nodes, n_edges, n_bins, bin_ms;
     const uint32_t *out_off;  // n_nodes + 1
     const uint2 *adj;         // per out-edge position: {edge, head node}
+    const uint32_t *pos;      // per edge: its out-edge position (nullptr: the edge id is the position)
     const uint32_t *src;      // per edge: tail node
-    const uint2 *cms;         // n_bins x n_edges: {link time ms, earliest arrival entering a later bin ms}
+    const uint32_t *in_off;   // n_nodes + 1
+    const uint2 *in_adj;      // per in-edge, ascending edge ids: {out-edge position, tail node}
+    // n_bins x n_edges by out-edge position: {link time ms, earliest arrival entering a later bin ms}; a search
+    // reads a node's out-edges and their times side by side
+    const uint2 *cms;
+    // td_trees_shared, networks of at most kWide out-edges per node: positions are wide * node + k, so a node's
+    // row is known without out_off (0: positions as above); n_pos of them per bin
+    uint32_t wide, n_pos;
     uint32_t n_groups;
     const GroupRec *groups;
     const uint32_t *order;    // trip per position, group by group
@@ -122,7 +132,9 @@ struct TreeArgs {
     uint32_t *edges;          // path edges, travel order
     unsigned long long cap;   // entries of edges
     unsigned long long *cursor;
-    // per-warp workspaces
+    // td_trees_shared: positions along each thread's path, kScratch per thread
+    uint32_t *scratch;
+    // td_trees: per-warp workspaces
     NodeRec *node;            // n_warps x n_nodes: label, round stamp of the last push, far-pile mark
     uint32_t *touched;        // n_warps x n_nodes
     uint32_t *fa, *fb;        // n_warps x n_nodes: near sets (this round, next round)
@@ -143,6 +155,8 @@ __device__ __forceinline__ uint64_t arrive(const uint2 lt, uint64_t t) {
     const uint64_t a = t + lt.x;
     return a < (uint64_t)lt.y ? a : (uint64_t)lt.y;
 }
+
+__device__ __forceinline__ uint32_t pos_of(const TreeArgs &A, uint32_t e) { return A.pos ? A.pos[e] : e; }
 
 // Latest current arrival over the group's destinations (its trips'), or
 // kUnreached while any is unreached; every lane gets the result.
@@ -243,7 +257,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSm) td_trees(Tr
                         if (t >= total) continue;
                         const uint32_t j = o_j0 + (t - (o_incl - o_deg));
                         const uint2 ev = A.adj[j];
-                        const uint64_t at = arrive(A.cms[(size_t)bin_of(A, o_tu) * A.n_edges + ev.x], o_tu);
+                        const uint64_t at = arrive(A.cms[(size_t)bin_of(A, o_tu) * A.n_edges + j], o_tu);
                         if (at > 0xFFFFFFFFull || at > ub) continue;
                         const unsigned long long cand = (at << 32) | ev.x;
                         const unsigned long long old = atomicMin(&nd[ev.y].lab, cand);
@@ -353,7 +367,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSm) td_trees(Tr
             }
             const uint64_t tj = A.dep_ms[j];
             uint64_t t = tj;
-            for (uint32_t p = 0; p < L; p++) t = arrive(A.cms[(size_t)bin_of(A, t) * A.n_edges + A.edges[off + p]], t);
+            for (uint32_t p = 0; p < L; p++)
+                t = arrive(A.cms[(size_t)bin_of(A, t) * A.n_edges + pos_of(A, A.edges[off + p])], t);
             A.path_off[j] = off;
             A.path_len[j] = L;
             A.tsp[j] = (float)((double)(t - tj) / 1000.0);
@@ -368,6 +383,273 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSm) td_trees(Tr
     if (lane == 0) A.stamp[gw] = stamp;
 }
 
+// The same search with a tree's labels in shared memory: one block per tree,
+// for networks whose labels fit (n_nodes * 4 bytes and a bit per node in a
+// block's 227 KB: some 55 thousand nodes).  The label-correcting search is a
+// chain of label reads and atomics; in device memory each costs a round trip to
+// L2 or DRAM (thousands of trees' labels do not fit in L2), here a few cycles,
+// and a block's threads relax a whole near set at once, four lanes per node.
+//   * a label is the arrival alone, in ms after the root time, so a node takes
+//     four bytes; the tree's entering edge of a node is found again where a path
+//     is walked back: the lowest edge id among those that give its arrival, which
+//     is the edge the 64-bit label holds;
+//   * a bit per node says that it waits to be relaxed (cleared before its label is
+//     read, so a later improvement queues it again); the waiting nodes' ids are
+//     in a ring besides, and a round whose ids did not fit reads the bits;
+//   * a node's out-edges and their times are looked up by 4 (or 8) times the
+//     node where no node has more, so they come in one round trip to L2 instead
+//     of two;
+//   * no far pile: the nodes with a label in the next bucket are found by
+//     scanning the labels (a node at or above the threshold was never relaxed).
+// One block barrier per round: the counters rotate over three rounds.  Bound by
+// the round trips to L2 of one round after another (some 400 a tree).
+constexpr uint32_t kWide = 8;       // most out-edges per node for the wide rows
+constexpr uint64_t kSharedDeltaMs = 240000;
+constexpr uint32_t kRing = 1024;    // ids of waiting nodes (a power of two)
+constexpr uint32_t kScratch = 512;  // positions kept per thread while a path is walked back
+constexpr uint32_t kNever = 0xFFFFFFFFu;
+
+__host__ __device__ inline size_t shared_tree_bytes(uint32_t n_nodes) {
+    return (size_t)((n_nodes + 3) & ~3u) * 4 + (size_t)((n_nodes + 31) / 32) * 4 + kRing * 2;
+}
+
+template <int T, int PER_SM>
+__global__ void __launch_bounds__(T, PER_SM) td_trees_shared(TreeArgs A) {
+    extern __shared__ __align__(16) uint32_t s_lab[];
+    const uint32_t n4 = (A.n_nodes + 3) & ~3u, nw = (A.n_nodes + 31) / 32;
+    uint32_t *bits = s_lab + n4;
+    uint16_t *ring = reinterpret_cast<uint16_t *>(bits + nw);
+    __shared__ uint32_t s_group, s_cnt[3], s_min[3], s_red[32];
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    volatile uint32_t *vlab = s_lab;
+    uint32_t *scratch = A.scratch + (size_t)blockIdx.x * T * kScratch + tid;
+    const uint64_t max_rounds = 8ull * A.n_nodes + (1ull << 20);
+    for (;;) {
+        if (tid == 0) s_group = atomicAdd(A.next_group, 1u);
+        __syncthreads();  // also: the last tree's paths have been read
+        const uint32_t g = s_group;
+        if (g >= A.n_groups) break;
+        const GroupRec G = A.groups[g];
+        const uint64_t t0 = G.t0;
+        for (uint32_t i = tid; i < n4 / 4; i += T) reinterpret_cast<uint4 *>(s_lab)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+        for (uint32_t i = tid; i < nw; i += T) bits[i] = 0u;
+        if (tid < 3) {
+            s_cnt[tid] = tid == 2 ? 1u : 0u;  // the round before the first left one node: the root
+            s_min[tid] = kNever;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            s_lab[G.src] = 0u;
+            bits[G.src >> 5] = 1u << (G.src & 31u);
+            ring[0] = (uint16_t)G.src;
+        }
+        uint64_t theta = A.delta_ms;  // labels below theta are final or waiting
+        uint64_t next = theta + A.delta_ms;
+        uint32_t ub = kNever;         // latest destination label, once all are reached
+        uint32_t base = 0, room = kRing, cur = 0, prev = 2;  // cur: this round's counters
+        bool bounded = true, advanced = false;
+        __syncthreads();
+        for (uint64_t round = 0;; round++) {
+            if (round > max_rounds) {
+                bounded = false;
+                break;
+            }
+            const uint32_t cnt = s_cnt[prev], low = s_min[prev];
+            const bool over = cnt > room;  // ids did not fit: the bits say which nodes wait
+            const uint32_t c = over ? 0u : cnt;
+            room = kRing - c;
+            auto queue = [&](uint32_t v, uint64_t below, uint32_t label) {
+                if (label >= below) return;
+                const uint32_t bit = 1u << (v & 31u);
+                if (atomicOr(&bits[v >> 5], bit) & bit) return;
+                const uint32_t p = atomicAdd(&s_cnt[cur], 1u);
+                if (p < room) ring[(base + c + p) & (kRing - 1u)] = (uint16_t)v;
+            };
+            auto relax = [&](uint32_t u, uint32_t first, uint32_t step) {
+                const uint32_t tu = vlab[u];
+                if (tu >= ub) return;
+                const uint64_t t = t0 + tu;
+                const uint32_t j0 = A.wide ? u * A.wide : A.out_off[u], j1 = A.wide ? j0 + A.wide : A.out_off[u + 1];
+                const uint2 *row = A.cms + (size_t)bin_of(A, t) * A.n_pos;
+                for (uint32_t j = j0 + first; j < j1; j += step) {
+                    const uint32_t v = A.adj[j].y;
+                    const uint64_t at = arrive(row[j], t);
+                    if (v == kNever || at > 0xFFFFFFFFull) continue;
+                    const uint32_t rel = (uint32_t)(at - t0);
+                    if (rel > ub) continue;
+                    if (rel < atomicMin(&s_lab[v], rel)) queue(v, theta, rel);
+                }
+            };
+            if (tid == 0) {
+                const uint32_t after = cur == 2 ? 0u : cur + 1;
+                s_cnt[after] = 0u;
+                s_min[after] = kNever;
+            }
+            if (over) {
+                for (uint32_t w = tid; w < nw; w += T) {
+                    uint32_t m = atomicExch(&bits[w], 0u);
+                    while (m) {
+                        const uint32_t b = (uint32_t)__ffs((int)m) - 1u;
+                        m &= m - 1u;
+                        relax(32 * w + b, 0u, 1u);
+                    }
+                }
+            } else if (c > 0) {
+                for (uint32_t i0 = warp * 8; i0 < c; i0 += T / 4) {
+                    const uint32_t i = i0 + (lane >> 2);
+                    const uint32_t u = i < c ? ring[(base + i) & (kRing - 1u)] : 0u;
+                    if (i < c && (lane & 3u) == 0) atomicAnd(&bits[u >> 5], ~(1u << (u & 31u)));
+                    __syncwarp();  // the bit is cleared before any of the four lanes reads the label
+                    if (i < c) relax(u, lane & 3u, 4u);
+                    __syncwarp();
+                }
+            } else {
+                // nothing waits: every label below theta is final
+                if (advanced) {
+                    if (low == kNever) break;  // no label at or above theta either
+                    next = (uint64_t)low + A.delta_ms;  // an empty bucket: on to the earliest label
+                }
+                uint32_t m = 0;
+                for (uint32_t q = tid; q < G.count; q += T) m = max(m, vlab[A.dest[A.order[G.first + q]]]);
+                m = __reduce_max_sync(0xFFFFFFFFu, m);
+                if (lane == 0) s_red[warp] = m;
+                __syncthreads();
+                ub = 0;
+                for (uint32_t w = 0; w < T / 32; w++) ub = max(ub, s_red[w]);
+                if (ub < theta) break;  // every destination settled
+                uint32_t far = kNever;
+                for (uint32_t i = tid; i < n4 / 4; i += T) {
+                    const uint4 l = reinterpret_cast<const uint4 *>(s_lab)[i];
+                    const uint32_t ls[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        if (ls[k] == kNever || ls[k] < theta) continue;
+                        if (ls[k] >= next) far = min(far, ls[k]);
+                        else queue(4 * i + k, next, ls[k]);
+                    }
+                }
+                far = __reduce_min_sync(0xFFFFFFFFu, far);
+                if (lane == 0 && far != kNever) atomicMin(&s_min[cur], far);
+                theta = next;
+                next = theta + A.delta_ms;
+            }
+            advanced = !over && c == 0;
+            base += c;
+            prev = cur;
+            cur = cur == 2 ? 0u : cur + 1;
+            __syncthreads();
+        }
+        if (!bounded && tid == 0) atomicOr(A.err, kErrBound);
+        // paths of the group's trips, in travel order, timed from each trip's departure
+        for (uint32_t q = tid; q < G.count; q += T) {
+            const uint32_t jt = A.order[G.first + q];
+            const uint32_t d = A.dest[jt];
+            A.path_len[jt] = 0;
+            if (s_lab[d] == kNever || d == G.src || !bounded) {
+                atomicOr(A.err, kErrUnreachable);
+                continue;
+            }
+            // the tree's edge into v: {its out-edge position, its tail}; position kNoEdge: none (never on a
+            // finished search)
+            auto entering = [&](uint32_t v) {
+                const uint32_t tv = s_lab[v], i1 = A.in_off[v + 1];
+                for (uint32_t i = A.in_off[v]; i < i1; i++) {
+                    const uint2 in = A.in_adj[i];
+                    const uint32_t tu = s_lab[in.y];
+                    if (tu >= tv) continue;
+                    const uint64_t t = t0 + tu;
+                    if (arrive(A.cms[(size_t)bin_of(A, t) * A.n_pos + in.x], t) == t0 + tv) return in;
+                }
+                return make_uint2(kNoEdge, 0u);
+            };
+            uint32_t L = 0;
+            bool ok = true;
+            for (uint32_t v = d; v != G.src; L++) {
+                const uint2 in = entering(v);
+                if (L >= A.n_nodes || in.x == kNoEdge) {
+                    ok = false;
+                    break;
+                }
+                if (L < kScratch) scratch[(size_t)L * T] = in.x;
+                v = in.y;
+            }
+            if (!ok) {
+                atomicOr(A.err, kErrBound);
+                continue;
+            }
+            const unsigned long long off = atomicAdd(A.cursor, (unsigned long long)L);
+            if (off + L > A.cap) {
+                atomicOr(A.err, kErrCapacity);
+                continue;
+            }
+            if (L > kScratch) {  // a path longer than the scratch: its positions go through the output
+                uint32_t p = L;
+                for (uint32_t v = d; v != G.src && p > 0;) {
+                    const uint2 in = entering(v);
+                    A.edges[off + --p] = in.x;
+                    v = in.y;
+                }
+            }
+            const uint64_t tj = A.dep_ms[jt];
+            uint64_t t = tj;
+            for (uint32_t p = 0; p < L; p++) {
+                const uint32_t j = L > kScratch ? A.edges[off + p] : scratch[(size_t)(L - 1 - p) * T];
+                A.edges[off + p] = A.adj[j].x;
+                t = arrive(A.cms[(size_t)bin_of(A, t) * A.n_pos + j], t);
+            }
+            A.path_off[jt] = off;
+            A.path_len[jt] = L;
+            A.tsp[jt] = (float)((double)(t - tj) / 1000.0);
+        }
+    }
+}
+
+// cost_ms on the device: s * 1000 rounded to the nearest whole number (halves
+// up), at least 1 (NaN too), at most 2^31 - 1.  In integers: the product of a
+// 24-bit mantissa and 1000 is exact, as it is in the host's double (FP64
+// instructions made the table kernel three times as long).
+__device__ __forceinline__ uint32_t cost_ms_dev(float s) {
+    if (!(s > 0.0f)) return 1u;
+    if (s >= 4194304.0f) return 0x7FFFFFFFu;
+    const uint32_t u = __float_as_uint(s), sh = 150u - (u >> 23);  // s = mantissa * 2^-sh, sh >= 2
+    if (sh > 40u) return 1u;
+    const uint64_t v = (uint64_t)((u & 0x7FFFFFu) | 0x800000u) * 1000u;
+    const uint64_t r = (v + (1ull << (sh - 1u))) >> sh;
+    return (uint32_t)(r < 1u ? 1u : r > 0x7FFFFFFFu ? 0x7FFFFFFFu : r);
+}
+
+// The link-time table of tt (n_edges x n_bins seconds) in whole milliseconds,
+// by bin and position (adj: the edge at each, kNoEdge for none), as fill_link_times gives it on the host: per
+// (edge, bin) the time to the nearest ms (at least 1, at most 2^31 - 1) and the
+// earliest arrival entering a later bin.  A block takes 32 positions: its threads
+// read and convert tiles of 32 bins, last bins first, one warp carries the
+// minimum over the later bins and writes whole rows.  Bound by the bytes it
+// moves.
+__global__ void __launch_bounds__(256)
+    link_table(const float *tt, const uint2 *adj, uint32_t n_pos, uint32_t n_bins, uint64_t bin_ms, uint2 *out) {
+    __shared__ uint32_t c[32][33];
+    const uint32_t j0 = blockIdx.x * 32, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    uint64_t m = 0xFFFFFFFFull;
+    for (uint32_t b1 = n_bins; b1 > 0;) {
+        const uint32_t b0 = b1 > 32 ? b1 - 32 : 0;
+        for (uint32_t r = warp; r < 32; r += 8) {
+            const uint32_t e = j0 + r < n_pos ? adj[j0 + r].x : kNoEdge;
+            if (e == kNoEdge || b0 + lane >= b1) continue;
+            c[r][lane] = cost_ms_dev(tt[(size_t)e * n_bins + b0 + lane]);
+        }
+        __syncthreads();
+        if (warp == 0 && j0 + lane < n_pos)
+            for (uint32_t b = b1; b-- > b0;) {
+                const uint32_t v = c[lane][b - b0];
+                out[(size_t)b * n_pos + j0 + lane] = make_uint2(v, (uint32_t)m);
+                const uint64_t a = (uint64_t)b * bin_ms + v;
+                m = a < m ? a : m;
+            }
+        __syncthreads();
+        b1 = b0;
+    }
+}
+
 // every node unreached, with no round stamp and no far mark
 __global__ void init_nodes(NodeRec *nd, size_t n) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
@@ -379,8 +661,8 @@ __global__ void init_nodes(NodeRec *nd, size_t n) {
 // in the bin of every link entry time (the host's lpsim_assign_load, on the
 // device: integer counts, so the order of the atomics does not matter).
 __global__ void load_routes(const unsigned long long *roff, const uint32_t *redge, const uint32_t *dep_ms,
-                            uint64_t n, const uint2 *cms, uint32_t n_edges, uint32_t n_bins, uint32_t bin_ms,
-                            uint32_t *inflow) {
+                            uint64_t n, const uint2 *cms, const uint32_t *pos, uint32_t n_edges, uint32_t n_bins,
+                            uint32_t bin_ms, uint32_t *inflow) {
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < n; j += (uint64_t)gridDim.x * blockDim.x) {
         uint64_t t = dep_ms[j];
         const unsigned long long q1 = roff[j + 1];
@@ -388,7 +670,7 @@ __global__ void load_routes(const unsigned long long *roff, const uint32_t *redg
             const uint32_t e = redge[q];
             const uint64_t b = t / bin_ms;
             if (b < n_bins) atomicAdd(&inflow[(size_t)e * n_bins + b], 1u);
-            t = arrive(cms[(size_t)(b < n_bins ? b : n_bins - 1) * n_edges + e], t);
+            t = arrive(cms[(size_t)(b < n_bins ? b : n_bins - 1) * n_edges + (pos ? pos[e] : e)], t);
         }
     }
 }
@@ -410,31 +692,18 @@ struct AssignGpu {
     unsigned long long *roff = nullptr;
     uint32_t *redge = nullptr;
     uint64_t redge_cap = 0;
+    uint64_t routes_version = ~0ull;  // of the routes on the device
+    float *tt = nullptr;              // link times as given
+    size_t tt_cells = 0;
+    // td_trees_shared: its grid at most (0: td_trees searches), its arguments where they are not A's
+    void (*shared_kernel)(TreeArgs) = nullptr;
+    uint32_t shared_blocks = 0, shared_threads = 0;
+    const uint2 *wide_adj = nullptr, *wide_in = nullptr;
+    uint32_t wide = 0;
+    uint2 *table[2] = {};  // link-time tables: by out-edge position, by wide position
+    size_t table_cells[2] = {};
     uint32_t *inflow = nullptr;
     size_t inflow_cells = 0;
-    // host staging kept between calls (grown, never shrunk, never cleared:
-    // every call writes what it reads), so the large tables are not
-    // zero-filled and their pages not faulted in again at every call
-    std::unique_ptr<LinkTime[]> h_table;
-    size_t h_table_cap = 0;
-    std::unique_ptr<uint32_t[]> h_edges;
-    size_t h_edges_cap = 0;
-    LinkTime *table_buf(size_t n) {
-        if (n > h_table_cap) {
-            h_table.reset(new (std::nothrow) LinkTime[n]);
-            h_table_cap = h_table ? n : 0;
-        }
-        return h_table.get();
-    }
-    uint32_t *edges_buf(size_t n) {
-        n = std::max<size_t>(n, 1);
-        if (n > h_edges_cap) {
-            const size_t want = n + n / 4;
-            h_edges.reset(new (std::nothrow) uint32_t[want]);
-            h_edges_cap = h_edges ? want : 0;
-        }
-        return h_edges.get();
-    }
 
     void *alloc(size_t bytes) {
         void *p = nullptr;
@@ -474,6 +743,24 @@ int dput(AssignGpu *g, T *&dst, const T *src, size_t count) {
         if (rc_ != LPSIM_OK) return rc_; \
     } while (0)
 
+// The block that searches a tree of n_nodes nodes in shared memory: more threads
+// where fewer blocks fit an SM and near sets are larger.  Measured (blocks of
+// 256 at 32 registers / 256 / 512 / 1024 threads, ms per search with all its
+// host work; td_trees last): 2,750 nodes and 30k trips 0.49 / 0.55 / 0.71 /
+// 1.11, 2.0; 4,900 nodes 0.81 / 0.96 / 1.28 / 2.16; 10,000 nodes 2.27 / 2.24 / 2.88
+// / 4.66; 16,900 nodes 5.66 / 5.46 / 5.88 / 9.01; 27,225 nodes and 340k trips
+// 13.9 / 13.2 / 10.9 / 17.0, 18.5; 52,900 nodes 33.5 / 31.7 / 24.7 / 22.4, 31.5.
+// Bucket widths of 60 / 120 / 240 / 480 s: 27,225 nodes 15.0 / 13.6 / 12.3 / 12.9
+// (before the wide rows, which took 12.3 to 10.9).
+using TreeKernel = void (*)(TreeArgs);
+TreeKernel shared_tree_kernel(uint32_t n_nodes, int &threads) {
+    threads = n_nodes <= 20480 ? 256 : n_nodes <= 27648 ? 512 : 1024;
+    return n_nodes <= 6144    ? td_trees_shared<256, 8>
+           : threads == 256   ? td_trees_shared<256, 4>
+           : threads == 512   ? td_trees_shared<512, 2>
+                              : td_trees_shared<1024, 1>;
+}
+
 // graph, trips and workspaces (first call)
 int gpu_setup(lpsim_assign *a) {
     auto *g = new (std::nothrow) AssignGpu();
@@ -494,8 +781,28 @@ int gpu_setup(lpsim_assign *a) {
         if (t > 0xFFFFFFFFull) return fail(LPSIM_E_INVALID_ARG, "departure beyond the 32-bit millisecond range");
         dep_ms[j] = (uint32_t)t;
     }
-    uint32_t *oo, *sr, *de, *dm;
-    uint2 *ad;
+    // positions of the edges among the out-edges, and the in-edges of every node by ascending edge id
+    std::vector<uint32_t> pos(a->n_edges), in_off(a->n_nodes + 1, 0);
+    bool identity = true;
+    for (uint32_t j = 0; j < a->n_edges; j++) {
+        pos[a->out_edge[j]] = j;
+        identity = identity && a->out_edge[j] == j;
+        in_off[adj[j].y + 1]++;
+    }
+    for (uint32_t v = 0; v < a->n_nodes; v++) in_off[v + 1] += in_off[v];
+    std::vector<uint2> in_adj(a->n_edges);
+    {
+        std::vector<uint32_t> at(in_off.begin(), in_off.end() - 1);
+        for (uint32_t e = 0; e < a->n_edges; e++) in_adj[at[a->dst[e]]++] = make_uint2(pos[e], a->src[e]);
+    }
+    uint32_t *oo, *sr, *de, *dm, *po = nullptr, *io;
+    uint2 *ad, *ia;
+    if (!identity) TRY(dput(g, po, pos.data(), pos.size()));
+    TRY(dput(g, io, in_off.data(), in_off.size()));
+    TRY(dput(g, ia, in_adj.data(), in_adj.size()));
+    A.pos = po;
+    A.in_off = io;
+    A.in_adj = ia;
     TRY(dput(g, oo, a->out_off.data(), a->out_off.size()));
     TRY(dput(g, ad, adj.data(), adj.size()));
     TRY(dput(g, sr, a->src.data(), a->src.size()));
@@ -514,6 +821,51 @@ int gpu_setup(lpsim_assign *a) {
     A.err = static_cast<uint32_t *>(g->alloc(4));
     if (!A.path_off || !A.path_len || !A.tsp || !A.cursor || !A.next_group || !A.err)
         return fail(LPSIM_E_OOM, "device allocation failed");
+    A.delta_ms = kDeltaMs;
+    // labels in shared memory where they fit
+    const size_t smem = shared_tree_bytes(a->n_nodes);
+    cudaFuncAttributes fa{};
+    int max_smem = 0;
+    int threads = 0;
+    const TreeKernel kernel = shared_tree_kernel(a->n_nodes, threads);
+    CU(cudaFuncGetAttributes(&fa, kernel));
+    CU(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
+    if (a->n_nodes <= 0xFFFFu && smem + fa.sharedSizeBytes <= (size_t)max_smem) {
+        CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                max_smem - (int)fa.sharedSizeBytes));
+        int per_sm = 0;
+        CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
+        if (per_sm > 0) {
+            uint32_t most = 0;
+            for (uint32_t u = 0; u < a->n_nodes; u++) most = std::max(most, a->out_off[u + 1] - a->out_off[u]);
+            if (most <= kWide) {
+                const uint32_t w = most <= 4 ? 4 : 8;
+                std::vector<uint2> wadj((size_t)w * a->n_nodes, make_uint2(kNoEdge, kNever)), win(a->n_edges);
+                std::vector<uint32_t> at(in_off.begin(), in_off.end() - 1);
+                for (uint32_t u = 0; u < a->n_nodes; u++)
+                    for (uint32_t j = a->out_off[u]; j < a->out_off[u + 1]; j++)
+                        wadj[(size_t)u * w + (j - a->out_off[u])] = adj[j];
+                for (uint32_t e = 0; e < a->n_edges; e++) {
+                    const uint32_t u = a->src[e];
+                    win[at[a->dst[e]]++] = make_uint2(u * w + (pos[e] - a->out_off[u]), u);
+                }
+                uint2 *wa, *wi;
+                TRY(dput(g, wa, wadj.data(), wadj.size()));
+                TRY(dput(g, wi, win.data(), win.size()));
+                CU(cudaStreamSynchronize(g->stream));
+                g->wide_adj = wa;
+                g->wide_in = wi;
+                g->wide = w;
+            }
+            g->shared_kernel = kernel;
+            g->shared_threads = (uint32_t)threads;
+            g->shared_blocks = (uint32_t)(g->n_sm * per_sm);
+            A.scratch = static_cast<uint32_t *>(g->alloc((size_t)g->shared_blocks * threads * kScratch * 4));
+            if (!A.scratch) return fail(LPSIM_E_OOM, "device allocation of the search workspaces failed");
+            CU(cudaStreamSynchronize(g->stream));  // the host arrays go away
+            return LPSIM_OK;
+        }
+    }
     // workspaces: as many warps as fit the budget, at most kBlocksPerSm * kWarpsPerBlock per SM
     const uint64_t per_warp = (uint64_t)a->n_nodes * (sizeof(NodeRec) + 4 * 4);
     uint64_t warps = std::min<uint64_t>((uint64_t)g->n_sm * kBlocksPerSm * kWarpsPerBlock,
@@ -531,10 +883,20 @@ int gpu_setup(lpsim_assign *a) {
         return fail(LPSIM_E_OOM, "device allocation of the search workspaces failed");
     init_nodes<<<g->n_sm * 4, 256, 0, g->stream>>>(A.node, nn);
     CU(cudaGetLastError());
-    A.delta_ms = kDeltaMs;
     CU(cudaMemsetAsync(A.stamp, 0, warps * 4, g->stream));
     CU(cudaStreamSynchronize(g->stream));
     return LPSIM_OK;
+}
+
+// the device copy, made at the first call (a failed attempt leaves none)
+int gpu_ready(lpsim_assign *a) {
+    if (a->gpu) return LPSIM_OK;
+    const int rc = gpu_setup(a);
+    if (rc) {
+        assign_gpu_free(a->gpu);
+        a->gpu = nullptr;
+    }
+    return rc;
 }
 
 // trip groups of a departure period length (kept between calls)
@@ -570,31 +932,38 @@ int gpu_groups(lpsim_assign *a, uint32_t period_steps) {
 
 namespace {
 
-// the link-time table of tt in whole milliseconds (the host searches' table) on the device
-int gpu_table(lpsim_assign *a, const float *tt, uint32_t n_bins, uint32_t bin_steps) {
+// the link-time table of tt in whole milliseconds on the device (as the host
+// searches' table), by out-edge position (A.cms) or, for a search with wide
+// rows, by those
+int gpu_table(lpsim_assign *a, const float *tt, uint32_t n_bins, uint32_t bin_steps, bool wide) {
     AssignGpu *g = a->gpu;
     TreeArgs &A = g->A;
     const uint64_t bin_ms = table_bin_ms(a, bin_steps);
     if (bin_ms > 0xFFFFFFFFull) return fail(LPSIM_E_INVALID_ARG, "bin longer than the 32-bit millisecond range");
-    static_assert(sizeof(LinkTime) == sizeof(uint2), "link-time record");
-    const size_t cells = (size_t)n_bins * a->n_edges;
-    // the previous call's upload of the staging table has finished (each call synchronises)
-    LinkTime *tbm = g->table_buf(cells);
-    if (!tbm) return fail(LPSIM_E_OOM, "host allocation of the link-time table failed");
-    fill_link_times(a, tt, n_bins, bin_ms, tbm);
-    if (A.cms && A.n_bins != n_bins) {
-        g->release(const_cast<uint2 *>(A.cms));
-        A.cms = nullptr;
+    const uint32_t n_pos = wide ? g->wide * a->n_nodes : a->n_edges;
+    const size_t in_cells = (size_t)n_bins * a->n_edges, cells = (size_t)n_bins * n_pos;
+    if (cells > g->table_cells[wide]) {
+        if (g->table[wide]) g->release(g->table[wide]);
+        g->table_cells[wide] = 0;
+        g->table[wide] = static_cast<uint2 *>(g->alloc(cells * sizeof(uint2)));
+        if (!g->table[wide]) return fail(LPSIM_E_OOM, "device allocation of the link-time table failed");
+        g->table_cells[wide] = cells;
     }
-    if (!A.cms) {
-        A.cms = static_cast<uint2 *>(g->alloc(cells * sizeof(uint2)));
-        if (!A.cms) return fail(LPSIM_E_OOM, "device allocation of the link-time table failed");
+    if (in_cells > g->tt_cells) {
+        if (g->tt) g->release(g->tt);
+        g->tt_cells = 0;
+        g->tt = static_cast<float *>(g->alloc(in_cells * 4));
+        if (!g->tt) return fail(LPSIM_E_OOM, "device allocation of the link times failed");
+        g->tt_cells = in_cells;
     }
-    CU(cudaMemcpyAsync(const_cast<uint2 *>(A.cms), tbm, cells * sizeof(uint2), cudaMemcpyHostToDevice, g->stream));
+    CU(cudaMemcpyAsync(g->tt, tt, in_cells * 4, cudaMemcpyHostToDevice, g->stream));
+    if (n_pos)
+        link_table<<<(n_pos + 31) / 32, 256, 0, g->stream>>>(g->tt, wide ? g->wide_adj : A.adj, n_pos, n_bins, bin_ms,
+                                                            g->table[wide]);
+    CU(cudaGetLastError());
+    A.cms = g->table[wide];
     A.n_bins = n_bins;
     A.bin_ms = (uint32_t)bin_ms;
-    // the staging table is rewritten by the next call: let the copy finish first
-    CU(cudaStreamSynchronize(g->stream));
     return LPSIM_OK;
 }
 
@@ -608,31 +977,33 @@ extern "C" int lpsim_assign_load_gpu(const lpsim_assign *ac, const float *tt, ui
         std::memset(inflow, 0, (size_t)a->n_edges * n_bins * 4);
         return LPSIM_OK;
     }
-    if (!a->gpu) TRY(gpu_setup(a));
+    TRY(gpu_ready(a));
     AssignGpu *g = a->gpu;
     int dev = -1;
     CU(cudaGetDevice(&dev));
     if (dev != g->device) return fail(LPSIM_E_STATE, "the device current at the first GPU call must be current");
-    TRY(gpu_table(a, tt, n_bins, bin_steps));
-    // the current routes, flattened (offsets on the host's threads)
-    std::vector<unsigned long long> off(a->n + 1);
-    off[0] = 0;
-    for (uint64_t j = 0; j < a->n; j++) off[j + 1] = off[j] + a->route[j].size();
-    const uint64_t total = off[a->n];
-    uint32_t *edges = g->edges_buf(total);
-    if (!edges) return fail(LPSIM_E_OOM, "host allocation of the route staging failed");
-    lpsim::parallel_pieces(a->n, [&](uint64_t j0, uint64_t j1, uint64_t) {
-        for (uint64_t j = j0; j < j1; j++) std::memcpy(edges + off[j], a->route[j].data(), a->route[j].size() * 4);
-    });
+    TRY(gpu_table(a, tt, n_bins, bin_steps, false));
+    // the engine's routes stay on the device until a re-routing changes them
     if (!g->roff) {
         g->roff = static_cast<unsigned long long *>(g->alloc((a->n + 1) * 8));
         if (!g->roff) return fail(LPSIM_E_OOM, "device allocation of the route offsets failed");
     }
-    if (total > g->redge_cap) {
-        if (g->redge) g->release(g->redge);
-        g->redge_cap = total + total / 4;
-        g->redge = static_cast<uint32_t *>(g->alloc(g->redge_cap * 4));
-        if (!g->redge) return fail(LPSIM_E_OOM, "device allocation of the routes failed");
+    if (g->routes_version != a->routes_version) {
+        const uint64_t total = a->roff[a->n];
+        if (total > g->redge_cap) {
+            if (g->redge) g->release(g->redge);
+            g->redge = nullptr;
+            g->redge_cap = 0;
+            g->redge = static_cast<uint32_t *>(g->alloc((total + total / 4) * 4));
+            if (!g->redge) return fail(LPSIM_E_OOM, "device allocation of the routes failed");
+            g->redge_cap = total + total / 4;
+        }
+        g->routes_version = ~0ull;
+        CU(cudaMemcpyAsync(g->roff, a->roff.data(), (a->n + 1) * 8, cudaMemcpyHostToDevice, g->stream));
+        if (total)
+            CU(cudaMemcpyAsync(g->redge, a->redge.p.get(), total * 4, cudaMemcpyHostToDevice, g->stream));
+        CU(cudaStreamSynchronize(g->stream));
+        g->routes_version = a->routes_version;
     }
     const size_t cells = (size_t)a->n_edges * n_bins;
     if (cells > g->inflow_cells) {
@@ -641,11 +1012,9 @@ extern "C" int lpsim_assign_load_gpu(const lpsim_assign *ac, const float *tt, ui
         if (!g->inflow) return fail(LPSIM_E_OOM, "device allocation of the inflow table failed");
         g->inflow_cells = cells;
     }
-    CU(cudaMemcpyAsync(g->roff, off.data(), (a->n + 1) * 8, cudaMemcpyHostToDevice, g->stream));
-    if (total) CU(cudaMemcpyAsync(g->redge, edges, total * 4, cudaMemcpyHostToDevice, g->stream));
     CU(cudaMemsetAsync(g->inflow, 0, cells * 4, g->stream));
     load_routes<<<(unsigned)std::min<uint64_t>((a->n + 255) / 256, 65535), 256, 0, g->stream>>>(
-        g->roff, g->redge, g->A.dep_ms, a->n, g->A.cms, a->n_edges, n_bins, g->A.bin_ms, g->inflow);
+        g->roff, g->redge, g->A.dep_ms, a->n, g->A.cms, g->A.pos, a->n_edges, n_bins, g->A.bin_ms, g->inflow);
     CU(cudaGetLastError());
     CU(cudaMemcpyAsync(inflow, g->inflow, cells * 4, cudaMemcpyDeviceToHost, g->stream));
     CU(cudaStreamSynchronize(g->stream));
@@ -657,19 +1026,17 @@ extern "C" int lpsim_assign_shortest_paths_gpu(lpsim_assign *a, const float *tt,
     if (!a || !tt || n_bins == 0 || bin_steps == 0 || period_steps == 0)
         return fail(LPSIM_E_INVALID_ARG, "bad argument");
     if (a->n == 0) return LPSIM_OK;
-    if (!a->gpu) TRY(gpu_setup(a));
+    TRY(gpu_ready(a));
     AssignGpu *g = a->gpu;
     int dev = -1;
     CU(cudaGetDevice(&dev));
     if (dev != g->device) return fail(LPSIM_E_STATE, "the device current at the first GPU search must be current");
     TRY(gpu_groups(a, period_steps));
     TreeArgs &A = g->A;
-    // link times in whole milliseconds, bin-major (the host searches' table)
-    TRY(gpu_table(a, tt, n_bins, bin_steps));
+    TRY(gpu_table(a, tt, n_bins, bin_steps, g->wide != 0));
     // path buffer: room for the current routes' length and half as much again
     if (!g->cap) {
-        uint64_t total = 0;
-        for (auto &r : a->route) total += r.size();
+        const uint64_t total = a->roff[a->n];
         g->cap = std::max<uint64_t>(total + total / 2, 1u << 20);
         A.edges = static_cast<uint32_t *>(g->alloc(g->cap * 4));
         if (!A.edges) return fail(LPSIM_E_OOM, "device allocation of the path buffer failed");
@@ -681,7 +1048,19 @@ extern "C" int lpsim_assign_shortest_paths_gpu(lpsim_assign *a, const float *tt,
         CU(cudaMemsetAsync(A.cursor, 0, 8, g->stream));
         CU(cudaMemsetAsync(A.next_group, 0, 4, g->stream));
         CU(cudaMemsetAsync(A.err, 0, 4, g->stream));
-        td_trees<<<g->n_warps / kWarpsPerBlock, kWarpsPerBlock * 32, 0, g->stream>>>(A);
+        if (g->shared_blocks) {
+            TreeArgs S = A;
+            S.delta_ms = kSharedDeltaMs;
+            S.wide = g->wide;
+            S.n_pos = g->wide ? g->wide * a->n_nodes : a->n_edges;
+            if (g->wide) {
+                S.adj = g->wide_adj;
+                S.in_adj = g->wide_in;
+            }
+            g->shared_kernel<<<std::min(g->shared_blocks, std::max(A.n_groups, 1u)), g->shared_threads,
+                               shared_tree_bytes(a->n_nodes), g->stream>>>(S);
+        } else
+            td_trees<<<g->n_warps / kWarpsPerBlock, kWarpsPerBlock * 32, 0, g->stream>>>(A);
         CU(cudaGetLastError());
         CU(cudaMemcpyAsync(&used, A.cursor, 8, cudaMemcpyDeviceToHost, g->stream));
         CU(cudaMemcpyAsync(&err, A.err, 4, cudaMemcpyDeviceToHost, g->stream));
@@ -696,18 +1075,15 @@ extern "C" int lpsim_assign_shortest_paths_gpu(lpsim_assign *a, const float *tt,
     if (err & kErrBound) return fail(LPSIM_E_INVARIANT, "GPU path search exceeded its round or path-length bound");
     if (err & kErrUnreachable) return fail(LPSIM_E_INVALID_ARG, "a destination is unreachable from its origin");
     if (err & kErrCapacity) return fail(LPSIM_E_OOM, "path buffer still too small after resizing");
-    std::vector<unsigned long long> off(a->n);
-    std::vector<uint32_t> len(a->n);
-    uint32_t *edges = g->edges_buf(used);
-    if (!edges) return fail(LPSIM_E_OOM, "host allocation of the path staging failed");
-    CU(cudaMemcpyAsync(off.data(), A.path_off, a->n * 8, cudaMemcpyDeviceToHost, g->stream));
-    CU(cudaMemcpyAsync(len.data(), A.path_len, a->n * 4, cudaMemcpyDeviceToHost, g->stream));
+    // the candidates as the search left them: offsets, lengths and one array of edges
+    std::fill(a->clen.begin(), a->clen.end(), 0u);
+    if (!a->cedge.reserve(used)) return fail(LPSIM_E_OOM, "host allocation of the paths failed");
+    static_assert(sizeof(unsigned long long) == sizeof(uint64_t), "path offsets");
+    if (used) CU(cudaMemcpyAsync(a->cedge.p.get(), A.edges, used * 4, cudaMemcpyDeviceToHost, g->stream));
+    CU(cudaMemcpyAsync(a->coff.data(), A.path_off, a->n * 8, cudaMemcpyDeviceToHost, g->stream));
     CU(cudaMemcpyAsync(a->tsp.data(), A.tsp, a->n * 4, cudaMemcpyDeviceToHost, g->stream));
-    if (used) CU(cudaMemcpyAsync(edges, A.edges, used * 4, cudaMemcpyDeviceToHost, g->stream));
+    CU(cudaMemcpyAsync(a->clen.data(), A.path_len, a->n * 4, cudaMemcpyDeviceToHost, g->stream));
     CU(cudaStreamSynchronize(g->stream));
-    lpsim::parallel_pieces(a->n, [&](uint64_t j0, uint64_t j1, uint64_t) {
-        for (uint64_t j = j0; j < j1; j++) a->cand[j].assign(edges + off[j], edges + off[j] + len[j]);
-    });
     if (t_sp) std::memcpy(t_sp, a->tsp.data(), a->n * 4);
     return LPSIM_OK;
 }

@@ -5,12 +5,32 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <cstring>
+#include <memory>
+#include <new>
 #include <vector>
 
 #include "host_par.h"
 
 struct AssignGpu;  // device copy of the graph and search workspaces (assign_gpu.cu)
 void assign_gpu_free(AssignGpu *g);
+
+// edge ids on the host, grown and kept, never cleared (a fresh buffer's pages
+// fault in at first touch: as slow as writing the ids)
+struct EdgeBuf {
+    std::unique_ptr<uint32_t[]> p;
+    uint64_t cap = 0;
+    // room for n ids (contents not kept); false when out of memory
+    bool reserve(uint64_t n) {
+        n = std::max<uint64_t>(n, 1);
+        if (n > cap) {
+            p.reset();
+            p.reset(new (std::nothrow) uint32_t[n + n / 4]);
+            cap = p ? n + n / 4 : 0;
+        }
+        return p != nullptr;
+    }
+};
 
 struct lpsim_assign {
     uint32_t n_nodes = 0, n_edges = 0;
@@ -20,13 +40,29 @@ struct lpsim_assign {
     // trips
     uint64_t n = 0;
     std::vector<uint32_t> orig, dest, dep;    // depart step
-    std::vector<std::vector<uint32_t>> route, cand;
+    // current routes, flat: trip j's edges are redge[roff[j]..roff[j + 1]), as a
+    // simulation, a route loading and the device take them; routes_version counts
+    // their changes
+    std::vector<uint64_t> roff;
+    EdgeBuf redge, redge_next;                // the routes; where the next ones are written
+    uint64_t routes_version = 0;
+    // candidate paths of the last search: trip j's edges are cedge[coff[j]..+clen[j])
+    // (clen 0: none yet)
+    std::vector<uint64_t> coff;
+    std::vector<uint32_t> clen;
+    EdgeBuf cedge;
     std::vector<float> tsp;                   // shortest time under the last tt (s)
     std::vector<float> excess;                // current route's time minus tsp (s), from a simulation or a prediction
     float dt = 0.5f;
     uint64_t seed = 0;
     AssignGpu *gpu = nullptr;
     ~lpsim_assign() { assign_gpu_free(gpu); }
+    const uint32_t *route(uint64_t j) const { return redge.p.get() + roff[j]; }
+    uint64_t route_len(uint64_t j) const { return roff[j + 1] - roff[j]; }
+    const uint32_t *cand(uint64_t j) const { return cedge.p.get() + coff[j]; }
+    bool cand_differs(uint64_t j) const {
+        return clen[j] != route_len(j) || std::memcmp(cand(j), route(j), (size_t)clen[j] * 4) != 0;
+    }
 };
 
 namespace lpsim_assign_detail {

@@ -83,6 +83,69 @@ def test_gpu_load_equals_host_load(scale):
     A.close()
 
 
+def _lattice(side):
+    i = np.arange(side * side)
+    r, c = np.divmod(i, side)
+    src = np.concatenate([i[c < side - 1], i[c > 0], i[r < side - 1], i[r > 0]])
+    dst = np.concatenate([i[c < side - 1] + 1, i[c > 0] - 1, i[r < side - 1] + side, i[r > 0] - side])
+    return side * side, src, dst
+
+
+def _odd_network(kind):
+    """{nodes, edge tails, edge heads, origins and destinations of trips}"""
+    rng = np.random.default_rng(5)
+    if kind == "hub":  # 3,000 nodes reached in one round
+        n = 3000
+        src = np.concatenate([np.zeros(n, int), np.arange(1, n + 1)])
+        dst = np.concatenate([np.arange(1, n + 1), np.full(n, n + 1)])
+        return n + 2, src, dst, np.zeros(40, int), np.concatenate([np.full(20, n + 1), rng.integers(1, n + 1, 20)])
+    if kind == "line":  # paths of up to 1,499 edges
+        n = 1500
+        return n, np.arange(n - 1), np.arange(1, n), np.zeros(40, int), rng.integers(1, n, 40)
+    n, src, dst = _lattice(int(kind))
+    o = rng.integers(0, n, 12).repeat(8)
+    d = rng.integers(0, n, len(o))
+    return n, src, dst, o, np.where(d == o, (d + 1) % n, d)
+
+
+@pytest.mark.parametrize("kind", ["2", "5", "hub", "line", "90", "91", "236", "237"])
+@pytest.mark.parametrize("n_bins,shuffled", [(1, True), (33, False), (96, True)])
+def test_gpu_paths_on_odd_networks(kind, n_bins, shuffled):
+    """Where the search can go wrong: a tree of a few nodes, more waiting nodes
+    than the ring of ids holds, paths longer than the walk's scratch, networks on
+    both sides of each choice of block (90 x 90 and 91 x 91 nodes) and of the
+    largest whose labels fit in shared memory (236 x 236 do, 237 x 237 do
+    not), edge ids in no order, and link times of one to three seconds, so that
+    many paths tie: routes and times equal the host's bit for bit."""
+    from paper_2406_08496_gb300.assignment import Assignment
+    n, src, dst, o, d = _odd_network(kind)
+    rng = np.random.default_rng(6)
+    if shuffled:
+        p = rng.permutation(len(src))
+        src, dst = src[p], dst[p]
+    m = len(src)
+    net = {"n_nodes": n, "n_edges": m, "edge_src": src.astype(np.uint32), "edge_dst": dst.astype(np.uint32),
+           "edge_len": np.full(m, 100.0, np.float32), "edge_lanes": np.ones(m, np.uint8),
+           "edge_vmax": np.full(m, 10.0, np.float32)}
+    dem = {"orig": o.astype(np.uint32), "dest": d.astype(np.uint32),
+           "depart_step": rng.integers(0, 4000, len(o)).astype(np.uint32),
+           "route_off": np.arange(len(o) + 1, dtype=np.uint64), "route_edges": np.zeros(len(o), np.uint32)}
+    tt = rng.integers(1, 4, (m, n_bins)).astype(np.float32)
+    host, gpu = Assignment(net, dem, seed=1), Assignment(net, dem, seed=1)
+    for period in (600, 7):
+        th, rh = _paths(host, host.shortest_paths, tt, 60, period)
+        tg, rg = _paths(gpu, gpu.shortest_paths_gpu, tt, 60, period)
+        assert np.array_equal(th.view(np.uint32), tg.view(np.uint32))
+        assert np.array_equal(rh["route_off"], rg["route_off"])
+        assert np.array_equal(rh["route_edges"], rg["route_edges"])
+        assert np.array_equal(host.load(tt, 60), gpu.load_gpu(tt, 60))
+    # times that round to less than a millisecond, to a half, and past 2^31 ms
+    odd = rng.choice(np.array([0.0, -3.0, 1e-4, 0.0005, 0.0025, 1.5, 2147483.5, 3e6], np.float32), (m, n_bins))
+    assert np.array_equal(host.load(odd, 60), gpu.load_gpu(odd, 60))
+    host.close()
+    gpu.close()
+
+
 def test_gpu_paths_match_brute_force():
     """On a five-edge diamond, every trip's GPU route is an earliest-arrival
     path among all simple paths, from the middle of its period, and its time
