@@ -69,8 +69,18 @@ __device__ __forceinline__ uint8_t speed_byte(float v) {
 // are bytes, 0xFF when empty, so a word's complement has a nonzero byte per
 // occupied cell: the search picks the first (or last) nonzero word of the
 // window, the cells before the window's start masked off its first chunk, and
-// the byte within it; a find past the window's end is none.  (A 16-bit mask
-// built per chunk from byte compares took four times the instructions.)
+// the byte within it, which is also the found vehicle's speed (no load of its
+// own); a find past the window's end is none.  (A 16-bit mask built per chunk
+// from byte compares took four times the instructions.)
+
+struct Found {
+    uint32_t cell;   // kNone: no occupied cell
+    uint32_t speed;  // its byte
+};
+
+__device__ __forceinline__ Found found_in(uint32_t word_cell, uint32_t w, uint32_t byte) {
+    return {word_cell + byte, (~w >> (8u * byte)) & 0xFFu};
+}
 
 // the complements of chunks c_first, c_first + step, ... (N of them, loaded
 // together: one memory round trip), zero where `in` says the window has ended
@@ -100,9 +110,9 @@ __device__ __forceinline__ void load_ahead(const uint8_t *row, uint32_t lo, uint
     for (int j = 0; j < 4; j++) w[j] &= __funnelshift_lc(0u, ~0u, max((int)(8u * (lo & 15u)) - 32 * j, 0));
 }
 
-// first occupied cell at or after lo in the loaded chunks, or kNone
+// first occupied cell at or after lo in the loaded chunks
 template <int N>
-__device__ __forceinline__ uint32_t find_first(const uint32_t (&w)[4 * N], uint32_t lo) {
+__device__ __forceinline__ Found find_first(const uint32_t (&w)[4 * N], uint32_t lo) {
     uint32_t t = 0, at = 0;
 #pragma unroll
     for (int j = 4 * N - 1; j >= 0; j--)
@@ -110,7 +120,7 @@ __device__ __forceinline__ uint32_t find_first(const uint32_t (&w)[4 * N], uint3
             t = w[j];
             at = 4u * j;
         }
-    return t ? (lo & ~15u) + at + ((uint32_t)(__ffs((int)t) - 1) >> 3) : kNone;
+    return t ? found_in((lo & ~15u) + at, t, (uint32_t)(__ffs((int)t) - 1) >> 3) : Found{kNone, 0u};
 }
 
 // chunks of [lo, hi] from hi's down, the cells after hi dropped
@@ -122,9 +132,9 @@ __device__ __forceinline__ void load_behind(const uint8_t *row, uint32_t lo, uin
     for (int j = 0; j < 4; j++) w[j] &= __funnelshift_rc(~0u, 0u, max(32 * (j + 1) - 8 * (int)((hi & 15u) + 1u), 0));
 }
 
-// last occupied cell at or before hi in the loaded chunks, or kNone
+// last occupied cell at or before hi in the loaded chunks
 template <int N>
-__device__ __forceinline__ uint32_t find_last(const uint32_t (&w)[4 * N], uint32_t hi) {
+__device__ __forceinline__ Found find_last(const uint32_t (&w)[4 * N], uint32_t hi) {
     uint32_t t = 0, at = 0;
 #pragma unroll
     for (int j = N - 1; j >= 0; j--)
@@ -134,23 +144,24 @@ __device__ __forceinline__ uint32_t find_last(const uint32_t (&w)[4 * N], uint32
                 t = w[4 * j + i];
                 at = 16u * j - 4u * i;
             }
-    return t ? (hi & ~15u) - at + ((uint32_t)(31 - __clz((int)t)) >> 3) : kNone;
+    return t ? found_in((hi & ~15u) - at, t, (uint32_t)(31 - __clz((int)t)) >> 3) : Found{kNone, 0u};
 }
 
-// first occupied cell in [lo, hi], or kNone; the first four 16-byte chunks of
+// first occupied cell in [lo, hi]; the first four 16-byte chunks of
 // the window are loaded together, so a window of up to 49 cells costs one
 // memory round trip
-__device__ __forceinline__ uint32_t first_occupied_wide(const uint8_t *row, uint32_t lo, uint32_t hi) {
-    if (lo > hi) return kNone;
+__device__ __forceinline__ Found first_occupied_wide(const uint8_t *row, uint32_t lo, uint32_t hi) {
+    if (lo > hi) return {kNone, 0u};
     uint32_t w[16];
     load_ahead<4>(row, lo, hi, w);
-    uint32_t f = find_first<4>(w, lo);
-    for (uint32_t c = (lo & ~15u) + 64u; f == kNone && c <= hi; c += 16u) {
+    Found f = find_first<4>(w, lo);
+    for (uint32_t c = (lo & ~15u) + 64u; f.cell == kNone && c <= hi; c += 16u) {
         uint32_t u[4];
         load_ahead<1>(row, c, hi, u);
         f = find_first<1>(u, c);
     }
-    return f <= hi ? f : kNone;
+    if (f.cell > hi) f.cell = kNone;
+    return f;
 }
 
 // car-following parameters of one vehicle (its type's, or the run's)
@@ -495,12 +506,13 @@ __device__ __forceinline__ bool p1_slot(const Dev &d, const StepView &w, const P
                                          : d.hkey[id];
     uint32_t hi = c + (uint32_t)fminf(reach, 65535.0f) + 2u;
     if (hi > len - 1) hi = len - 1;
-    const uint32_t cf = first_occupied_wide(Mc + base, c + 1, hi);
+    const Found lead = first_occupied_wide(Mc + base, c + 1, hi);
+    const uint32_t cf = lead.cell;
     const bool has_f = cf != kNone;
 
     float vn;
     if (has_f && ((float)cf - x) <= d_front)
-        vn = idm_speed(y, m.dt, v, (float)Mc[base + cf], (float)cf - x, v0);
+        vn = idm_speed(y, m.dt, v, (float)lead.speed, (float)cf - x, v0);
     else
         vn = v0;
     float xn = x + vn * m.dt;
@@ -578,7 +590,7 @@ __device__ __forceinline__ bool p1_slot(const Dev &d, const StepView &w, const P
             up = tl > ln ? 1u : 0u;
         }
     } else if (m.dlc_prob > 0.0f && has_f && vn < v0 && !(tl != kNoLane && tl != ln && (L - x) < m.x0) &&
-               (float)Mc[base + cf] < v0) {
+               (float)lead.speed < v0) {
         // discretionary lane change (outside the mandatory zone, held below
         // its free speed by a slower leader): one lane up on odd steps, down
         // on even ones, when that lane's lead gap is absent or longer by
@@ -588,7 +600,7 @@ __device__ __forceinline__ bool p1_slot(const Dev &d, const StepView &w, const P
         if (up ? ln + 1 < nl : ln > 0) {
             const uint32_t stride = row_stride(len);
             const uint32_t base2 = up ? base + stride : base - stride;
-            const uint32_t ca = first_occupied_wide(Mc + base2, c, min(c + 63u, len - 1));
+            const uint32_t ca = first_occupied_wide(Mc + base2, c, min(c + 63u, len - 1)).cell;
             if (ca == kNone || (float)ca - (float)cf >= m.dlc_gain) {
                 hkd = d.hkey_from_id ? d.m.seed ^ ((uint64_t)id * 0x9E3779B97F4A7C15ull) : d.hkey[id];
                 intend = unit24(splitmix64_mix(hkd ^ ((uint64_t)k * 0xD1B54A32D192ED03ull))) < m.dlc_prob;
@@ -823,10 +835,9 @@ __device__ __forceinline__ void lane_change(const Dev &d, const StepView &w, con
     uint64_t h = 0;
     if (m.eps_amp > 0.0f) h = splitmix64_mix(ir.hk ^ ((uint64_t)k * 0xD1B54A32D192ED03ull));
     // lead: first occupied cell in [c0, hi]; lag: last in [lo, c0 - 1]
-    uint32_t ca = find_first<5>(wa, c0);
-    if (ca > hi) ca = kNone;
-    uint32_t cb = c0 > 0 ? find_last<5>(wb, c0 - 1) : kNone;
-    if (cb != kNone && cb < lo) cb = kNone;
+    const Found fa = find_first<5>(wa, c0), fb = find_last<5>(wb, c0 > 0 ? c0 - 1 : 0u);
+    const uint32_t ca = fa.cell <= hi ? fa.cell : kNone;
+    const uint32_t cb = c0 > 0 && fb.cell != kNone && fb.cell >= lo ? fb.cell : kNone;
     float eps_a = 0.0f, eps_b = 0.0f;
     if (m.eps_amp > 0.0f) {
         eps_a = m.eps_amp * (2.0f * unit24(splitmix64_mix(h ^ 0x632BE59BD9B4E019ull)) - 1.0f);
@@ -834,12 +845,12 @@ __device__ __forceinline__ void lane_change(const Dev &d, const StepView &w, con
     }
     bool ok = true;
     if (ca != kNone) {
-        const float va = (float)row2[ca];
+        const float va = (float)fa.speed;
         const float G_lead = (m.g_a + fmax0(m.alpha_i * vn - m.alpha_a * va)) + eps_a;
         ok = ((float)ca - xn) >= G_lead;
     }
     if (ok && cb != kNone) {
-        const float vb = (float)row2[cb];
+        const float vb = (float)fb.speed;
         const float G_lag = (m.g_b + fmax0(m.alpha_b * vb - m.alpha_i * vn)) + eps_b;
         ok = (xn - (float)cb) >= G_lag;
     }
