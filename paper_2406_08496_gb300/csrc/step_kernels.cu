@@ -401,10 +401,9 @@ __device__ __forceinline__ void p1_origin(const Dev &d, const StepView &w, const
     }
 }
 
-// Slot s (every field loaded in one round trip, together with whatever the
-// caller loaded just before); false once s is past the slot count n.
-__device__ __forceinline__ bool p1_slot(const Dev &d, const StepView &w, const P1Sinks &sk, uint32_t s, uint32_t n,
-                                        uint32_t &live, uint32_t &arrived) {
+// Slot s (every field loaded in one round trip).
+__device__ __forceinline__ void p1_slot(const Dev &d, const StepView &w, const P1Sinks &sk, uint32_t s, uint32_t &live,
+                                        uint32_t &arrived) {
     const uint32_t k = w.k, par = w.par;
     const uint8_t *Mc = w.Mc;
     uint8_t *Mn = w.Mn, *Mo = w.Mo, *Iw = w.Iw, *Io = w.Io;
@@ -413,8 +412,7 @@ __device__ __forceinline__ bool p1_slot(const Dev &d, const StepView &w, const P
     float *xw = w.xw, *vw = w.vw;
     const bool sample = w.sample;
     const Model &m = d.m;
-    // every slot field, loaded together (one memory round trip, shared
-    // with the loads of the step number and the slot count)
+    // every slot field, loaded together (one memory round trip)
     const uint8_t flag = d.s.flag[s];
     const uint32_t pc = d.s.pcell[s];
     const uint32_t im = d.s.imark[s];
@@ -430,9 +428,7 @@ __device__ __forceinline__ bool p1_slot(const Dev &d, const StepView &w, const P
     const uint32_t ln = d.s.lane[s];
     const uint32_t id = d.s.id[s];
     const uint32_t rpos = es.rpos, rlast = d.s.rlast[s];
-    loads_issued();
-    if (s >= n) return false;
-    if (flag == kDead) return true;
+    if (flag == kDead) return;
     if (pc != kNone) Mo[pc] = kEmpty;
     if (im != kNone) {
         Io[im] = 0;
@@ -445,7 +441,7 @@ __device__ __forceinline__ bool p1_slot(const Dev &d, const StepView &w, const P
     if (flag == kArrivedPending) {
         d.s.flag[s] = kDead;
         d.s.pcell[s] = kNone;
-        return true;
+        return;
     }
     live++;
     const uint32_t c = (uint32_t)x;
@@ -531,7 +527,7 @@ __device__ __forceinline__ bool p1_slot(const Dev &d, const StepView &w, const P
             d.status[id] = kArrived;
             d.s.flag[s] = kArrivedPending;
             arrived++;
-            return true;
+            return;
         }
         bool cross = false;
         if (green) {
@@ -572,7 +568,7 @@ __device__ __forceinline__ bool p1_slot(const Dev &d, const StepView &w, const P
             vw[s] = 0.0f;
             put_cell(d, Mn, base + (uint32_t)xh, 0);
         }
-        return true;
+        return;
     }
     xw[s] = xn;
     vw[s] = vn;
@@ -630,8 +626,7 @@ __device__ __forceinline__ bool p1_slot(const Dev &d, const StepView &w, const P
             atomicAdd(sk.n + 3, 1u);
         }
     }
-    return true;
-}
+    }
 
 // 16-byte words of the staged records into a global list (every thread)
 template <class T>
@@ -669,7 +664,13 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) step_p1(Dev d, uint32_t k
     }
     const StepView w = step_view(d, k, kph);
     const uint32_t norg = d.n_org;
-    const uint32_t lim = norg + d.cap;  // items: origin edges first, then slots
+    const uint32_t lim = norg + n;  // items: origin edges first, then slots
+    if (blockIdx.x * BLOCK >= lim) {
+        // Nothing for this block.  (Loading a slot before its number is known to be
+        // one saved a round trip and cost more: every idle thread's 80 bytes.)
+        span_end(d, 3 * koff);
+        return;
+    }
     __shared__ __align__(16) CrossRec s_cr[kStageCross];
     __shared__ __align__(16) IntendRec s_ir[kStageIntend];
     __shared__ __align__(16) DepRec s_dr[kStageDep];
@@ -684,7 +685,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) step_p1(Dev d, uint32_t k
             p1_origin(d, w, sk, i);
             continue;
         }
-        if (!p1_slot(d, w, sk, i - norg, n, live, arrived)) break;
+        p1_slot(d, w, sk, i - norg, live, arrived);
     }
     block_add<BLOCK>(&d.ctr[0], live, d.tacc ? &d.tacc[8] : nullptr);
     warp_add(&d.ctr[1], arrived);
@@ -805,6 +806,9 @@ __device__ __forceinline__ void p2_dep(const Dev &d, const StepView &w, const De
 // `late` (the intent aims at cell len - 1 and runs alongside the crossing
 // requests) a hold that a losing crosser of the target lane is placing in the
 // same kernel counts as occupying the target cell.
+// TOGETHER: both windows are loaded before either is searched (one round trip;
+// 20 registers more).
+template <bool TOGETHER>
 __device__ __forceinline__ void lane_change(const Dev &d, const StepView &w, const IntendRec &ir, uint32_t &changes,
                                           bool late) {
     const uint32_t k = w.k;
@@ -826,16 +830,20 @@ __device__ __forceinline__ void lane_change(const Dev &d, const StepView &w, con
     const uint32_t hi = c0 + 63u < len - 1 ? c0 + 63u : len - 1;
     // at most five chunks on either side of c0; without cells behind c0 the
     // window behind is cell 0 with nothing in it that counts
+    const uint32_t bhi = c0 > 0 ? c0 - 1 : 0u;
     uint32_t wa[20], wb[20];
+    Found fa, fb;
     load_ahead<5>(row2, c0, hi, wa);
-    load_behind<5>(row2, lo, c0 > 0 ? c0 - 1 : 0u, wb);
+    if (TOGETHER) load_behind<5>(row2, lo, bhi, wb);
+    fa = find_first<5>(wa, c0);
+    if (!TOGETHER) load_behind<5>(row2, lo, bhi, wb);
+    fb = find_last<5>(wb, bhi);
     const uint32_t tgt = base2 + cn;
     const uint8_t tgt_map = Mn[tgt], tgt_mark = Iw[tgt];
     const uint4 xr = late ? d.xreq[base2 >> 4] : make_uint4(kNone, 0u, 0u, 0u);
     uint64_t h = 0;
     if (m.eps_amp > 0.0f) h = splitmix64_mix(ir.hk ^ ((uint64_t)k * 0xD1B54A32D192ED03ull));
     // lead: first occupied cell in [c0, hi]; lag: last in [lo, c0 - 1]
-    const Found fa = find_first<5>(wa, c0), fb = find_last<5>(wb, c0 > 0 ? c0 - 1 : 0u);
     const uint32_t ca = fa.cell <= hi ? fa.cell : kNone;
     const uint32_t cb = c0 > 0 && fb.cell != kNone && fb.cell >= lo ? fb.cell : kNone;
     float eps_a = 0.0f, eps_b = 0.0f;
@@ -876,8 +884,15 @@ __device__ __forceinline__ void lane_change(const Dev &d, const StepView &w, con
 // next step's lists start empty, this step's departures have taken their
 // slots and its crossings their log entries (every other thread reads the
 // step's starting values from the snapshot step_p1 took).
+// 48 registers, so that five 256-thread blocks fit an SM and the whole grid
+// (half of step_p1's for each long list, and the rest) is resident at once; a
+// lane change searches its two windows one after the other for that.  Measured
+// with 62 registers / 48, and step_p1 leaving the blocks past the last slot at once:
+// 1,536 steps of 250k vehicles 44.6 / 42.6 ms, of 60k in 24 scenarios 19.4 / 18.1, 2,000
+// of 13k 24.2 / 22.8 (both windows together in 64 registers: 45.0, 19.9, 22.4; in 48 with
+// spills: 46.0, 19.9, 23.8).
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK) step_p2(Dev d, uint32_t koff, uint32_t kph, uint32_t gc, uint32_t gi) {
+__global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) step_p2(Dev d, uint32_t koff, uint32_t kph, uint32_t gc, uint32_t gi) {
     pdl_prologue();
     span_start(d, 3 * koff + 1);
     const uint32_t par = kph & 1u;
@@ -916,7 +931,7 @@ __global__ void __launch_bounds__(BLOCK) step_p2(Dev d, uint32_t koff, uint32_t 
             const IntendRec ir = list[i];
             loads_issued();
             if (i >= nint) break;
-            lane_change(d, w, ir, changes, false);
+            lane_change<false>(d, w, ir, changes, false);
         }
     } else if (blockIdx.x == gc + gi) {
         const uint32_t nlate = d.counts[6 + par];
@@ -925,7 +940,7 @@ __global__ void __launch_bounds__(BLOCK) step_p2(Dev d, uint32_t koff, uint32_t 
             const IntendRec ir = *(top - i);
             loads_issued();
             if (i >= nlate) break;
-            lane_change(d, w, ir, changes, true);
+            lane_change<false>(d, w, ir, changes, true);
         }
     } else {
         const uint32_t ndep = d.counts[4 + par];
@@ -959,8 +974,12 @@ __global__ void __launch_bounds__(BLOCK) step_p2(Dev d, uint32_t koff, uint32_t 
 // beyond a stage's room go through the global lists, from position 0), the
 // list lengths come from the stage counters, the slot count and the crossing
 // log position live in registers and the statistics counters are summed
-// over the whole chunk.  A step then costs three block barriers and no
-// global round trip of its own.  (Clusters of 2-8 such blocks, synchronised
+// over the whole chunk.  A step then costs two block barriers (three with a
+// stop-line intent) and no global round trip of its own.  What a phase does for
+// different kinds of items starts in different warps (slots and crossings in
+// the first, intents from the middle, origin edges and departures from the last
+// down), so that their chains run side by side instead of one after another in
+// the first warps.  (Clusters of 2-8 such blocks, synchronised
 // by cluster barriers, were measured slower than the grid-wide kernels for
 // 2k-12k trips.)
 // map_words > 0: the network's five lane maps (three rotating occupancy
@@ -988,10 +1007,10 @@ __global__ void __launch_bounds__(kSmallBlock, 1)
     __shared__ __align__(16) CrossRec s_cr[kStageCross];
     __shared__ __align__(16) IntendRec s_ir[kStageIntend];
     __shared__ __align__(16) DepRec s_dr[kStageDep];
-    __shared__ uint32_t s_n[4];
-    const P1Sinks sk{s_cr, s_ir, s_dr, s_n};
-    if (tid < 4) s_n[tid] = 0;
+    __shared__ uint32_t s_n[2][4];  // stage counters, by step parity
+    if (tid < 8) s_n[tid >> 2][tid & 3u] = 0;
     __syncthreads();
+    const uint32_t tid_mid = (tid - kSmallBlock * 3 / 8) % kSmallBlock, tid_down = kSmallBlock - 1 - tid;
     uint32_t live = 0, arrived = 0, events = 0, departed = 0, changes = 0;
     for (uint32_t t = 0; t < nsteps; t++) {
         const uint32_t k = k0 + t, par = k & 1u;
@@ -1008,22 +1027,25 @@ __global__ void __launch_bounds__(kSmallBlock, 1)
             w.Io = sm + (3u + (par ^ 1u)) * mb;
         }
         // P1
-        for (uint32_t i = tid; i < no; i += kSmallBlock) p1_origin(d, w, sk, olist[i]);
-        for (uint32_t s = tid; s < n; s += kSmallBlock) p1_slot(d, w, sk, s, n, live, arrived);
+        const P1Sinks sk{s_cr, s_ir, s_dr, s_n[par]};
+        for (uint32_t i = tid_down; i < no; i += kSmallBlock) p1_origin(d, w, sk, olist[i]);
+        for (uint32_t s = tid; s < n; s += kSmallBlock) p1_slot(d, w, sk, s, live, arrived);
         __syncthreads();
         // P2: staged items first, then the overflow in the global lists
-        const uint32_t ncross = s_n[0], nint = s_n[1], ndep = s_n[2], nlate = s_n[3];
+        const uint32_t ncross = s_n[par][0], nint = s_n[par][1], ndep = s_n[par][2], nlate = s_n[par][3];
+        if (tid < 4) s_n[par ^ 1u][tid] = 0;  // the next step's
         for (uint32_t i = tid; i < ncross; i += kSmallBlock)
             p2_cross(d, w, i < kStageCross ? s_cr[i] : d.cross_list[par][i - kStageCross], ev0 + i, events);
-        for (uint32_t i = tid; i < nint; i += kSmallBlock)
-            lane_change(d, w, i < kStageIntend ? s_ir[i] : d.intend_list[par][i - kStageIntend], changes, false);
-        for (uint32_t q = tid; q < ndep; q += kSmallBlock)
+        for (uint32_t i = tid_mid; i < nint; i += kSmallBlock)
+            lane_change<false>(d, w, i < kStageIntend ? s_ir[i] : d.intend_list[par][i - kStageIntend], changes, false);
+        for (uint32_t q = tid_down; q < ndep; q += kSmallBlock)
             p2_dep(d, w, q < kStageDep ? s_dr[q] : d.dep_rec[par][q - kStageDep], q, n, events, departed);
-        __syncthreads();
-        // P3 (every thread has read the stage counters: the next step's start here)
-        if (tid < 4) s_n[tid] = 0;
-        for (uint32_t i = tid; i < nlate; i += kSmallBlock)
-            lane_change(d, w, d.intend_list[par][d.cap - 1 - i], changes, false);
+        if (nlate) {
+            // P3: the intents at stop-line cells, after every hold
+            __syncthreads();
+            for (uint32_t i = tid; i < nlate; i += kSmallBlock)
+                lane_change<false>(d, w, d.intend_list[par][d.cap - 1 - i], changes, false);
+        }
         if (tid == 0) {  // the next step's global lists start empty
             d.counts[par ^ 1u] = 0;
             d.counts[2 + (par ^ 1u)] = 0;
