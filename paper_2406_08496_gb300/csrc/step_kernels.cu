@@ -82,17 +82,29 @@ __device__ __forceinline__ Found found_in(uint32_t word_cell, uint32_t w, uint32
     return {word_cell + byte, (~w >> (8u * byte)) & 0xFFu};
 }
 
-// the complements of chunks c_first, c_first + step, ... (N of them, loaded
-// together: one memory round trip), zero where `in` says the window has ended
-template <int N, class In>
-__device__ __forceinline__ void load_cells(const uint8_t *row, uint32_t c_first, int step, In in,
-                                           uint32_t (&w)[4 * N]) {
-    uint4 q[N];
+// chunks of [lo, hi] from lo's on, as they are (N of them, loaded together: one
+// memory round trip; empty where the window has ended)
+template <int N>
+__device__ __forceinline__ void load_ahead(const uint8_t *row, uint32_t lo, uint32_t hi, uint4 (&q)[N]) {
 #pragma unroll
     for (int j = 0; j < N; j++) {
-        const uint32_t c = c_first + (uint32_t)(step * j);
-        q[j] = in(c, j) ? *reinterpret_cast<const uint4 *>(row + c) : make_uint4(~0u, ~0u, ~0u, ~0u);
+        const uint32_t c = (lo & ~15u) + 16u * j;
+        q[j] = c <= hi ? *reinterpret_cast<const uint4 *>(row + c) : make_uint4(~0u, ~0u, ~0u, ~0u);
     }
+}
+
+// chunks of [lo, hi] from hi's down
+template <int N>
+__device__ __forceinline__ void load_behind(const uint8_t *row, uint32_t lo, uint32_t hi, uint4 (&q)[N]) {
+    const uint32_t n = (hi >> 4) - (lo >> 4);  // chunks of the window after the first
+#pragma unroll
+    for (int j = 0; j < N; j++)
+        q[j] = (uint32_t)j <= n ? *reinterpret_cast<const uint4 *>(row + ((hi & ~15u) - 16u * j))
+                                : make_uint4(~0u, ~0u, ~0u, ~0u);
+}
+
+template <int N>
+__device__ __forceinline__ void complements(const uint4 (&q)[N], uint32_t (&w)[4 * N]) {
 #pragma unroll
     for (int j = 0; j < N; j++) {
         w[4 * j] = ~q[j].x;
@@ -102,17 +114,13 @@ __device__ __forceinline__ void load_cells(const uint8_t *row, uint32_t c_first,
     }
 }
 
-// chunks of [lo, hi] from lo's on, the cells before lo dropped
-template <int N>
-__device__ __forceinline__ void load_ahead(const uint8_t *row, uint32_t lo, uint32_t hi, uint32_t (&w)[4 * N]) {
-    load_cells<N>(row, lo & ~15u, 16, [hi](uint32_t c, int) { return c <= hi; }, w);
-#pragma unroll
-    for (int j = 0; j < 4; j++) w[j] &= __funnelshift_lc(0u, ~0u, max((int)(8u * (lo & 15u)) - 32 * j, 0));
-}
-
 // first occupied cell at or after lo in the loaded chunks
 template <int N>
-__device__ __forceinline__ Found find_first(const uint32_t (&w)[4 * N], uint32_t lo) {
+__device__ __forceinline__ Found find_first(const uint4 (&q)[N], uint32_t lo) {
+    uint32_t w[4 * N];
+    complements(q, w);
+#pragma unroll
+    for (int j = 0; j < 4; j++) w[j] &= __funnelshift_lc(0u, ~0u, max((int)(8u * (lo & 15u)) - 32 * j, 0));
     uint32_t t = 0, at = 0;
 #pragma unroll
     for (int j = 4 * N - 1; j >= 0; j--)
@@ -123,18 +131,13 @@ __device__ __forceinline__ Found find_first(const uint32_t (&w)[4 * N], uint32_t
     return t ? found_in((lo & ~15u) + at, t, (uint32_t)(__ffs((int)t) - 1) >> 3) : Found{kNone, 0u};
 }
 
-// chunks of [lo, hi] from hi's down, the cells after hi dropped
-template <int N>
-__device__ __forceinline__ void load_behind(const uint8_t *row, uint32_t lo, uint32_t hi, uint32_t (&w)[4 * N]) {
-    const uint32_t n = (hi >> 4) - (lo >> 4);  // chunks of the window after the first
-    load_cells<N>(row, hi & ~15u, -16, [n](uint32_t, int j) { return (uint32_t)j <= n; }, w);
-#pragma unroll
-    for (int j = 0; j < 4; j++) w[j] &= __funnelshift_rc(~0u, 0u, max(32 * (j + 1) - 8 * (int)((hi & 15u) + 1u), 0));
-}
-
 // last occupied cell at or before hi in the loaded chunks
 template <int N>
-__device__ __forceinline__ Found find_last(const uint32_t (&w)[4 * N], uint32_t hi) {
+__device__ __forceinline__ Found find_last(const uint4 (&q)[N], uint32_t hi) {
+    uint32_t w[4 * N];
+    complements(q, w);
+#pragma unroll
+    for (int j = 0; j < 4; j++) w[j] &= __funnelshift_rc(~0u, 0u, max(32 * (j + 1) - 8 * (int)((hi & 15u) + 1u), 0));
     uint32_t t = 0, at = 0;
 #pragma unroll
     for (int j = N - 1; j >= 0; j--)
@@ -147,16 +150,12 @@ __device__ __forceinline__ Found find_last(const uint32_t (&w)[4 * N], uint32_t 
     return t ? found_in((hi & ~15u) - at, t, (uint32_t)(31 - __clz((int)t)) >> 3) : Found{kNone, 0u};
 }
 
-// first occupied cell in [lo, hi]; the first four 16-byte chunks of
-// the window are loaded together, so a window of up to 49 cells costs one
-// memory round trip
-__device__ __forceinline__ Found first_occupied_wide(const uint8_t *row, uint32_t lo, uint32_t hi) {
-    if (lo > hi) return {kNone, 0u};
-    uint32_t w[16];
-    load_ahead<4>(row, lo, hi, w);
-    Found f = find_first<4>(w, lo);
+// first occupied cell in [lo, hi], lo <= hi, with the window's first four chunks
+// loaded before (load_ahead): up to 49 cells in that round trip
+__device__ __forceinline__ Found first_occupied(const uint8_t *row, const uint4 (&q)[4], uint32_t lo, uint32_t hi) {
+    Found f = find_first<4>(q, lo);
     for (uint32_t c = (lo & ~15u) + 64u; f.cell == kNone && c <= hi; c += 16u) {
-        uint32_t u[4];
+        uint4 u[1];
         load_ahead<1>(row, c, hi, u);
         f = find_first<1>(u, c);
     }
@@ -259,22 +258,6 @@ __device__ __forceinline__ void stage_put(T *buf, uint32_t room, uint32_t *n, T 
 // Keeps the loads above it above a following branch (so the first records of
 // a thread are in flight while the list length is still on its way).
 __device__ __forceinline__ void loads_issued() { asm volatile("" ::: "memory"); }
-
-template <int BLOCK>
-__device__ __forceinline__ void block_add(unsigned long long *dst, uint32_t val, unsigned long long *dst2 = nullptr) {
-    __shared__ uint32_t red[BLOCK / 32];
-    uint32_t w = __reduce_add_sync(0xFFFFFFFFu, val);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = w;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        uint32_t t = threadIdx.x < BLOCK / 32 ? red[threadIdx.x] : 0u;
-        t = __reduce_add_sync(0xFFFFFFFFu, t);
-        if (threadIdx.x == 0 && t) {
-            atomicAdd(dst, (unsigned long long)t);
-            if (dst2) atomicAdd(dst2, (unsigned long long)t);
-        }
-    }
-}
 
 // A statistics counter summed over a full warp, then one atomic per warp:
 // per-thread atomics on one address serialise in L2 (one per crossing
@@ -473,9 +456,14 @@ __device__ __forceinline__ void p1_slot(const Dev &d, const StepView &w, const P
     const bool green = may_end && en != kNone && (G == 0 || (k / G) % (ph & 0xFFu) == (ph >> 8));
     const bool may_cross = green;
     const bool may_draw = tl != kNoLane && tl != ln && ((tl > ln) == (par == 1u)) && (L - x) < m.x0;
+    uint32_t hi = c + (uint32_t)fminf(reach, 65535.0f) + 2u;
+    if (hi > len - 1) hi = len - 1;
+    uint4 window[4];
+    load_ahead<4>(Mc + base, c + 1, hi, window);
     float nv0 = 0.0f;
     RouteRec rr{};
-    uint32_t nen = kNone, e = kNone, tent = 0, empty = 0, so = 0;
+    uint32_t nen = kNone, e = kNone, tent = 0, so = 0;
+    uint32_t entry[4] = {0u, 0u, 0u, 0u};  // cell 0 of the next edge's lanes (0: none, or not to be entered)
     if (may_cross || (may_end && en == kNone)) {
         // the current edge and its entry step (for the statistics of a
         // crossing or an arrival)
@@ -491,7 +479,7 @@ __device__ __forceinline__ void p1_slot(const Dev &d, const StepView &w, const P
         const uint32_t stride = row_stride(es.nlen);
 #pragma unroll
         for (uint32_t l = 0; l < 4; l++)
-            if (l < es.nlanes && Mc[es.nmoff + l * stride] == kEmpty) empty |= 1u << l;
+            if (l < es.nlanes) entry[l] = Mc[es.nmoff + l * stride];
     }
     // lane-change draw at step k: SplitMix64 of hkey ^ k * C2, where
     // hkey[id] = seed ^ local_id * C1 was formed at load time (local_id =
@@ -500,9 +488,7 @@ __device__ __forceinline__ void p1_slot(const Dev &d, const StepView &w, const P
     const uint64_t hk = !may_draw ? 0ull
                         : d.hkey_from_id ? d.m.seed ^ ((uint64_t)id * 0x9E3779B97F4A7C15ull)
                                          : d.hkey[id];
-    uint32_t hi = c + (uint32_t)fminf(reach, 65535.0f) + 2u;
-    if (hi > len - 1) hi = len - 1;
-    const Found lead = first_occupied_wide(Mc + base, c + 1, hi);
+    const Found lead = c < hi ? first_occupied(Mc + base, window, c + 1, hi) : Found{kNone, 0u};
     const uint32_t cf = lead.cell;
     const bool has_f = cf != kNone;
 
@@ -532,6 +518,9 @@ __device__ __forceinline__ void p1_slot(const Dev &d, const StepView &w, const P
         bool cross = false;
         if (green) {
             // may_cross holds here: x' >= L needs x + vmax_step * dt >= L
+            uint32_t empty = 0;
+#pragma unroll
+            for (uint32_t q = 0; q < 4; q++) empty |= (entry[q] == kEmpty ? 1u : 0u) << q;
             const uint32_t l = pick_entry_lane(empty, es.nlanes, rr.tl);
             if (l != kNone) {
                 const uint32_t slot = so + l;
@@ -596,7 +585,10 @@ __device__ __forceinline__ void p1_slot(const Dev &d, const StepView &w, const P
         if (up ? ln + 1 < nl : ln > 0) {
             const uint32_t stride = row_stride(len);
             const uint32_t base2 = up ? base + stride : base - stride;
-            const uint32_t ca = first_occupied_wide(Mc + base2, c, min(c + 63u, len - 1)).cell;
+            const uint32_t hi2 = min(c + 63u, len - 1);
+            uint4 beside[4];
+            load_ahead<4>(Mc + base2, c, hi2, beside);
+            const uint32_t ca = first_occupied(Mc + base2, beside, c, hi2).cell;
             if (ca == kNone || (float)ca - (float)cf >= m.dlc_gain) {
                 hkd = d.hkey_from_id ? d.m.seed ^ ((uint64_t)id * 0x9E3779B97F4A7C15ull) : d.hkey[id];
                 intend = unit24(splitmix64_mix(hkd ^ ((uint64_t)k * 0xD1B54A32D192ED03ull))) < m.dlc_prob;
@@ -674,8 +666,9 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) step_p1(Dev d, uint32_t k
     __shared__ __align__(16) CrossRec s_cr[kStageCross];
     __shared__ __align__(16) IntendRec s_ir[kStageIntend];
     __shared__ __align__(16) DepRec s_dr[kStageDep];
-    __shared__ uint32_t s_n[4], s_base[3];
+    __shared__ uint32_t s_n[4], s_base[3], s_live;
     if (threadIdx.x < 4) s_n[threadIdx.x] = 0;
+    if (threadIdx.x == 4) s_live = 0;
     __syncthreads();
     const P1Sinks sk{s_cr, s_ir, s_dr, s_n};
     uint32_t live = 0;
@@ -687,8 +680,16 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) step_p1(Dev d, uint32_t k
         }
         p1_slot(d, w, sk, i - norg, live, arrived);
     }
-    block_add<BLOCK>(&d.ctr[0], live, d.tacc ? &d.tacc[8] : nullptr);
+    {
+        const uint32_t wl = __reduce_add_sync(0xFFFFFFFFu, live);
+        if ((threadIdx.x & 31u) == 0 && wl) atomicAdd(&s_live, wl);
+    }
     warp_add(&d.ctr[1], arrived);
+    __syncthreads();
+    if (threadIdx.x == 32 && s_live) {
+        atomicAdd(&d.ctr[0], (unsigned long long)s_live);
+        if (d.tacc) atomicAdd(&d.tacc[8], (unsigned long long)s_live);
+    }
     p1_flush(d, w.par, sk, s_base);
     span_end(d, 3 * koff);
 }
@@ -831,13 +832,15 @@ __device__ __forceinline__ void lane_change(const Dev &d, const StepView &w, con
     // at most five chunks on either side of c0; without cells behind c0 the
     // window behind is cell 0 with nothing in it that counts
     const uint32_t bhi = c0 > 0 ? c0 - 1 : 0u;
-    uint32_t wa[20], wb[20];
     Found fa, fb;
-    load_ahead<5>(row2, c0, hi, wa);
-    if (TOGETHER) load_behind<5>(row2, lo, bhi, wb);
-    fa = find_first<5>(wa, c0);
-    if (!TOGETHER) load_behind<5>(row2, lo, bhi, wb);
-    fb = find_last<5>(wb, bhi);
+    {
+        uint4 qa[5], qb[5];
+        load_ahead<5>(row2, c0, hi, qa);
+        if (TOGETHER) load_behind<5>(row2, lo, bhi, qb);
+        fa = find_first<5>(qa, c0);
+        if (!TOGETHER) load_behind<5>(row2, lo, bhi, qb);
+        fb = find_last<5>(qb, bhi);
+    }
     const uint32_t tgt = base2 + cn;
     const uint8_t tgt_map = Mn[tgt], tgt_mark = Iw[tgt];
     const uint4 xr = late ? d.xreq[base2 >> 4] : make_uint4(kNone, 0u, 0u, 0u);
