@@ -792,14 +792,16 @@ __device__ __forceinline__ void gelu_grad_pair(float acc0, float acc1, float b0,
     float s0, s1, d0, d1, p0, p1;
     f2_unpack(f2_mul(z, q), s0, s1);
     f2_unpack(f2_add(f2_pack(1.0f, 1.0f), f2_pack(ex2_fast(s0), ex2_fast(s1))), d0, d1);
-    const f32x2_t cdf = f2_pack(rcp_fast(d0), rcp_fast(d1));
-    f2_unpack(f2_mul(z, cdf), h0, h1);
+    const float c0 = rcp_fast(d0), c1 = rcp_fast(d1);
+    f2_unpack(f2_mul(z, f2_pack(c0, c1)), h0, h1);
     f2_unpack(f2_mul(f2_pack(-0.7213475204f, -0.7213475204f), z2), p0, p1);
     const f32x2_t pdf = f2_mul(f2_pack(0.3989422804f, 0.3989422804f), f2_pack(ex2_fast(p0), ex2_fast(p1)));
-    float u0, u1;
-    f2_unpack(f2_add(cdf, f2_mul(z, pdf)), u0, u1);
-    g0 = __float_as_uint(u0);
-    g1 = __float_as_uint(u1);
+    float z0, z1, u0, u1;
+    f2_unpack(z, z0, z1);
+    f2_unpack(pdf, u0, u1);
+    // scalar: a paired product and sum come out as one rounding
+    g0 = __float_as_uint(__fadd_rn(c0, __fmul_rn(z0, u0)));
+    g1 = __float_as_uint(__fadd_rn(c1, __fmul_rn(z1, u1)));
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrThreads, 1)
@@ -1186,8 +1188,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrThreads, 1)
 // [64 rows][64 columns] box in the 128-byte swizzle is an MN-major operand
 // whose K index is the row, so no transposed copies exist.  One CTA per
 // 128 x 128 output tile (128 x 64 for layer 1: ten tiles in all) and split of
-// the rows; partial sums go to global memory in the accumulator's own order
-// (whole 512-byte lines per warp) and are added by mlp_update.
+// the rows.  A split's even and odd 64-row slices go to an accumulator each,
+// added at the end: half as many sums in the tensor core's own rounding (dW of
+// 20,000 rows 1.5e-7 off the sums of 128-row blocks instead of 4.4e-7).  Partial
+// sums go to global memory in the accumulator's own order (whole 512-byte lines
+// per warp) and are added by mlp_update.
 
 constexpr int kWgStages = 3;
 constexpr uint32_t kWgBox = 64 * kBK * 2;  // 64 rows x 64 columns: 8 KB
@@ -1238,7 +1243,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(128));
+                     "r"(256));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1278,8 +1283,8 @@ __global__ void __launch_bounds__(kThreads, 2)
             const uint32_t a0 = smem_u32(smem + s * 4 * kWgBox), b0 = a0 + 2 * kWgBox;
 #pragma unroll
             for (int kk = 0; kk < 4; kk++)  // 16 rows per instruction: two 8-row groups
-                umma_f16(tmem, umma_desc_mn(a0 + kk * 2048, kWgBox), umma_desc_mn(b0 + kk * 2048, kWgBox), idesc,
-                         (i | kk) != 0);
+                umma_f16(tmem + (uint32_t)(i & 1) * 128u, umma_desc_mn(a0 + kk * 2048, kWgBox),
+                         umma_desc_mn(b0 + kk * 2048, kWgBox), idesc, i >= 2 || kk > 0);
             umma_commit(&empty[s]);
         }
         umma_commit(done);
@@ -1297,6 +1302,12 @@ __global__ void __launch_bounds__(kThreads, 2)
             const int cb = ch * nb + c;  // 32-column block
             uint32_t r[32];
             tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cb * 32), r);
+            if (nk > 1) {
+                uint32_t r2[32];
+                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(128 + cb * 32), r2);
+#pragma unroll
+                for (int i = 0; i < 32; i++) r[i] = __float_as_uint(__uint_as_float(r[i]) + __uint_as_float(r2[i]));
+            }
 #pragma unroll
             for (int i = 0; i < 8; i++)
                 out[((cb * 4 + q) * 8 + i) * 32 + lane] =
@@ -1306,7 +1317,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256));
 }
 
 // ------------------------------------------------------------------- update
