@@ -17,6 +17,8 @@ int lpsim_fail(int code, const std::string &msg);
 // error word and the slot count, so that one copy brings a status to the host
 constexpr int kCtrErr = 16, kCtrSlots = 17, kCtrWords = 18;
 
+constexpr uint64_t kStateKept = 1u << 20;  // device bytes a context keeps for lpsim_get_state
+
 struct lpsim_ctx {
     int device = 0;
     int n_sm = 0;
@@ -47,6 +49,9 @@ struct lpsim_ctx {
     int grid = 0, block = 256;
     bool sort = true;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
+    bool ctr_current = false;             // h_ctr holds the counters as they are
+    uint8_t *state_dev = nullptr;         // lpsim_get_state: device block of a small demand, host block
+    std::vector<uint8_t> state_host;
     unsigned long long *h_ctr = nullptr;  // pinned: kCtrWords words of ctr
     uint32_t *d_tmp = nullptr;
     lpsim::QRec *org_hd0 = nullptr;  // first trip of each origin queue (reset)

@@ -318,7 +318,9 @@ uint32_t compact_tile();
 void launch_route_records(const Dev &d, uint64_t n_trips, RouteRec *out, cudaStream_t st);
 void launch_transpose_bins(const uint32_t *in, uint32_t n_edges, uint32_t n_bins, uint32_t *out, cudaStream_t st);
 
-// helpers for the query functions
+// helpers for the query functions: every vehicle as one not on the network, with its status, then those on it
+void launch_state_clear(const Dev &d, uint64_t n, float *x, float *v, uint32_t *edge, uint8_t *lane, uint32_t *ridx,
+                        uint8_t *status, cudaStream_t st);
 void launch_state_scatter(const Dev &d, uint32_t k, float *x, float *v, uint32_t *edge, uint8_t *lane,
                           uint32_t *ridx, cudaStream_t st);
 void launch_max_arrival(const Dev &d, uint64_t n, uint32_t *out, cudaStream_t st);

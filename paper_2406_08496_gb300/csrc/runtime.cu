@@ -69,7 +69,7 @@ int dnew(lpsim_ctx *c, T *&out, size_t count) {
 struct Scratch {
     lpsim_ctx *c;
     void *p;
-    Scratch(lpsim_ctx *ctx, size_t bytes) : c(ctx), p(ctx->dalloc(bytes)) {}
+    Scratch(lpsim_ctx *ctx, size_t bytes) : c(ctx), p(bytes ? ctx->dalloc(bytes) : nullptr) {}
     Scratch(const Scratch &) = delete;
     Scratch &operator=(const Scratch &) = delete;
     ~Scratch() {
@@ -129,49 +129,111 @@ int alloc_slots(lpsim_ctx *c, Slots &s, uint32_t cap) {
     return LPSIM_OK;
 }
 
+// Many device buffers filled or copied in one launch: a reset fills two dozen,
+// a snapshot or a restore copies fifty-odd, most of them small, and a call each
+// costs the host 2 us and the stream its own launch.  The buffers are cut into
+// pieces of kSegPiece bytes, one block per piece at a time; they start on
+// 16-byte boundaries (as the records in them need), a last part below 16 bytes
+// goes by bytes.
+constexpr uint32_t kMaxSegs = 64;
+constexpr uint32_t kSegPiece = 32768;
+struct Seg {
+    void *dst;
+    const void *src;  // nullptr: fill with the byte `fill`
+    uint64_t bytes;
+    uint32_t fill, first;  // first piece of the buffer
+};
+struct Segs {
+    Seg s[kMaxSegs];
+    uint32_t n, pieces;
+};
+
+__global__ void __launch_bounds__(256) move_segments(const __grid_constant__ Segs g) {
+    uint32_t q = 0;
+    for (uint32_t p = blockIdx.x; p < g.pieces; p += gridDim.x) {
+        while (q + 1 < g.n && g.s[q + 1].first <= p) q++;
+        const Seg &x = g.s[q];
+        const uint64_t o = (uint64_t)(p - x.first) * kSegPiece;
+        const uint32_t len = (uint32_t)min((uint64_t)kSegPiece, x.bytes - o);
+        uint8_t *dst = static_cast<uint8_t *>(x.dst) + o;
+        const uint8_t *src = static_cast<const uint8_t *>(x.src) + o;
+        const uint32_t f = x.fill * 0x01010101u;
+#pragma unroll 4
+        for (uint32_t i = threadIdx.x; i < len / 16; i += 256)
+            reinterpret_cast<uint4 *>(dst)[i] = x.src ? reinterpret_cast<const uint4 *>(src)[i] : make_uint4(f, f, f, f);
+        const uint32_t t = (len & ~15u) + threadIdx.x;
+        if (t < len) dst[t] = x.src ? src[t] : (uint8_t)x.fill;
+    }
+}
+
+struct SegList {
+    lpsim_ctx *c;
+    Segs g{};
+    explicit SegList(lpsim_ctx *ctx) : c(ctx) {}
+    int add(void *dst, const void *src, uint64_t bytes, uint8_t fill) {
+        if (bytes == 0) return LPSIM_OK;
+        if (g.n == kMaxSegs) TRY(run());
+        g.s[g.n++] = Seg{dst, src, bytes, fill, g.pieces};
+        g.pieces += (uint32_t)((bytes + kSegPiece - 1) / kSegPiece);
+        return LPSIM_OK;
+    }
+    int fill(void *dst, uint8_t v, uint64_t bytes) { return add(dst, nullptr, bytes, v); }
+    int run() {
+        if (g.n == 0) return LPSIM_OK;
+        move_segments<<<std::min<uint32_t>(g.pieces, (uint32_t)c->n_sm * 8u), 256, 0, c->stream>>>(g);
+        CU(cudaGetLastError());
+        g.n = g.pieces = 0;
+        return LPSIM_OK;
+    }
+};
+
 // empty maps, waiting trips, cleared statistics, step 0
 int reset_state(lpsim_ctx *c) {
     Dev &d = c->d;
-    cudaStream_t st = c->stream;
-    for (int i = 0; i < 3; i++) CU(cudaMemsetAsync(d.map[i], 0xFF, c->map_bytes, st));
-    for (int i = 0; i < 2; i++) CU(cudaMemsetAsync(d.imap[i], 0, c->map_bytes, st));
-    CU(cudaMemsetAsync(d.xreq, 0xFF, c->map_bytes, st));  // no request at any step
-    for (int i = 0; i < 2; i++) CU(cudaMemsetAsync(d.claim[i], 0xFF, c->lane_slots * 4, st));
-    CU(cudaMemsetAsync(d.ent, 0, c->n_edges * 8ull, st));
-    CU(cudaMemsetAsync(d.ext, 0, c->n_edges * 8ull, st));
-    CU(cudaMemsetAsync(d.tts, 0, c->n_edges * 8ull, st));
-    size_t nb = (size_t)c->n_edges * c->p.n_bins * 4;
-    if (nb) {
-        CU(cudaMemsetAsync(d.bin_in, 0, nb, st));
-        CU(cudaMemsetAsync(d.bin_tt, 0, nb, st));
-        CU(cudaMemsetAsync(d.bin_cnt, 0, nb, st));
-        CU(cudaMemsetAsync(d.bin_occ, 0, nb, st));
-    }
-    CU(cudaMemsetAsync(d.counts, 0, 8 * 4, st));
-    CU(cudaMemsetAsync(d.kbase, 0, 4, st));
-    CU(cudaMemsetAsync(d.ev_n, 0, 4, st));
-    CU(cudaMemsetAsync(d.ctr, 0, kCtrWords * 8, st));  // with the error word and the slot count
+    SegList z(c);
+    for (int i = 0; i < 3; i++) TRY(z.fill(d.map[i], 0xFF, c->map_bytes));
+    for (int i = 0; i < 2; i++) TRY(z.fill(d.imap[i], 0, c->map_bytes));
+    TRY(z.fill(d.xreq, 0xFF, c->map_bytes / 16 * 16));  // no request at any step
+    for (int i = 0; i < 2; i++) TRY(z.fill(d.claim[i], 0xFF, c->lane_slots * 4));
+    TRY(z.fill(d.ent, 0, c->n_edges * 8ull));
+    TRY(z.fill(d.ext, 0, c->n_edges * 8ull));
+    TRY(z.fill(d.tts, 0, c->n_edges * 8ull));
+    const size_t nb = (size_t)c->n_edges * c->p.n_bins * 4;
+    TRY(z.fill(d.bin_in, 0, nb));
+    TRY(z.fill(d.bin_tt, 0, nb));
+    TRY(z.fill(d.bin_cnt, 0, nb));
+    TRY(z.fill(d.bin_occ, 0, nb));
+    TRY(z.fill(d.counts, 0, 8 * 4));
+    TRY(z.fill(d.kbase, 0, 4));
+    TRY(z.fill(d.ev_n, 0, 4));
+    TRY(z.fill(d.ctr, 0, kCtrWords * 8));  // with the error word and the slot count
     if (c->loaded) {
-        CU(cudaMemsetAsync(d.dep_act, 0xFF, c->n_trips * 4, st));
-        CU(cudaMemsetAsync(d.arr, 0xFF, c->n_trips * 4, st));
-        CU(cudaMemsetAsync(d.status, 0, c->n_trips, st));
-        CU(cudaMemsetAsync(d.org_head, 0, (size_t)d.n_org * 4, st));
-        CU(cudaMemsetAsync(d.dprev, 0xFF, (size_t)d.n_org * 4, st));
-        CU(cudaMemcpyAsync(d.org_hd, c->org_hd0, (size_t)d.n_org * sizeof(QRec), cudaMemcpyDeviceToDevice, st));
+        TRY(z.fill(d.dep_act, 0xFF, c->n_trips * 4));
+        TRY(z.fill(d.arr, 0xFF, c->n_trips * 4));
+        TRY(z.fill(d.status, 0, c->n_trips));
+        TRY(z.fill(d.org_head, 0, (size_t)d.n_org * 4));
+        TRY(z.fill(d.dprev, 0xFF, (size_t)d.n_org * 4));
+        TRY(z.add(d.org_hd, c->org_hd0, (size_t)d.n_org * sizeof(QRec), 0));
     }
+    TRY(z.run());
     c->k = 0;
     c->cur = 0;
     c->d.s = c->sets[0];
     c->stall_steps = 0;
     c->last_progress = 0;
-    CU(cudaStreamSynchronize(st));
+    CU(cudaStreamSynchronize(c->stream));
+    std::memset(c->h_ctr, 0, kCtrWords * 8);
+    c->ctr_current = true;
     return LPSIM_OK;
 }
 
 int read_status(lpsim_ctx *c) {
     // h_ctr: [0..7] counters, [kCtrErr] err, [kCtrSlots] n_slots
-    CU(cudaMemcpyAsync(c->h_ctr, c->d.ctr, kCtrWords * 8, cudaMemcpyDeviceToHost, c->stream));
-    CU(cudaStreamSynchronize(c->stream));
+    if (!c->ctr_current) {
+        CU(cudaMemcpyAsync(c->h_ctr, c->d.ctr, kCtrWords * 8, cudaMemcpyDeviceToHost, c->stream));
+        CU(cudaStreamSynchronize(c->stream));
+        c->ctr_current = true;
+    }
     uint32_t err = (uint32_t)(c->h_ctr[kCtrErr] & 0xFFFFFFFFull);
     if (err & kErrCellTaken) return fail(LPSIM_E_INVARIANT, "two vehicles were written to one lane-map cell");
     if (err & kErrSlotOverflow) return fail(LPSIM_E_INVARIANT, "vehicle slot capacity exceeded");
@@ -199,6 +261,7 @@ int enqueue_step(lpsim_ctx *c, uint32_t koff, uint32_t kph, int cur, bool compac
 // two more launches a step: 2,000 steps of a 13k-vehicle town, 464 of them
 // direct, 27.2 ms, now 24.8 ms.)
 int direct_steps(lpsim_ctx *c, uint32_t steps) {
+    c->ctr_current = false;
     for (uint32_t j = 0; j < steps; j++) {
         const bool compact = (c->k + j + 1) % c->R == 0;
         c->cur = enqueue_step(c, j, (uint32_t)((c->k + j) % 6), c->cur, compact);
@@ -241,6 +304,7 @@ uint64_t chunk_launches(const lpsim_ctx *c) {
 
 int chunk(lpsim_ctx *c) {
     if (c->C % 6 != 0 || c->k % c->C != 0) return fail(LPSIM_E_STATE, "graph chunk not aligned to a multiple of 6 steps");
+    c->ctr_current = false;
     if (!c->graph[c->cur]) TRY(capture_chunk(c, c->cur));
     CU(cudaGraphLaunch(c->graph[c->cur], c->stream));
     c->launches += chunk_launches(c);
@@ -264,6 +328,7 @@ bool light_ok(const lpsim_ctx *c, uint32_t steps) {
 // never more than a chunk's departures between two) and the step-counter
 // update.
 int light_steps(lpsim_ctx *c, uint32_t steps) {
+    c->ctr_current = false;
     Dev d = c->d;
     d.s = c->sets[c->cur];
     // with LPSIM_F_SHARED_MAPS the lane maps of a small network ride in the
@@ -1013,10 +1078,12 @@ int snapshot_impl(lpsim_ctx *c) {
     }
     if (total != c->snap_bytes) return fail(LPSIM_E_STATE, "state layout changed since the first snapshot");
     size_t o = 0;
+    SegList z(c);
     for (auto &b : c->mut) {
-        CU(cudaMemcpyAsync(c->snap + o, b.first, b.second, cudaMemcpyDeviceToDevice, c->stream));
+        TRY(z.add(c->snap + o, b.first, b.second, 0));
         o += (b.second + 255) & ~size_t(255);
     }
+    TRY(z.run());
     CU(cudaStreamSynchronize(c->stream));
     c->snap_host = {c->k, c->cur, c->stall_steps, c->last_progress};
     c->has_snap = true;
@@ -1025,12 +1092,14 @@ int snapshot_impl(lpsim_ctx *c) {
 
 int restore_impl(lpsim_ctx *c) {
     if (!c->has_snap) return fail(LPSIM_E_STATE, "no snapshot taken");
-    CU(cudaStreamSynchronize(c->stream));
+    c->ctr_current = false;
     size_t o = 0;
+    SegList z(c);
     for (auto &b : c->mut) {
-        CU(cudaMemcpyAsync(b.first, c->snap + o, b.second, cudaMemcpyDeviceToDevice, c->stream));
+        TRY(z.add(b.first, c->snap + o, b.second, 0));
         o += (b.second + 255) & ~size_t(255);
     }
+    TRY(z.run());
     CU(cudaStreamSynchronize(c->stream));
     c->k = c->snap_host.k;
     c->cur = c->snap_host.cur;
@@ -1199,29 +1268,44 @@ int lpsim_get_state(lpsim_ctx *c, uint64_t n, float *x, float *v, uint32_t *edge
     if (!c) return fail(LPSIM_E_INVALID_ARG, "ctx is NULL");
     if (!c->loaded) return fail(LPSIM_E_STATE, "lpsim_load_demand has not been called");
     if (n != c->n_trips) return fail(LPSIM_E_INVALID_ARG, "n does not match the trips loaded");
-    // scratch: x, v, edge, ridx (4 B each) and lane (1 B) per vehicle; given
-    // back on every exit path (after the stream has finished with it)
-    Scratch scratch(c, n * 17 + 64);
-    if (!scratch.p) return fail(LPSIM_E_OOM, "device scratch allocation failed");
-    uint8_t *tmp = static_cast<uint8_t *>(scratch.p);
+    // x, v, edge, ridx (4 B each), lane and status (1 B) per vehicle, gathered on
+    // the device in one block.  A small demand's comes over in one copy and is
+    // shared out on the host (a copy costs 8 us however small: six took 48); both
+    // blocks are kept.  A larger one's goes straight to the caller's arrays, and its
+    // device block is given back on every exit path (after the stream has finished
+    // with it); through a host block 250k vehicles took 1.1 ms instead of 0.17.
+    const uint64_t bytes = n * 18;
+    if (n == 0) return LPSIM_OK;
+    Scratch scratch(c, bytes > kStateKept ? bytes : 0);
+    if (bytes <= kStateKept && !c->state_dev) TRY(dnew(c, c->state_dev, kStateKept));
+    uint8_t *tmp = bytes > kStateKept ? static_cast<uint8_t *>(scratch.p) : c->state_dev;
+    if (!tmp) return fail(LPSIM_E_OOM, "device scratch allocation failed");
     float *dx = reinterpret_cast<float *>(tmp);
     float *dv = dx + n;
     uint32_t *de = reinterpret_cast<uint32_t *>(dv + n);
     uint32_t *dr = de + n;
     uint8_t *dl = reinterpret_cast<uint8_t *>(dr + n);
-    CU(cudaMemsetAsync(tmp, 0, n * 17, c->stream));
-    CU(cudaMemsetAsync(de, 0xFF, n * 4, c->stream));
     Dev d = c->d;
     d.s = c->sets[c->cur];
+    launch_state_clear(d, n, dx, dv, de, dl, dr, dl + n, c->stream);
     launch_state_scatter(d, c->k, dx, dv, de, dl, dr, c->stream);
     CU(cudaGetLastError());
-    CU(cudaStreamSynchronize(c->stream));
-    if (x) CU(cudaMemcpy(x, dx, n * 4, cudaMemcpyDeviceToHost));
-    if (v) CU(cudaMemcpy(v, dv, n * 4, cudaMemcpyDeviceToHost));
-    if (edge) CU(cudaMemcpy(edge, de, n * 4, cudaMemcpyDeviceToHost));
-    if (ridx) CU(cudaMemcpy(ridx, dr, n * 4, cudaMemcpyDeviceToHost));
-    if (lane) CU(cudaMemcpy(lane, dl, n, cudaMemcpyDeviceToHost));
-    if (status) CU(cudaMemcpy(status, c->d.status, n, cudaMemcpyDeviceToHost));
+    struct {
+        void *to;
+        uint64_t from, bytes;
+    } outs[] = {{x, 0, n * 4},         {v, n * 4, n * 4},   {edge, n * 8, n * 4},
+                {ridx, n * 12, n * 4}, {lane, n * 16, n},   {status, n * 17, n}};
+    if (bytes <= kStateKept) {
+        c->state_host.resize(bytes);
+        CU(cudaMemcpyAsync(c->state_host.data(), tmp, bytes, cudaMemcpyDeviceToHost, c->stream));
+        CU(cudaStreamSynchronize(c->stream));
+        for (auto &o : outs)
+            if (o.to) std::memcpy(o.to, c->state_host.data() + o.from, o.bytes);
+    } else {
+        for (auto &o : outs)
+            if (o.to) CU(cudaMemcpyAsync(o.to, tmp + o.from, o.bytes, cudaMemcpyDeviceToHost, c->stream));
+        CU(cudaStreamSynchronize(c->stream));
+    }
     return LPSIM_OK;
 }
 

@@ -1227,6 +1227,18 @@ namespace lpsim {
 
 namespace {
 
+__global__ void state_clear(const uint8_t *trip_status, uint64_t n, float *x, float *v, uint32_t *edge, uint8_t *lane,
+                            uint32_t *ridx, uint8_t *status) {
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+        x[i] = 0.0f;
+        v[i] = 0.0f;
+        edge[i] = kNone;
+        ridx[i] = 0u;
+        lane[i] = 0;
+        status[i] = trip_status[i];
+    }
+}
+
 // state of every live slot, scattered to vehicle-id order
 __global__ void state_scatter(Dev d, uint32_t k, float *x, float *v, uint32_t *edge, uint8_t *lane, uint32_t *ridx) {
     const uint32_t n = *d.n_slots;
@@ -1268,6 +1280,12 @@ void launch_transpose_bins(const uint32_t *in, uint32_t n_edges, uint32_t n_bins
 
 void launch_route_records(const Dev &d, uint64_t n_trips, RouteRec *out, cudaStream_t st) {
     route_records<<<1024, 128, 0, st>>>(d, n_trips, out);
+}
+
+void launch_state_clear(const Dev &d, uint64_t n, float *x, float *v, uint32_t *edge, uint8_t *lane, uint32_t *ridx,
+                        uint8_t *status, cudaStream_t st) {
+    state_clear<<<(unsigned)std::min<uint64_t>((n + 255) / 256, 1024), 256, 0, st>>>(d.status, n, x, v, edge, lane, ridx,
+                                                                                  status);
 }
 
 void launch_state_scatter(const Dev &d, uint32_t k, float *x, float *v, uint32_t *edge, uint8_t *lane,
