@@ -20,10 +20,9 @@ constexpr uint8_t kWaiting = 0;
 constexpr uint8_t kActive = 1;
 constexpr uint8_t kArrived = 2;
 
-// light-load mode: one block of kSmallBlock threads runs a whole chunk when at
+// light-load mode: one block runs a whole chunk (or a piece of one) when at
 // most kSmallMax trips (the default of lpsim_params.light_trips) can be on the
 // network or waiting during it
-constexpr int kSmallBlock = 1024;
 constexpr uint32_t kSmallMax = 1536;
 
 // device error bits
@@ -293,12 +292,13 @@ void launch_apply_crossings(const Dev &d, int grid, cudaStream_t st);
 // kernel timing: the spans of steps [0, nsteps) of the chunk (and of the
 // light-load kernel) into the accumulators; clears the span slots
 void launch_timing_fold(const Dev &d, uint32_t nsteps, cudaStream_t st);
-// steps [k0, k0 + nsteps) in one block (light load); olist: n_org scratch
-// entries, no: one device counter
+// steps [k0, k0 + nsteps) in one block (light load: at most `trips` trips on
+// the network or waiting in them); olist: n_org scratch entries, no: one device
+// counter
 // shared memory the light-load kernel may take for the lane maps (five maps)
 constexpr size_t kSmallMapSmem = 200 * 1024;
 cudaError_t launch_small(const Dev &d, uint32_t k0, uint32_t nsteps, uint32_t *olist, uint32_t *no,
-                         uint32_t map_words, cudaStream_t st);
+                         uint32_t map_words, uint32_t trips, cudaStream_t st);
 
 // compaction (and optional sort by lane-map cell) of the slots after step k;
 // src/dst slot sets; writes *n_slots

@@ -315,11 +315,12 @@ int chunk(lpsim_ctx *c) {
 // Light load: at most light_trips trips can be on the network or waiting in
 // the `steps` steps from step k on (trips due before their end minus those
 // arrived; h_ctr is current).
-bool light_ok(const lpsim_ctx *c, uint32_t steps) {
+bool light_ok(const lpsim_ctx *c, uint32_t steps, uint32_t &trips) {
     if (c->p.flags & LPSIM_F_NO_LIGHT) return false;
     const uint64_t due = (uint64_t)(std::lower_bound(c->dep_sorted.begin(), c->dep_sorted.end(),
                                                      (uint64_t)c->k + steps) -
                                     c->dep_sorted.begin());
+    trips = (uint32_t)(due - std::min<uint64_t>(due, c->h_ctr[1]));
     return due <= c->h_ctr[1] + (c->p.light_trips ? c->p.light_trips : kSmallMax);
 }
 
@@ -327,7 +328,7 @@ bool light_ok(const lpsim_ctx *c, uint32_t steps) {
 // (when the piece reaches a sort period's end, so at least once per chunk:
 // never more than a chunk's departures between two) and the step-counter
 // update.
-int light_steps(lpsim_ctx *c, uint32_t steps) {
+int light_steps(lpsim_ctx *c, uint32_t steps, uint32_t trips) {
     c->ctr_current = false;
     Dev d = c->d;
     d.s = c->sets[c->cur];
@@ -336,7 +337,7 @@ int light_steps(lpsim_ctx *c, uint32_t steps) {
     const uint64_t words = (c->map_bytes + 15) / 16;
     const uint32_t map_words =
         ((c->p.flags & LPSIM_F_SHARED_MAPS) && words * 16 * 5 <= kSmallMapSmem) ? (uint32_t)words : 0u;
-    CU(launch_small(d, c->k, steps, c->small_list, c->small_n, map_words, c->stream));
+    CU(launch_small(d, c->k, steps, c->small_list, c->small_n, map_words, trips, c->stream));
     c->launches += 4;
     if ((c->k + steps) / c->R > c->k / c->R) {
         launch_compact(d, c->sets[c->cur ^ 1], c->w, steps - 1, c->sort, c->grid, c->stream);
@@ -369,16 +370,17 @@ int run_steps(lpsim_ctx *c, uint64_t n, bool stop_done, uint64_t *taken) {
     while (left > 0) {
         if (stop_done && c->h_ctr[1] >= c->n_trips) break;  // h_ctr is current throughout the loop
         uint64_t before = c->k;
+        uint32_t trips = 0;
         if (c->k % c->C == 0 && left >= c->C) {
-            if (light_ok(c, c->C))
-                TRY(light_steps(c, c->C));
+            if (light_ok(c, c->C, trips))
+                TRY(light_steps(c, c->C, trips));
             else
                 TRY(chunk(c));
         } else {
             uint32_t todo = (uint32_t)std::min<uint64_t>(left, c->k % c->C == 0 ? left : c->C - c->k % c->C);
             // (with kernel timing on, a timed light-load launch is a whole chunk: its readers count on it)
-            if (todo >= kLightMinSteps && !c->d.tspan && light_ok(c, todo))
-                TRY(light_steps(c, todo));
+            if (todo >= kLightMinSteps && !c->d.tspan && light_ok(c, todo, trips))
+                TRY(light_steps(c, todo, trips));
             else
                 TRY(direct_steps(c, todo));
         }

@@ -990,7 +990,8 @@ __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) step_p2(Dev d, uint32_t k
 // block's shared memory for the chunk and back at its end, and every phase
 // reads and writes them there (through generic addresses: the phase bodies
 // are the same code); 0: they stay in global memory.
-__global__ void __launch_bounds__(kSmallBlock, 1)
+template <int BLOCK>
+__global__ void __launch_bounds__(BLOCK, 1)
     step_small(Dev d, uint32_t k0, uint32_t nsteps, const uint32_t *olist, const uint32_t *no_ptr,
                uint32_t map_words) {
     extern __shared__ __align__(16) uint4 s_maps[];
@@ -1004,7 +1005,7 @@ __global__ void __launch_bounds__(kSmallBlock, 1)
         for (int a = 0; a < 5; a++) {
             const uint4 *g = reinterpret_cast<const uint4 *>(gmaps[a]);
             uint4 *sm = s_maps + (size_t)a * map_words;
-            for (uint32_t i = tid; i < map_words; i += kSmallBlock) sm[i] = g[i];
+            for (uint32_t i = tid; i < map_words; i += BLOCK) sm[i] = g[i];
         }
     }
     __shared__ __align__(16) CrossRec s_cr[kStageCross];
@@ -1013,7 +1014,7 @@ __global__ void __launch_bounds__(kSmallBlock, 1)
     __shared__ uint32_t s_n[2][4];  // stage counters, by step parity
     if (tid < 8) s_n[tid >> 2][tid & 3u] = 0;
     __syncthreads();
-    const uint32_t tid_mid = (tid - kSmallBlock * 3 / 8) % kSmallBlock, tid_down = kSmallBlock - 1 - tid;
+    const uint32_t tid_mid = (tid - BLOCK * 3 / 8) % BLOCK, tid_down = BLOCK - 1 - tid;
     uint32_t live = 0, arrived = 0, events = 0, departed = 0, changes = 0;
     for (uint32_t t = 0; t < nsteps; t++) {
         const uint32_t k = k0 + t, par = k & 1u;
@@ -1031,22 +1032,22 @@ __global__ void __launch_bounds__(kSmallBlock, 1)
         }
         // P1
         const P1Sinks sk{s_cr, s_ir, s_dr, s_n[par]};
-        for (uint32_t i = tid_down; i < no; i += kSmallBlock) p1_origin(d, w, sk, olist[i]);
-        for (uint32_t s = tid; s < n; s += kSmallBlock) p1_slot(d, w, sk, s, live, arrived);
+        for (uint32_t i = tid_down; i < no; i += BLOCK) p1_origin(d, w, sk, olist[i]);
+        for (uint32_t s = tid; s < n; s += BLOCK) p1_slot(d, w, sk, s, live, arrived);
         __syncthreads();
         // P2: staged items first, then the overflow in the global lists
         const uint32_t ncross = s_n[par][0], nint = s_n[par][1], ndep = s_n[par][2], nlate = s_n[par][3];
         if (tid < 4) s_n[par ^ 1u][tid] = 0;  // the next step's
-        for (uint32_t i = tid; i < ncross; i += kSmallBlock)
+        for (uint32_t i = tid; i < ncross; i += BLOCK)
             p2_cross(d, w, i < kStageCross ? s_cr[i] : d.cross_list[par][i - kStageCross], ev0 + i, events);
-        for (uint32_t i = tid_mid; i < nint; i += kSmallBlock)
+        for (uint32_t i = tid_mid; i < nint; i += BLOCK)
             lane_change<false>(d, w, i < kStageIntend ? s_ir[i] : d.intend_list[par][i - kStageIntend], changes, false);
-        for (uint32_t q = tid_down; q < ndep; q += kSmallBlock)
+        for (uint32_t q = tid_down; q < ndep; q += BLOCK)
             p2_dep(d, w, q < kStageDep ? s_dr[q] : d.dep_rec[par][q - kStageDep], q, n, events, departed);
         if (nlate) {
             // P3: the intents at stop-line cells, after every hold
             __syncthreads();
-            for (uint32_t i = tid; i < nlate; i += kSmallBlock)
+            for (uint32_t i = tid; i < nlate; i += BLOCK)
                 lane_change<false>(d, w, d.intend_list[par][d.cap - 1 - i], changes, false);
         }
         if (tid == 0) {  // the next step's global lists start empty
@@ -1068,7 +1069,7 @@ __global__ void __launch_bounds__(kSmallBlock, 1)
         for (int a = 0; a < 5; a++) {
             const uint4 *sm = s_maps + (size_t)a * map_words;
             uint4 *g = reinterpret_cast<uint4 *>(gmaps[a]);
-            for (uint32_t i = tid; i < map_words; i += kSmallBlock) g[i] = sm[i];
+            for (uint32_t i = tid; i < map_words; i += BLOCK) g[i] = sm[i];
         }
     }
     warp_add64(&d.ctr[0], live);
@@ -1205,19 +1206,24 @@ void launch_apply_crossings(const Dev &d, int grid, cudaStream_t st) { apply_cro
 void launch_timing_fold(const Dev &d, uint32_t nsteps, cudaStream_t st) { timing_fold<<<1, 1024, 0, st>>>(d, nsteps); }
 
 cudaError_t launch_small(const Dev &d, uint32_t k0, uint32_t nsteps, uint32_t *olist, uint32_t *no,
-                         uint32_t map_words, cudaStream_t st) {
+                         uint32_t map_words, uint32_t trips, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(no, 0, 4, st);
     if (e != cudaSuccess) return e;
     const size_t smem = (size_t)map_words * 16 * 5;
     if (smem > kSmallMapSmem) return cudaErrorInvalidValue;
-    static bool attr_set = false;
-    if (smem > 48 * 1024 && !attr_set) {
-        e = cudaFuncSetAttribute(step_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallMapSmem);
+    // The block for the trips there can be: idle warps cost every barrier and
+    // loop, and a smaller block leaves a thread more registers.  Measured with 256
+    // / 512 / 1024 threads, ms per run to completion: 500 trips on 8x8 nodes 9.8 /
+    // 10.3 / 11.6, 2,000 trips on 8x8 (most chunks up to 1,000) 18.6 / 15.5 / 16.2;
+    // with the lines at 256 and 768 trips 9.9 and 15.2.
+    const int block = trips <= 256u ? 256 : trips <= 768u ? 512 : 1024;
+    const auto kernel = block == 256 ? step_small<256> : block == 512 ? step_small<512> : step_small<1024>;
+    if (smem > 48 * 1024) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallMapSmem);
         if (e != cudaSuccess) return e;
-        attr_set = true;
     }
     small_origins<<<(d.n_org + 255) / 256 + 1, 256, 0, st>>>(d, k0 + nsteps, olist, no);
-    step_small<<<1, kSmallBlock, smem, st>>>(d, k0, nsteps, olist, no, map_words);
+    kernel<<<1, block, smem, st>>>(d, k0, nsteps, olist, no, map_words);
     return cudaGetLastError();
 }
 
