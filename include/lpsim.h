@@ -98,7 +98,7 @@ typedef struct lpsim_params {
                              networks of up to ~40k lane-metres; results are the same either way;
                              measured 2% slower on a 4x4 grid, whose maps stay in L2 anyway);
                              other bits must be 0 */
-    uint32_t light_trips; /* a chunk runs in the single-block light-load kernel when at most this many
+    uint32_t light_trips; /* a chunk (or a piece of one) runs in the single-block light-load kernel when at most this many
                              trips can be on the network or waiting during it (0 = 1536); a speed
                              setting only, results are the same for every value */
     float dlc_prob;       /* discretionary lane change (an extension; the paper defines only the

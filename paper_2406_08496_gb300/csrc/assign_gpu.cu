@@ -132,8 +132,9 @@ struct TreeArgs {
     uint32_t *edges;          // path edges, travel order
     unsigned long long cap;   // entries of edges
     unsigned long long *cursor;
-    // td_trees_shared: positions along each thread's path, kScratch per thread
+    // td_trees_shared: positions along each thread's path, scratch_len per thread
     uint32_t *scratch;
+    uint32_t scratch_len;     // kScratch, or the node count where that is less (no path is as long)
     // td_trees: per-warp workspaces
     NodeRec *node;            // n_warps x n_nodes: label, round stamp of the last push, far-pile mark
     uint32_t *touched;        // n_warps x n_nodes
@@ -406,7 +407,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSm) td_trees(Tr
 constexpr uint32_t kWide = 8;       // most out-edges per node for the wide rows
 constexpr uint64_t kSharedDeltaMs = 240000;
 constexpr uint32_t kRing = 1024;    // ids of waiting nodes (a power of two)
-constexpr uint32_t kScratch = 512;  // positions kept per thread while a path is walked back
+constexpr uint32_t kScratch = 512;  // positions kept per thread at most while a path is walked back
 constexpr uint32_t kNever = 0xFFFFFFFFu;
 
 __host__ __device__ inline size_t shared_tree_bytes(uint32_t n_nodes) {
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(T, PER_SM) td_trees_shared(TreeArgs A) {
     __shared__ uint32_t s_group, s_cnt[3], s_min[3], s_red[32];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     volatile uint32_t *vlab = s_lab;
-    uint32_t *scratch = A.scratch + (size_t)blockIdx.x * T * kScratch + tid;
+    uint32_t *scratch = A.scratch + (size_t)blockIdx.x * T * A.scratch_len + tid;
     const uint64_t max_rounds = 8ull * A.n_nodes + (1ull << 20);
     for (;;) {
         if (tid == 0) s_group = atomicAdd(A.next_group, 1u);
@@ -570,7 +571,7 @@ __global__ void __launch_bounds__(T, PER_SM) td_trees_shared(TreeArgs A) {
                     ok = false;
                     break;
                 }
-                if (L < kScratch) scratch[(size_t)L * T] = in.x;
+                if (L < A.scratch_len) scratch[(size_t)L * T] = in.x;
                 v = in.y;
             }
             if (!ok) {
@@ -582,7 +583,7 @@ __global__ void __launch_bounds__(T, PER_SM) td_trees_shared(TreeArgs A) {
                 atomicOr(A.err, kErrCapacity);
                 continue;
             }
-            if (L > kScratch) {  // a path longer than the scratch: its positions go through the output
+            if (L > A.scratch_len) {  // a path longer than the scratch: its positions go through the output
                 uint32_t p = L;
                 for (uint32_t v = d; v != G.src && p > 0;) {
                     const uint2 in = entering(v);
@@ -593,7 +594,7 @@ __global__ void __launch_bounds__(T, PER_SM) td_trees_shared(TreeArgs A) {
             const uint64_t tj = A.dep_ms[jt];
             uint64_t t = tj;
             for (uint32_t p = 0; p < L; p++) {
-                const uint32_t j = L > kScratch ? A.edges[off + p] : scratch[(size_t)(L - 1 - p) * T];
+                const uint32_t j = L > A.scratch_len ? A.edges[off + p] : scratch[(size_t)(L - 1 - p) * T];
                 A.edges[off + p] = A.adj[j].x;
                 t = arrive(A.cms[(size_t)bin_of(A, t) * A.n_pos + j], t);
             }
@@ -860,7 +861,8 @@ int gpu_setup(lpsim_assign *a) {
             g->shared_kernel = kernel;
             g->shared_threads = (uint32_t)threads;
             g->shared_blocks = (uint32_t)(g->n_sm * per_sm);
-            A.scratch = static_cast<uint32_t *>(g->alloc((size_t)g->shared_blocks * threads * kScratch * 4));
+            A.scratch_len = std::min(kScratch, a->n_nodes);
+            A.scratch = static_cast<uint32_t *>(g->alloc((size_t)g->shared_blocks * threads * A.scratch_len * 4));
             if (!A.scratch) return fail(LPSIM_E_OOM, "device allocation of the search workspaces failed");
             CU(cudaStreamSynchronize(g->stream));  // the host arrays go away
             return LPSIM_OK;

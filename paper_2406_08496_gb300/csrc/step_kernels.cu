@@ -31,10 +31,11 @@
 //
 // Latency, not bandwidth, bounds these kernels (a step moves a few MB), so
 // each is arranged to need as few dependent memory round trips as possible:
-// the parity buffers and maps are chosen from a launch argument, the first
-// records of a thread are loaded together with the step number and the list
-// lengths, and records that a later phase needs are packed by the phase that
-// already holds the values.
+// the parity buffers and maps are chosen from a launch argument, step_p2 loads
+// a thread's first record together with the step number and the list lengths,
+// loads that a vehicle may need are issued before the values of others are used,
+// and records that a later phase needs are packed by the phase that already
+// holds the values.
 //
 // Every floating-point expression is written in the same operation order as
 // the rules state; the library is compiled with -fmad=false -prec-div=true

@@ -317,6 +317,36 @@ def test_uneven_pieces_match_oracle(grid_day, flags, light_trips):
         assert co[key] == cg[key], (key, co[key], cg[key])
 
 
+@pytest.mark.parametrize("n_trips", [3, 250, 300, 760, 800, 1500])
+def test_light_block_sizes_reset_and_restore(n_trips):
+    """Trip counts on both sides of each choice of the light-load kernel's block
+    (256, 512, 1,024 threads), all departing within a minute, on a network whose
+    buffers are no whole 16-byte words: every output matches the oracle at the
+    end, after a reset and a second run, and after a restore in between."""
+    import oracle as O
+    from paper_2406_08496_gb300 import Simulation
+    net = W.grid_network(5, 7)
+    dem = W.route(net, W.uniform_demand(net, n_trips, 17, t_max_s=60.0))
+    params = dict(bin_steps=250, n_bins=7, dlc_prob=0.2, dlc_gain=3.0, eps_amp=1.0)
+    o = O.Oracle(net, params)
+    o.load_demand(dem)
+    g = Simulation(net, dict(params, flags=2))
+    g.load_demand(dem)
+    g.step(203)
+    g.snapshot()
+    g.step(1000)
+    g.restore()
+    o.step(203)
+    assert_outputs_equal(o, g, n_bins=7, where="restored")
+    o.run(20000)
+    for _ in range(2):
+        g.run(20000)
+        assert_outputs_equal(o, g, n_bins=7)
+        assert g.counters()["arrived"] == o.counters()["arrived"]
+        g.reset()
+        assert g.counters()["veh_steps"] == 0 and g.counters()["k"] == 0
+
+
 def test_light_and_grid_wide_chunks_alternate():
     """8,000 trips on a 12x12 grid: the chunks switch between the grid-wide
     kernels and the light-load block as the network fills and drains; every
