@@ -1512,10 +1512,11 @@ struct lpsim_mlp {
     __nv_bfloat16 *Wb[3] = {}, *WbT[3] = {};
     // one batch: inputs as given, inputs and hidden activations in bf16, the
     // backward's dZ1..3
-    float *Xf, *t, *y;
+    float *Xf, *t, *y_block, *y;  // y follows an error word of its own, so one copy brings both
     __nv_bfloat16 *X0, *H[2], *dZ[3];
     float *small, *part;  // partial sums of mlp_train_fused (per cluster) and mlp_wgrad (per split)
     uint32_t *err;
+    uint32_t failed = 0;  // error bits any call of this model has met
     CUtensorMap mW[3];
     TrainMaps tmaps;
     WgradMaps gmaps;
@@ -1565,7 +1566,8 @@ const int kDims[5] = {64, 256, 256, 256, 1};
 
 constexpr int kLossAt = (param_off(8) + 3) / 4 * 4, kErrAt = kLossAt + 1;  // in the gradients' flat array
 
-int err_status(uint32_t e) {
+int err_status(lpsim_mlp *m, uint32_t e) {
+    e = m->failed |= e;
     if (e & 64u) return fail(LPSIM_E_TIMEOUT, "training-pool permutation walk exceeded its bound");
     if (e) return fail(LPSIM_E_TIMEOUT, "tensor-core GEMM wait gave up (code " + std::to_string(e) + ")");
     return LPSIM_OK;
@@ -1575,7 +1577,7 @@ int mlp_check_err(lpsim_mlp *m) {
     uint32_t e = 0;
     CU(cudaMemcpyAsync(&e, m->err, 4, cudaMemcpyDeviceToHost, m->stream));
     CU(cudaStreamSynchronize(m->stream));
-    return err_status(e);
+    return err_status(m, e);
 }
 
 int refresh_weights(lpsim_mlp *m) {
@@ -1661,7 +1663,7 @@ int train_update(lpsim_mlp *m, const UpdateArgs &u) {
 }
 
 // inference forward of n rows of m->nf inputs (device) into y
-int forward_fused(lpsim_mlp *m, const float *X, uint64_t n, float *y) {
+int forward_fused(lpsim_mlp *m, const float *X, uint64_t n, float *y, uint32_t *err) {
     CU(cudaFuncSetAttribute(mlp_forward_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem));
     FwdArgs g{};
     g.n_rows = (int)n;
@@ -1675,13 +1677,18 @@ int forward_fused(lpsim_mlp *m, const float *X, uint64_t n, float *y) {
     g.w4 = m->P[6];
     g.b4 = m->P[7];
     g.y = y;
-    g.err = m->err;
+    g.err = err;
     const int grid = std::min(g.n_tiles, m->n_sm);
     mlp_forward_fused<<<grid, kFwdThreads, kFwdSmem, m->stream>>>(m->mW[0], m->mW[1], m->mW[2], g);
     m->launches++;
     CU(cudaGetLastError());
     return LPSIM_OK;
 }
+
+// Inference calls of at most this many rows bring their outputs and the error
+// word over in one copy, then copy the outputs on the host (a copy from the
+// device costs some 8 us however small).
+constexpr uint64_t kOneCopyRows = 16384;
 
 // Rows per launch of a long inference call: four tiles per SM, whole waves, for
 // which the kernel takes 35.5 us and the copy in 22 us.  (One launch per batch
@@ -1702,7 +1709,7 @@ int forward_pieces(lpsim_mlp *m, uint64_t n, const float *X, float *y) {
         CU(cudaMemcpyAsync(m->in[b], X + r0 * m->nf, nb * m->nf * 4, cudaMemcpyHostToDevice, m->in_stream));
         CU(cudaEventRecord(m->in_here[b], m->in_stream));
         CU(cudaStreamWaitEvent(m->stream, m->in_here[b], 0));
-        TRY(forward_fused(m, m->in[b], nb, m->y_all + r0));
+        TRY(forward_fused(m, m->in[b], nb, m->y_all + r0, m->err));
         CU(cudaEventRecord(m->in_used[b], m->stream));
     }
     CU(cudaMemcpyAsync(y, m->y_all, n * 4, cudaMemcpyDeviceToHost, m->stream));
@@ -1712,7 +1719,7 @@ int forward_pieces(lpsim_mlp *m, uint64_t n, const float *X, float *y) {
 // a flat parameter-shaped device array into the caller's tensors (each
 // nullable): one copy, then host copies
 int flat_to_tensors(lpsim_mlp *m, const float *flat, float *const *tensors) {
-    m->h_flat.resize(kErrAt + 1);
+    m->h_flat.resize(std::max<size_t>(m->h_flat.size(), kErrAt + 1));
     CU(cudaMemcpyAsync(m->h_flat.data(), flat, (kErrAt + 1) * 4, cudaMemcpyDeviceToHost, m->stream));
     CU(cudaStreamSynchronize(m->stream));
     for (int i = 0; i < 8 && tensors; i++)
@@ -1773,10 +1780,12 @@ int lpsim_mlp_create(lpsim_mlp **out, uint32_t n_features, uint32_t batch, uint6
     }
     m->X0 = (__nv_bfloat16 *)m->alloc((size_t)B * 64 * 2);
     m->Xf = (float *)m->alloc((size_t)B * n_features * 4);
-    m->y = (float *)m->alloc((size_t)B * 4);
+    m->y_block = (float *)m->alloc(((size_t)B + 4) * 4);
+    m->y = m->y_block ? m->y_block + 4 : nullptr;
     m->t = (float *)m->alloc((size_t)B * 4);
     if (!m->X0 || !m->Xf || !m->y || !m->t) return bail(fail(LPSIM_E_OOM, "device allocation failed"));
-    if (cudaMemsetAsync(m->err, 0, 4, m->stream) != cudaSuccess) return bail(fail(LPSIM_E_CUDA, "memset"));
+    if (cudaMemsetAsync(m->err, 0, 4, m->stream) != cudaSuccess ||
+        cudaMemsetAsync(m->y_block, 0, 16, m->stream) != cudaSuccess) return bail(fail(LPSIM_E_CUDA, "memset"));
     // tensor maps of every operand
     int rc;
     TrainMaps &tm = m->tmaps;
@@ -1838,7 +1847,18 @@ int lpsim_mlp_forward(lpsim_mlp *m, uint64_t n, const float *X, float *y) {
     if (n <= (uint64_t)m->B) {
         if (n == 0) return mlp_check_err(m);
         CU(cudaMemcpyAsync(m->Xf, X, n * m->nf * 4, cudaMemcpyHostToDevice, m->stream));
-        TRY(forward_fused(m, m->Xf, n, m->y));
+        if (n <= kOneCopyRows) {
+            m->h_flat.resize(std::max<size_t>(m->h_flat.size(), n + 4));
+            TRY(forward_fused(m, m->Xf, n, m->y, reinterpret_cast<uint32_t *>(m->y_block)));
+            CU(cudaMemcpyAsync(m->h_flat.data(), m->y_block, (n + 4) * 4, cudaMemcpyDeviceToHost, m->stream));
+            CU(cudaStreamSynchronize(m->stream));
+            uint32_t e;
+            std::memcpy(&e, m->h_flat.data(), 4);
+            TRY(err_status(m, e));
+            std::memcpy(y, m->h_flat.data() + 4, n * 4);
+            return LPSIM_OK;
+        }
+        TRY(forward_fused(m, m->Xf, n, m->y, m->err));
         CU(cudaMemcpyAsync(y, m->y, n * 4, cudaMemcpyDeviceToHost, m->stream));
         return mlp_check_err(m);
     }
@@ -1886,7 +1906,7 @@ int lpsim_mlp_grad(lpsim_mlp *m, uint64_t n, const float *X, const float *t, flo
     TRY(flat_to_tensors(m, m->Gf, grads));
     uint32_t e;
     std::memcpy(&e, &m->h_flat[kErrAt], 4);
-    TRY(err_status(e));
+    TRY(err_status(m, e));
     if (loss) *loss = m->h_flat[kLossAt] / (float)n;
     return LPSIM_OK;
 }
@@ -2045,9 +2065,9 @@ int lpsim_mlp_time(lpsim_mlp *m, uint32_t iters, double *fwd_ms, double *train_m
     CU(cudaEventCreate(&e0));
     CU(cudaEventCreate(&e1));
     // whatever the batch buffers hold is a valid input; warm up once
-    TRY(forward_fused(m, m->Xf, (uint64_t)m->B, m->y));
+    TRY(forward_fused(m, m->Xf, (uint64_t)m->B, m->y, m->err));
     CU(cudaEventRecord(e0, m->stream));
-    for (uint32_t i = 0; i < iters; i++) TRY(forward_fused(m, m->Xf, (uint64_t)m->B, m->y));
+    for (uint32_t i = 0; i < iters; i++) TRY(forward_fused(m, m->Xf, (uint64_t)m->B, m->y, m->err));
     CU(cudaEventRecord(e1, m->stream));
     CU(cudaEventSynchronize(e1));
     float ms = 0.0f;
