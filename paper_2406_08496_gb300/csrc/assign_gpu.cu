@@ -49,6 +49,7 @@
 #include <memory>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/lpsim_assign.h"
@@ -719,6 +720,18 @@ struct AssignGpu {
             cudaFree(p);
         }
     }
+    // room for n entries in place of p's block (contents not kept).  A failure
+    // leaves p null and cap 0, so that the next call allocates again instead of
+    // running on what is not there.
+    template <class T, class N>
+    bool regrow(T *&p, N &cap, size_t n) {
+        if (p) release(const_cast<std::remove_const_t<T> *>(p));
+        p = nullptr;
+        cap = 0;
+        p = static_cast<T *>(alloc(n * sizeof(T)));
+        if (p) cap = (N)n;
+        return p != nullptr;
+    }
     ~AssignGpu() {
         if (stream) cudaStreamSynchronize(stream);
         for (void *b : blocks) cudaFree(b);
@@ -917,13 +930,17 @@ int gpu_groups(lpsim_assign *a, uint32_t period_steps) {
         recs[q] = GroupRec{a->orig[j0], (uint32_t)t0, (uint32_t)g->gstart[q],
                            (uint32_t)(g->gstart[q + 1] - g->gstart[q])};
     }
+    // no grouping until the new one is there
+    g->period_steps = 0;
     if (g->A.groups) g->release(const_cast<GroupRec *>(g->A.groups));
     if (g->A.order) g->release(const_cast<uint32_t *>(g->A.order));
+    g->A.groups = nullptr;
+    g->A.order = nullptr;
     GroupRec *dg;
     uint32_t *dord;
     TRY(dput(g, dg, recs.data(), recs.size()));
-    TRY(dput(g, dord, ord.data(), ord.size()));
     g->A.groups = dg;
+    TRY(dput(g, dord, ord.data(), ord.size()));
     g->A.order = dord;
     g->A.n_groups = (uint32_t)ng;
     g->period_steps = period_steps;
@@ -944,20 +961,10 @@ int gpu_table(lpsim_assign *a, const float *tt, uint32_t n_bins, uint32_t bin_st
     if (bin_ms > 0xFFFFFFFFull) return fail(LPSIM_E_INVALID_ARG, "bin longer than the 32-bit millisecond range");
     const uint32_t n_pos = wide ? g->wide * a->n_nodes : a->n_edges;
     const size_t in_cells = (size_t)n_bins * a->n_edges, cells = (size_t)n_bins * n_pos;
-    if (cells > g->table_cells[wide]) {
-        if (g->table[wide]) g->release(g->table[wide]);
-        g->table_cells[wide] = 0;
-        g->table[wide] = static_cast<uint2 *>(g->alloc(cells * sizeof(uint2)));
-        if (!g->table[wide]) return fail(LPSIM_E_OOM, "device allocation of the link-time table failed");
-        g->table_cells[wide] = cells;
-    }
-    if (in_cells > g->tt_cells) {
-        if (g->tt) g->release(g->tt);
-        g->tt_cells = 0;
-        g->tt = static_cast<float *>(g->alloc(in_cells * 4));
-        if (!g->tt) return fail(LPSIM_E_OOM, "device allocation of the link times failed");
-        g->tt_cells = in_cells;
-    }
+    if (cells > g->table_cells[wide] && !g->regrow(g->table[wide], g->table_cells[wide], cells))
+        return fail(LPSIM_E_OOM, "device allocation of the link-time table failed");
+    if (in_cells > g->tt_cells && !g->regrow(g->tt, g->tt_cells, in_cells))
+        return fail(LPSIM_E_OOM, "device allocation of the link times failed");
     CU(cudaMemcpyAsync(g->tt, tt, in_cells * 4, cudaMemcpyHostToDevice, g->stream));
     if (n_pos)
         link_table<<<(n_pos + 31) / 32, 256, 0, g->stream>>>(g->tt, wide ? g->wide_adj : A.adj, n_pos, n_bins, bin_ms,
@@ -992,15 +999,9 @@ extern "C" int lpsim_assign_load_gpu(const lpsim_assign *ac, const float *tt, ui
     }
     if (g->routes_version != a->routes_version) {
         const uint64_t total = a->roff[a->n];
-        if (total > g->redge_cap) {
-            if (g->redge) g->release(g->redge);
-            g->redge = nullptr;
-            g->redge_cap = 0;
-            g->redge = static_cast<uint32_t *>(g->alloc((total + total / 4) * 4));
-            if (!g->redge) return fail(LPSIM_E_OOM, "device allocation of the routes failed");
-            g->redge_cap = total + total / 4;
-        }
         g->routes_version = ~0ull;
+        if (total > g->redge_cap && !g->regrow(g->redge, g->redge_cap, total + total / 4))
+            return fail(LPSIM_E_OOM, "device allocation of the routes failed");
         CU(cudaMemcpyAsync(g->roff, a->roff.data(), (a->n + 1) * 8, cudaMemcpyHostToDevice, g->stream));
         if (total)
             CU(cudaMemcpyAsync(g->redge, a->redge.p.get(), total * 4, cudaMemcpyHostToDevice, g->stream));
@@ -1008,12 +1009,8 @@ extern "C" int lpsim_assign_load_gpu(const lpsim_assign *ac, const float *tt, ui
         g->routes_version = a->routes_version;
     }
     const size_t cells = (size_t)a->n_edges * n_bins;
-    if (cells > g->inflow_cells) {
-        if (g->inflow) g->release(g->inflow);
-        g->inflow = static_cast<uint32_t *>(g->alloc(cells * 4));
-        if (!g->inflow) return fail(LPSIM_E_OOM, "device allocation of the inflow table failed");
-        g->inflow_cells = cells;
-    }
+    if (cells > g->inflow_cells && !g->regrow(g->inflow, g->inflow_cells, cells))
+        return fail(LPSIM_E_OOM, "device allocation of the inflow table failed");
     CU(cudaMemsetAsync(g->inflow, 0, cells * 4, g->stream));
     load_routes<<<(unsigned)std::min<uint64_t>((a->n + 255) / 256, 65535), 256, 0, g->stream>>>(
         g->roff, g->redge, g->A.dep_ms, a->n, g->A.cms, g->A.pos, a->n_edges, n_bins, g->A.bin_ms, g->inflow);
@@ -1039,9 +1036,8 @@ extern "C" int lpsim_assign_shortest_paths_gpu(lpsim_assign *a, const float *tt,
     // path buffer: room for the current routes' length and half as much again
     if (!g->cap) {
         const uint64_t total = a->roff[a->n];
-        g->cap = std::max<uint64_t>(total + total / 2, 1u << 20);
-        A.edges = static_cast<uint32_t *>(g->alloc(g->cap * 4));
-        if (!A.edges) return fail(LPSIM_E_OOM, "device allocation of the path buffer failed");
+        if (!g->regrow(A.edges, g->cap, std::max<uint64_t>(total + total / 2, 1u << 20)))
+            return fail(LPSIM_E_OOM, "device allocation of the path buffer failed");
     }
     unsigned long long used = 0;
     uint32_t err = 0;
@@ -1069,10 +1065,8 @@ extern "C" int lpsim_assign_shortest_paths_gpu(lpsim_assign *a, const float *tt,
         CU(cudaStreamSynchronize(g->stream));
         if (!(err & kErrCapacity)) break;
         // the paths did not fit: a buffer of the length they asked for, and again
-        g->release(A.edges);
-        g->cap = used + used / 4 + 1024;
-        A.edges = static_cast<uint32_t *>(g->alloc(g->cap * 4));
-        if (!A.edges) return fail(LPSIM_E_OOM, "device allocation of the path buffer failed");
+        if (!g->regrow(A.edges, g->cap, used + used / 4 + 1024))
+            return fail(LPSIM_E_OOM, "device allocation of the path buffer failed");
     }
     if (err & kErrBound) return fail(LPSIM_E_INVARIANT, "GPU path search exceeded its round or path-length bound");
     if (err & kErrUnreachable) return fail(LPSIM_E_INVALID_ARG, "a destination is unreachable from its origin");

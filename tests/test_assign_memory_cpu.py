@@ -1,0 +1,134 @@
+"""The assignment engine's device memory, without a GPU: the library's host code
+linked against a CUDA runtime that only keeps account of allocations, copies
+and launches (fake_cudart.cpp; no kernel runs)."""
+from __future__ import annotations
+
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+P = ctypes.c_void_p
+E_OOM = -2
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    from paper_2406_08496_gb300 import _build
+    out = tmp_path_factory.mktemp("fake")
+    objs = []
+    # (the fake first: its tables are there before the kernels register)
+    for src in (os.path.join(HERE, "fake_cudart.cpp"), os.path.join(_build.CSRC, "assign.cpp"),
+                os.path.join(_build.CSRC, "assign_gpu.cu")):
+        objs.append(str(out / (os.path.basename(src) + ".o")))
+        subprocess.run([_build._nvcc(), *_build.ARCH, "-O1", "-std=c++17", "-Xcompiler", "-fPIC", "-c", src, "-o", objs[-1]],
+                       check=True)
+    so = str(out / "libfake.so")
+    subprocess.run(["g++", "-shared", "-o", so, *objs, "-lpthread"], check=True)
+    lib = ctypes.CDLL(so, mode=os.RTLD_LOCAL | os.RTLD_NOW | os.RTLD_DEEPBIND)
+    u32, u64 = ctypes.c_uint32, ctypes.c_uint64
+    lib.lpsim_assign_create.argtypes = [P, u32, u32, P, P, P, P, P, u64, P, P, P, P, P, ctypes.c_float, u64]
+    lib.lpsim_assign_shortest_paths_gpu.argtypes = [P, P, u32, u32, u32, P]
+    lib.lpsim_assign_load_gpu.argtypes = [P, P, u32, u32, P]
+    lib.lpsim_assign_destroy.argtypes = [P]
+    lib.fake_reset.argtypes = [ctypes.c_long]
+    lib.fake_next_read.argtypes = [ctypes.c_size_t, u64]
+    lib.fake_launch.argtypes = [ctypes.c_int, P]
+    lib.fake_launch.restype = ctypes.c_char_p
+    lib.fake_occupancy.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_size_t]
+    for f in ("fake_calls", "fake_uploaded", "fake_live_bytes"):
+        getattr(lib, f).restype = ctypes.c_long
+    return lib
+
+
+def _p(a):
+    return a.ctypes.data_as(P)
+
+
+class _Engine:
+    """A ring of nodes, both ways round, and trips from a few of them."""
+
+    def __init__(self, lib, n_nodes, n_trips=64, origins=4):
+        self.lib, self.n = lib, n_trips
+        i = np.arange(n_nodes, dtype=np.uint32)
+        src, dst = np.concatenate([i, i]), np.concatenate([(i + 1) % n_nodes, (i - 1) % n_nodes]).astype(np.uint32)
+        self.m = len(src)
+        length, lanes, vmax = np.full(self.m, 100.0, np.float32), np.ones(self.m, np.uint8), np.full(self.m, 10.0, np.float32)
+        orig = (np.arange(n_trips) % origins).astype(np.uint32)
+        dest, dep = ((orig + 2) % n_nodes).astype(np.uint32), np.arange(n_trips, dtype=np.uint32)
+        off = 2 * np.arange(n_trips + 1, dtype=np.uint64)
+        edges = np.stack([orig, (orig + 1) % n_nodes], 1).reshape(-1).astype(np.uint32)
+        h = P()
+        self._keep = (src, dst, length, lanes, vmax, orig, dest, dep, off, edges)
+        assert lib.lpsim_assign_create(ctypes.byref(h), n_nodes, self.m, *[_p(a) for a in self._keep[:5]], n_trips,
+                                       *[_p(a) for a in self._keep[5:]], 0.5, 1) == 0
+        self.h = h
+
+    def search(self, period, n_bins=4):
+        tt, t = np.full((self.m, n_bins), 5.0, np.float32), np.empty(self.n, np.float32)
+        return self.lib.lpsim_assign_shortest_paths_gpu(self.h, _p(tt), n_bins, 60, period, _p(t))
+
+    def load(self, n_bins):
+        tt, f = np.full((self.m, n_bins), 5.0, np.float32), np.empty((self.m, n_bins), np.uint32)
+        return self.lib.lpsim_assign_load_gpu(self.h, _p(tt), n_bins, 60, _p(f))
+
+    def close(self):
+        self.lib.lpsim_assign_destroy(self.h)
+
+
+def _launches(lib, first=0):
+    out = []
+    for i in range(first, lib.fake_launches()):
+        v = np.empty(5, np.int32)
+        name = lib.fake_launch(i, _p(v)).decode()
+        out.append((name, *[int(x) for x in v]))
+    return out
+
+
+def _calls(lib, e):
+    """Every kind of device allocation: set-up, a first search, another period, a
+    path buffer that was too small, a loading, larger tables for both."""
+    def too_small():
+        lib.fake_next_read(8, 3 << 20)  # path edges asked for
+        lib.fake_next_read(4, 2)        # the search's word: the path buffer was too small
+        return e.search(7)
+    return [lambda: e.search(600), lambda: e.search(7), too_small, lambda: e.load(4), lambda: e.load(8),
+            lambda: e.search(600, 8)]
+
+
+@pytest.mark.parametrize("n_nodes", [100, 60000])  # labels in shared memory; workspaces in device memory
+def test_an_engine_survives_each_failed_allocation(lib, n_nodes):
+    """One device allocation fails, each in turn: that call reports
+    LPSIM_E_OOM, and every call after it allocates what is missing again, so
+    that no kernel is launched on a freed or missing buffer."""
+    before = lib.fake_live_bytes()
+    e = _Engine(lib, n_nodes)
+    lib.fake_reset(0)
+    want = []  # launches of each call when nothing fails
+    for call in _calls(lib, e):
+        at = lib.fake_launches()
+        assert call() == 0, lib.lpsim_last_error()
+        want.append({(x[0], x[3]) for x in _launches(lib, at)})
+    total = lib.fake_calls()
+    e.close()
+    assert lib.fake_live_bytes() == before and total > 20
+    for n in range(1, total + 1):
+        e = _Engine(lib, n_nodes)
+        lib.fake_reset(n)
+        rcs = []
+        for call in _calls(lib, e):
+            rcs.append(call())
+        assert rcs.count(E_OOM) == 1 and rcs.count(0) == len(rcs) - 1, (n, rcs)
+        for q, call in enumerate(_calls(lib, e)):
+            at = lib.fake_launches()
+            assert call() == 0, (n, q)
+            for x in _launches(lib, at):
+                assert (x[0], x[3]) in want[q] and x[4] == 0, (n, q, x, want[q])
+        for x in _launches(lib):
+            assert x[4] == 0, (n, x)
+        e.close()
+        assert lib.fake_live_bytes() == before
