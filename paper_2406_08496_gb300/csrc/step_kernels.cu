@@ -1219,7 +1219,8 @@ cudaError_t launch_small(const Dev &d, uint32_t k0, uint32_t nsteps, uint32_t *o
     // with the lines at 256 and 768 trips 9.9 and 15.2.
     const int block = trips <= 256u ? 256 : trips <= 768u ? 512 : 1024;
     const auto kernel = block == 256 ? step_small<256> : block == 512 ? step_small<512> : step_small<1024>;
-    if (smem > 48 * 1024) {
+    if (smem > 0) {
+        // the 48 KB a block has unasked hold the kernel's own stages too, so that maps well below them need the rest
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallMapSmem);
         if (e != cudaSuccess) return e;
     }

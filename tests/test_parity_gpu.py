@@ -467,3 +467,28 @@ def test_kernel_timing_direct_and_graph_steps(grid_day, flags):
     ref.load_demand(dem)
     ref.step(4608)
     assert_state_equal(ref.state(), g.state(), "timing on vs off")
+
+
+@pytest.mark.parametrize("n_edges", [8, 9, 12, 13])
+def test_lane_maps_on_chip_beside_the_stages(n_edges):
+    """A ring of two-lane 400 m links with its lane maps on chip (flags 8): five
+    maps of 800 bytes a link beside the 16 KB of the light-load kernel's own
+    stages, on both sides of the 48 KB a block has without asking for more
+    (maps and stages together from 9 links on, the maps alone from 13 on), in
+    whole chunks and in a piece; every output matches the oracle."""
+    import oracle as O
+    from netutil import make_demand, make_net
+    from paper_2406_08496_gb300 import Simulation
+    net = make_net(n_edges, [(i, (i + 1) % n_edges, 400.0, 2, 13.9) for i in range(n_edges)])
+    dem = make_demand([(3 * j, [(j + q) % n_edges for q in range(n_edges - 1)]) for j in range(90)])
+    params = dict(bin_steps=600, n_bins=4, dlc_prob=0.3, dlc_gain=3.0, eps_amp=1.0)
+    o = O.Oracle(net, params)
+    o.load_demand(dem)
+    g = Simulation(net, dict(params, flags=8 | 2))
+    g.load_demand(dem)
+    for n in (300, 1236, 1536):
+        o.step(n)
+        g.step(n)
+        assert_outputs_equal(o, g, n_bins=4, where=f"step {o.counters()['k']}")
+    assert g.counters()["light_chunks"] >= 1 and g.counters()["arrived"] == o.counters()["arrived"] > 0
+    g.close()
