@@ -394,3 +394,25 @@ def test_training_pool_parts_equal_one_upload():
     assert b.pool_size() == 0
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("n", [1000, 8192, 8193, 200000])
+def test_forward_reads_inputs_after_the_stream_s_work(n):
+    """The rows of a call may still be on their way to (pinned) host memory on
+    the model's stream: the call reads them after that work, in one batch
+    and in pieces alike."""
+    import torch
+    from paper_2406_08496_gb300 import Surrogate
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        s = Surrogate(n_features=11, batch=8192, seed=1)
+        rows = torch.randn((n, 11), device="cuda")
+    st.synchronize()
+    want = s.forward(rows.cpu().numpy())
+    X = torch.full((n, 11), 5.0, pin_memory=True)
+    with torch.cuda.stream(st):
+        torch.cuda._sleep(100_000_000)  # some 50 ms
+        X.copy_(rows, non_blocking=True)
+        got = s.forward(X.numpy())
+    assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
+    s.close()
