@@ -196,9 +196,9 @@ def use_torch_allocator() -> bool:
     def _free(ptr, user):
         torch.cuda.caching_allocator_delete(int(ptr))
 
-    cbs = (ALLOC_T(_alloc), FREE_T(_free))
-    _check(lib, lib.lpsim_set_allocator(cbs[0], cbs[1], None))
-    _alloc_cbs = cbs
+    if _alloc_cbs is None:  # made once: contexts keep the callbacks they were made with
+        _alloc_cbs = (ALLOC_T(_alloc), FREE_T(_free))
+    _check(lib, lib.lpsim_set_allocator(_alloc_cbs[0], _alloc_cbs[1], None))
     return True
 
 

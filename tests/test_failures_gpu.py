@@ -170,3 +170,27 @@ def test_empty_demand_matches_oracle():
     assert_outputs_equal(o, g, n_bins=4, where="empty demand")
     assert np.all(g.lane_map() == 255)
     g.close()
+
+
+def test_callbacks_outlive_their_contexts():
+    """The PyTorch allocator installed again (as the benchmark, the tests and a
+    user's modules each do) while a context made before is open: the context
+    still gives its memory back through the callbacks it was made with."""
+    import gc
+    import torch
+    import workloads as W
+    import paper_2406_08496_gb300 as L
+    net, dem = W.grid_day(seed=2, n_trips=50)
+    L.use_torch_allocator()
+    gc.collect()
+    held = torch.cuda.memory_allocated()
+    s = L.Simulation(net, {})
+    s.load_demand(dem)
+    first = L._alloc_cbs
+    addresses = [ctypes.cast(f, ctypes.c_void_p).value for f in first]
+    del first
+    L.use_torch_allocator()
+    gc.collect()
+    assert [ctypes.cast(f, ctypes.c_void_p).value for f in L._alloc_cbs] == addresses
+    s.close()
+    assert torch.cuda.memory_allocated() == held
