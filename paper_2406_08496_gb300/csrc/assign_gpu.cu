@@ -558,7 +558,8 @@ __global__ void __launch_bounds__(T, PER_SM) td_trees_shared(TreeArgs A) {
                 for (uint32_t i = A.in_off[v]; i < i1; i++) {
                     const uint2 in = A.in_adj[i];
                     const uint32_t tu = s_lab[in.y];
-                    if (tu >= tv) continue;
+                    // (a tail reached as late as v gives its arrival only at the last millisecond, where all later ones stop)
+                    if (tu > tv) continue;
                     const uint64_t t = t0 + tu;
                     if (arrive(A.cms[(size_t)bin_of(A, t) * A.n_pos + in.x], t) == t0 + tv) return in;
                 }

@@ -277,3 +277,31 @@ def test_surrogate_beats_stale_times_on_the_regional_day():
           {k: {q: round(v, 3) for q, v in d.items()} for k, d in e.items()})
     assert e["all"]["surrogate"] < e["all"]["stale"] < 0.5 * e["all"]["free_flow"]
     assert e["changed"]["surrogate"] < e["changed"]["stale"]
+
+
+@pytest.mark.parametrize("n_nodes", [6, 600])
+def test_gpu_paths_past_the_last_millisecond(n_nodes):
+    """Links shut for longer than the 32-bit milliseconds last (times past
+    2^31 ms, two of them in a row on a one-way road): arrivals stop at the last
+    millisecond, a trip to a node behind it still has its path, and the GPU
+    search returns the host's."""
+    from paper_2406_08496_gb300.assignment import Assignment
+    m = n_nodes - 1
+    net = {"n_nodes": n_nodes, "n_edges": m, "edge_src": np.arange(m, dtype=np.uint32),
+           "edge_dst": np.arange(1, m + 1, dtype=np.uint32), "edge_len": np.full(m, 100.0, np.float32),
+           "edge_lanes": np.ones(m, np.uint8), "edge_vmax": np.full(m, 10.0, np.float32)}
+    dest = np.arange(1, n_nodes, dtype=np.uint32)
+    n = len(dest)
+    dem = {"orig": np.zeros(n, np.uint32), "dest": dest, "depart_step": np.arange(n, dtype=np.uint32),
+           "route_off": np.arange(n + 1, dtype=np.uint64), "route_edges": np.zeros(n, np.uint32)}
+    for n_bins in (1, 4):
+        tt = np.full((m, n_bins), 20.0, np.float32)
+        tt[1:3] = 3e6
+        host, gpu = Assignment(net, dem, seed=1), Assignment(net, dem, seed=1)
+        th, rh = _paths(host, host.shortest_paths, tt, 1800, 3600)
+        tg, rg = _paths(gpu, gpu.shortest_paths_gpu, tt, 1800, 3600)
+        assert np.array_equal(th.view(np.uint32), tg.view(np.uint32))
+        assert np.array_equal(rh["route_off"], rg["route_off"])
+        assert np.array_equal(rh["route_edges"], rg["route_edges"])
+        host.close()
+        gpu.close()
