@@ -228,11 +228,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSm) td_trees(Tr
                 // with a few nodes of a few edges each keeps most lanes busy
                 for (uint32_t c0 = 0; c0 < nn; c0 += 32) {
                     const uint32_t i = c0 + lane;
-                    uint32_t u = 0, j0 = 0, deg = 0;
-                    uint64_t tu = kUnreached;
+                    uint32_t u = 0, j0 = 0, deg = 0, tu = 0;  // a queued node is reached: its arrival has 32 bits
                     if (i < nn) {
                         u = __ldcg(fa + i);
-                        tu = __ldcg(&nd[u].lab) >> 32;
+                        tu = (uint32_t)(__ldcg(&nd[u].lab) >> 32);
                         j0 = A.out_off[u];
                         deg = tu < ub ? A.out_off[u + 1] - j0 : 0u;
                     }
@@ -243,6 +242,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSm) td_trees(Tr
                         if (lane >= (uint32_t)o) incl += y;
                     }
                     const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+                    const uint32_t first = j0 - (incl - deg);  // edge t of the warp's is out-edge first + t of its owner
                     for (uint32_t b0 = 0; b0 < total; b0 += 32) {
                         const uint32_t t = b0 + lane;
                         // the lane whose node owns edge t: the first with incl > t
@@ -252,12 +252,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSm) td_trees(Tr
                             const uint32_t y = __shfl_sync(0xFFFFFFFFu, incl, (int)(owner + step - 1));
                             if (y <= t) owner += step;
                         }
-                        const uint32_t o_incl = __shfl_sync(0xFFFFFFFFu, incl, (int)owner);
-                        const uint32_t o_deg = __shfl_sync(0xFFFFFFFFu, deg, (int)owner);
-                        const uint32_t o_j0 = __shfl_sync(0xFFFFFFFFu, j0, (int)owner);
-                        const uint64_t o_tu = __shfl_sync(0xFFFFFFFFu, tu, (int)owner);
+                        const uint32_t o_first = __shfl_sync(0xFFFFFFFFu, first, (int)owner);
+                        const uint32_t o_tu = __shfl_sync(0xFFFFFFFFu, tu, (int)owner);
                         if (t >= total) continue;
-                        const uint32_t j = o_j0 + (t - (o_incl - o_deg));
+                        const uint32_t j = o_first + t;
                         const uint2 ev = A.adj[j];
                         const uint64_t at = arrive(A.cms[(size_t)bin_of(A, o_tu) * A.n_edges + j], o_tu);
                         if (at > 0xFFFFFFFFull || at > ub) continue;

@@ -25,10 +25,11 @@ def lib(tmp_path_factory):
     for src in (os.path.join(HERE, "fake_cudart.cpp"), os.path.join(_build.CSRC, "assign.cpp"),
                 os.path.join(_build.CSRC, "assign_gpu.cu")):
         objs.append(str(out / (os.path.basename(src) + ".o")))
-        subprocess.run([_build._nvcc(), *_build.ARCH, "-O1", "-std=c++17", "-Xcompiler", "-fPIC", "-c", src, "-o", objs[-1]],
-                       check=True)
+        r = subprocess.run([_build._nvcc(), *_build.ARCH, *_build.NVCC_FLAGS, "-Xptxas", "-v", "-c", src, "-o", objs[-1]],
+                           check=True, capture_output=True, text=True)
     so = str(out / "libfake.so")
     subprocess.run(["g++", "-shared", "-o", so, *objs, "-lpthread"], check=True)
+    report = r.stderr  # of assign_gpu.cu, the last
     lib = ctypes.CDLL(so, mode=os.RTLD_LOCAL | os.RTLD_NOW | os.RTLD_DEEPBIND)
     u32, u64 = ctypes.c_uint32, ctypes.c_uint64
     lib.lpsim_assign_create.argtypes = [P, u32, u32, P, P, P, P, P, u64, P, P, P, P, P, ctypes.c_float, u64]
@@ -42,6 +43,7 @@ def lib(tmp_path_factory):
     lib.fake_occupancy.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_size_t]
     for f in ("fake_calls", "fake_uploaded", "fake_live_bytes"):
         getattr(lib, f).restype = ctypes.c_long
+    lib.compiler_report = report
     return lib
 
 
@@ -132,3 +134,12 @@ def test_an_engine_survives_each_failed_allocation(lib, n_nodes):
             assert x[4] == 0, (n, x)
         e.close()
         assert lib.fake_live_bytes() == before
+
+
+def test_search_of_large_networks_keeps_to_its_registers(lib):
+    """td_trees runs 40 warps on an SM, which leaves 48 registers a thread: the
+    compiler's report has it use no more and spill none."""
+    at = lib.compiler_report.index("8td_trees")
+    props = lib.compiler_report[at:].split("Used", 1)
+    assert " 0 bytes spill stores, 0 bytes spill loads" in props[0], props[0]
+    assert int(props[1].split()[0]) <= 48
