@@ -107,6 +107,8 @@ struct __align__(16) NodeRec {
     uint32_t fmark;          // tree mark while the node is in the far pile
 };
 
+constexpr uint64_t kWorkspacePerNode = sizeof(NodeRec) + 4 * 4;  // td_trees: bytes per node and warp
+
 struct TreeArgs {
     uint32_t n_nodes, n_edges, n_bins, bin_ms;
     const uint32_t *out_off;  // n_nodes + 1
@@ -135,7 +137,7 @@ struct TreeArgs {
     unsigned long long *cursor;
     // td_trees_shared: positions along each thread's path, scratch_len per thread
     uint32_t *scratch;
-    uint32_t scratch_len;     // kScratch, or the node count where that is less (no path is as long)
+    uint32_t scratch_len;     // kScratch at most, less on small networks
     // td_trees: per-warp workspaces
     NodeRec *node;            // n_warps x n_nodes: label, round stamp of the last push, far-pile mark
     uint32_t *touched;        // n_warps x n_nodes
@@ -699,6 +701,7 @@ struct AssignGpu {
     // td_trees_shared: its grid at most (0: td_trees searches), its arguments where they are not A's
     void (*shared_kernel)(TreeArgs) = nullptr;
     uint32_t shared_blocks = 0, shared_threads = 0;
+    uint64_t scratch_cap = 0;  // entries of A.scratch
     const uint2 *wide_adj = nullptr, *wide_in = nullptr;
     uint32_t wide = 0;
     uint2 *table[2] = {};  // link-time tables: by out-edge position, by wide position
@@ -873,15 +876,17 @@ int gpu_setup(lpsim_assign *a) {
             g->shared_kernel = kernel;
             g->shared_threads = (uint32_t)threads;
             g->shared_blocks = (uint32_t)(g->n_sm * per_sm);
-            A.scratch_len = std::min(kScratch, a->n_nodes);
-            A.scratch = static_cast<uint32_t *>(g->alloc((size_t)g->shared_blocks * threads * A.scratch_len * 4));
-            if (!A.scratch) return fail(LPSIM_E_OOM, "device allocation of the search workspaces failed");
+            // all resident threads' positions take no more than the workspaces of td_trees' warps would
+            // (a longer path is written to the output in two walks)
+            const uint64_t room = (uint64_t)kBlocksPerSm * kWarpsPerBlock * g->n_sm * kWorkspacePerNode * a->n_nodes / 4;
+            A.scratch_len = (uint32_t)std::min<uint64_t>(std::min(kScratch, a->n_nodes),
+                                                         room / ((uint64_t)g->shared_blocks * threads) + 1);
             CU(cudaStreamSynchronize(g->stream));  // the host arrays go away
             return LPSIM_OK;
         }
     }
     // workspaces: as many warps as fit the budget, at most kBlocksPerSm * kWarpsPerBlock per SM
-    const uint64_t per_warp = (uint64_t)a->n_nodes * (sizeof(NodeRec) + 4 * 4);
+    const uint64_t per_warp = (uint64_t)a->n_nodes * kWorkspacePerNode;
     uint64_t warps = std::min<uint64_t>((uint64_t)g->n_sm * kBlocksPerSm * kWarpsPerBlock,
                                         std::max<uint64_t>(kWorkspaceBudget / std::max<uint64_t>(per_warp, 1), 1));
     warps = std::max<uint64_t>(kWarpsPerBlock, warps / kWarpsPerBlock * kWarpsPerBlock);
@@ -1032,6 +1037,11 @@ extern "C" int lpsim_assign_shortest_paths_gpu(lpsim_assign *a, const float *tt,
     TRY(gpu_groups(a, period_steps));
     TreeArgs &A = g->A;
     TRY(gpu_table(a, tt, n_bins, bin_steps, g->wide != 0));
+    // positions along the paths: for the blocks these trees need, grown when another grouping has more
+    const uint32_t blocks = std::min(g->shared_blocks, std::max(A.n_groups, 1u));
+    const uint64_t scratch = (uint64_t)blocks * g->shared_threads * A.scratch_len;
+    if (scratch > g->scratch_cap && !g->regrow(A.scratch, g->scratch_cap, scratch))
+        return fail(LPSIM_E_OOM, "device allocation of the search workspaces failed");
     // path buffer: room for the current routes' length and half as much again
     if (!g->cap) {
         const uint64_t total = a->roff[a->n];
@@ -1054,8 +1064,7 @@ extern "C" int lpsim_assign_shortest_paths_gpu(lpsim_assign *a, const float *tt,
                 S.adj = g->wide_adj;
                 S.in_adj = g->wide_in;
             }
-            g->shared_kernel<<<std::min(g->shared_blocks, std::max(A.n_groups, 1u)), g->shared_threads,
-                               shared_tree_bytes(a->n_nodes), g->stream>>>(S);
+            g->shared_kernel<<<blocks, g->shared_threads, shared_tree_bytes(a->n_nodes), g->stream>>>(S);
         } else
             td_trees<<<g->n_warps / kWarpsPerBlock, kWarpsPerBlock * 32, 0, g->stream>>>(A);
         CU(cudaGetLastError());

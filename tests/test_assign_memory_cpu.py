@@ -143,3 +143,21 @@ def test_search_of_large_networks_keeps_to_its_registers(lib):
     props = lib.compiler_report[at:].split("Used", 1)
     assert " 0 bytes spill stores, 0 bytes spill loads" in props[0], props[0]
     assert int(props[1].split()[0]) <= 48
+
+
+@pytest.mark.parametrize("n_trips,origins,period", [(64, 4, 600), (3000, 600, 1)])
+def test_a_small_engine_takes_little_device_memory(lib, n_trips, origins, period):
+    """600 nodes: a loading needs no search workspace, a search of four trees one
+    for four blocks, and a search of thousands no more than the warps' workspaces
+    of a search in device memory (32 bytes per node for 40 trees on each of 152
+    SMs), besides tables and a path buffer of some 5 MB."""
+    before = lib.fake_live_bytes()
+    e = _Engine(lib, 600, n_trips, origins)
+    lib.fake_reset(0)
+    assert e.load(4) == 0
+    assert lib.fake_live_bytes() - before < 2 << 20
+    assert e.search(period) == 0
+    trees = len(set(zip((np.arange(n_trips) % origins).tolist(), (np.arange(n_trips) // period).tolist())))
+    assert lib.fake_live_bytes() - before < (8 << 20) + (32 * 600 * 40 * 152 if trees > 4 else 4 << 20)
+    e.close()
+    assert lib.fake_live_bytes() == before
