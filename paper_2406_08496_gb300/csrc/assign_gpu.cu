@@ -759,22 +759,49 @@ int dput(AssignGpu *g, T *&dst, const T *src, size_t count) {
         if (rc_ != LPSIM_OK) return rc_; \
     } while (0)
 
-// The block that searches a tree of n_nodes nodes in shared memory: more threads
-// where fewer blocks fit an SM and near sets are larger.  Measured (blocks of
-// 256 at 32 registers / 256 / 512 / 1024 threads, ms per search with all its
-// host work; td_trees last): 2,750 nodes and 30k trips 0.49 / 0.55 / 0.71 /
-// 1.11, 2.0; 4,900 nodes 0.81 / 0.96 / 1.28 / 2.16; 10,000 nodes 2.27 / 2.24 / 2.88
-// / 4.66; 16,900 nodes 5.66 / 5.46 / 5.88 / 9.01; 27,225 nodes and 340k trips
-// 13.9 / 13.2 / 10.9 / 17.0, 18.5; 52,900 nodes 33.5 / 31.7 / 24.7 / 22.4, 31.5.
+// The block that searches a tree in shared memory: the one of which most fit an
+// SM (a tree is a chain of round trips, so trees in flight count first), of
+// those the one with most threads, of those the one with most registers.
+// Measured, ms per search with all its host work (td_trees_shared<256, 8> / <256, 4> /
+// <512, 2> / <1024, 1>; trees per SM in brackets; lattices of the nodes given, 5 and 15 trips a
+// node, the latter after the comma): 2,500 nodes (8 / 4 / 2 / 1) and 1,840 trees 0.55 / 0.69 / 1.01;
+// 6,084 (8 / 4 / 2) and 2,860 trees 1.72 / 2.04 / 2.81; 8,464 (6 / 4 / 2 / 1) 1.70 / 1.69 / 2.34 / 3.76, 3.30
+// / 3.92 / 5.80 / 9.84; 10,201 (5 / 4 / 2 / 1) 2.16 / 2.28 / 3.07 / 4.90, 5.96 / 6.19 / 7.78 / 12.5; 12,100 (4 / 4 /
+// 2 / 1) 3.01 / 2.89 / 3.77 / 6.08, 7.12 / 6.82 / 9.55 / 15.8; 17,956 (3 / 3 / 2 / 1) - / 6.16 / 6.36 / 9.86; 18,225
+// (2 / 2 / 2 / 1) - / 7.33 / 6.22 / 9.86; 27,225 (the same) - / 13.1 / 10.9 / 17.0; 27,556 (1 / 1 / 1 / 1) - / 22.9
+// / 18.4 / 17.0.  (7,225 nodes with 1,803 trees, a little more than the seven per SM take at once, are the
+// exception found: 1.81 / 1.59; with 4,758 trees 3.15 / 3.34.)  At 32 registers <256, 8> spills 24 bytes.
 // Bucket widths of 60 / 120 / 240 / 480 s: 27,225 nodes 15.0 / 13.6 / 12.3 / 12.9
 // (before the wide rows, which took 12.3 to 10.9).
 using TreeKernel = void (*)(TreeArgs);
-TreeKernel shared_tree_kernel(uint32_t n_nodes, int &threads) {
-    threads = n_nodes <= 20480 ? 256 : n_nodes <= 27648 ? 512 : 1024;
-    return n_nodes <= 6144    ? td_trees_shared<256, 8>
-           : threads == 256   ? td_trees_shared<256, 4>
-           : threads == 512   ? td_trees_shared<512, 2>
-                              : td_trees_shared<1024, 1>;
+constexpr struct {
+    TreeKernel kernel;
+    int threads;
+} kTreeBlocks[] = {{td_trees_shared<256, 8>, 256},
+                   {td_trees_shared<256, 4>, 256},
+                   {td_trees_shared<512, 2>, 512},
+                   {td_trees_shared<1024, 1>, 1024}};  // more threads, then more registers, to the end
+
+int choose_tree_block(AssignGpu *g, uint32_t n_nodes) {
+    if (n_nodes > 0xFFFFu) return LPSIM_OK;  // ids in the ring have 16 bits
+    const size_t smem = shared_tree_bytes(n_nodes);
+    int max_smem = 0, most = 0;
+    CU(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
+    for (const auto &b : kTreeBlocks) {
+        cudaFuncAttributes fa{};
+        CU(cudaFuncGetAttributes(&fa, b.kernel));
+        if (smem + fa.sharedSizeBytes > (size_t)max_smem) continue;
+        CU(cudaFuncSetAttribute(b.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                max_smem - (int)fa.sharedSizeBytes));
+        int per_sm = 0;
+        CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b.kernel, b.threads, smem));
+        if (per_sm == 0 || per_sm < most) continue;
+        most = per_sm;
+        g->shared_kernel = b.kernel;
+        g->shared_threads = (uint32_t)b.threads;
+        g->shared_blocks = (uint32_t)(g->n_sm * per_sm);
+    }
+    return LPSIM_OK;
 }
 
 // graph, trips and workspaces (first call)
@@ -839,51 +866,36 @@ int gpu_setup(lpsim_assign *a) {
         return fail(LPSIM_E_OOM, "device allocation failed");
     A.delta_ms = kDeltaMs;
     // labels in shared memory where they fit
-    const size_t smem = shared_tree_bytes(a->n_nodes);
-    cudaFuncAttributes fa{};
-    int max_smem = 0;
-    int threads = 0;
-    const TreeKernel kernel = shared_tree_kernel(a->n_nodes, threads);
-    CU(cudaFuncGetAttributes(&fa, kernel));
-    CU(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
-    if (a->n_nodes <= 0xFFFFu && smem + fa.sharedSizeBytes <= (size_t)max_smem) {
-        CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                max_smem - (int)fa.sharedSizeBytes));
-        int per_sm = 0;
-        CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
-        if (per_sm > 0) {
-            uint32_t most = 0;
-            for (uint32_t u = 0; u < a->n_nodes; u++) most = std::max(most, a->out_off[u + 1] - a->out_off[u]);
-            if (most <= kWide) {
-                const uint32_t w = most <= 4 ? 4 : 8;
-                std::vector<uint2> wadj((size_t)w * a->n_nodes, make_uint2(kNoEdge, kNever)), win(a->n_edges);
-                std::vector<uint32_t> at(in_off.begin(), in_off.end() - 1);
-                for (uint32_t u = 0; u < a->n_nodes; u++)
-                    for (uint32_t j = a->out_off[u]; j < a->out_off[u + 1]; j++)
-                        wadj[(size_t)u * w + (j - a->out_off[u])] = adj[j];
-                for (uint32_t e = 0; e < a->n_edges; e++) {
-                    const uint32_t u = a->src[e];
-                    win[at[a->dst[e]]++] = make_uint2(u * w + (pos[e] - a->out_off[u]), u);
-                }
-                uint2 *wa, *wi;
-                TRY(dput(g, wa, wadj.data(), wadj.size()));
-                TRY(dput(g, wi, win.data(), win.size()));
-                CU(cudaStreamSynchronize(g->stream));
-                g->wide_adj = wa;
-                g->wide_in = wi;
-                g->wide = w;
+    TRY(choose_tree_block(g, a->n_nodes));
+    if (g->shared_blocks) {
+        uint32_t most = 0;
+        for (uint32_t u = 0; u < a->n_nodes; u++) most = std::max(most, a->out_off[u + 1] - a->out_off[u]);
+        if (most <= kWide) {
+            const uint32_t w = most <= 4 ? 4 : 8;
+            std::vector<uint2> wadj((size_t)w * a->n_nodes, make_uint2(kNoEdge, kNever)), win(a->n_edges);
+            std::vector<uint32_t> at(in_off.begin(), in_off.end() - 1);
+            for (uint32_t u = 0; u < a->n_nodes; u++)
+                for (uint32_t j = a->out_off[u]; j < a->out_off[u + 1]; j++)
+                    wadj[(size_t)u * w + (j - a->out_off[u])] = adj[j];
+            for (uint32_t e = 0; e < a->n_edges; e++) {
+                const uint32_t u = a->src[e];
+                win[at[a->dst[e]]++] = make_uint2(u * w + (pos[e] - a->out_off[u]), u);
             }
-            g->shared_kernel = kernel;
-            g->shared_threads = (uint32_t)threads;
-            g->shared_blocks = (uint32_t)(g->n_sm * per_sm);
-            // all resident threads' positions take no more than the workspaces of td_trees' warps would
-            // (a longer path is written to the output in two walks)
-            const uint64_t room = (uint64_t)kBlocksPerSm * kWarpsPerBlock * g->n_sm * kWorkspacePerNode * a->n_nodes / 4;
-            A.scratch_len = (uint32_t)std::min<uint64_t>(std::min(kScratch, a->n_nodes),
-                                                         room / ((uint64_t)g->shared_blocks * threads) + 1);
-            CU(cudaStreamSynchronize(g->stream));  // the host arrays go away
-            return LPSIM_OK;
+            uint2 *wa, *wi;
+            TRY(dput(g, wa, wadj.data(), wadj.size()));
+            TRY(dput(g, wi, win.data(), win.size()));
+            CU(cudaStreamSynchronize(g->stream));
+            g->wide_adj = wa;
+            g->wide_in = wi;
+            g->wide = w;
         }
+        // all resident threads' positions take no more than the workspaces of td_trees' warps would
+        // (a longer path is written to the output in two walks)
+        const uint64_t room = (uint64_t)kBlocksPerSm * kWarpsPerBlock * g->n_sm * kWorkspacePerNode * a->n_nodes / 4;
+        A.scratch_len = (uint32_t)std::min<uint64_t>(std::min(kScratch, a->n_nodes),
+                                                     room / ((uint64_t)g->shared_blocks * g->shared_threads) + 1);
+        CU(cudaStreamSynchronize(g->stream));  // the host arrays go away
+        return LPSIM_OK;
     }
     // workspaces: as many warps as fit the budget, at most kBlocksPerSm * kWarpsPerBlock per SM
     const uint64_t per_warp = (uint64_t)a->n_nodes * kWorkspacePerNode;

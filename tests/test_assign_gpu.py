@@ -305,3 +305,53 @@ def test_gpu_paths_past_the_last_millisecond(n_nodes):
         assert np.array_equal(rh["route_edges"], rg["route_edges"])
         host.close()
         gpu.close()
+
+
+@pytest.mark.parametrize("side", [79, 80, 102, 103, 115, 116, 134, 135, 165, 166])
+def test_gpu_paths_where_the_block_changes(side):
+    """Lattices on both sides of the sizes at which the search takes another
+    block (six thousand to twenty-eight thousand nodes), shuffled edge ids
+    and many ties: routes and times equal the host's bit for bit."""
+    _, src, dst = _lattice(side)
+    _compare_paths(side * side, src, dst, 4)
+
+
+@pytest.mark.parametrize("degree", [5, 8, 9])
+def test_gpu_paths_with_many_out_edges(degree):
+    """Up to five, eight and nine out-edges a node: rows of eight, full rows of
+    eight, and none (positions through the offsets), shuffled, with ties."""
+    side = 41
+    _, src, dst = _lattice(side)
+    i = np.arange(side * side)
+    r, c = np.divmod(i, side)
+    for k, (dr, dc) in enumerate([(1, 1), (-1, -1), (1, -1), (-1, 1), (2, 1)][:degree - 4]):
+        m = (0 <= r + dr) & (r + dr < side) & (0 <= c + dc) & (c + dc < side)
+        src, dst = np.concatenate([src, i[m]]), np.concatenate([dst, i[m] + dr * side + dc])
+    assert np.bincount(src).max() == degree
+    _compare_paths(side * side, src, dst, 33)
+
+
+def _compare_paths(n, src, dst, n_bins):
+    from paper_2406_08496_gb300.assignment import Assignment
+    rng = np.random.default_rng(n)
+    p = rng.permutation(len(src))
+    src, dst, m = src[p].astype(np.uint32), dst[p].astype(np.uint32), len(p)
+    o = rng.integers(0, n, 12).repeat(8)
+    d = rng.integers(0, n, len(o))
+    d = np.where(d == o, (d + 1) % n, d)
+    net = {"n_nodes": n, "n_edges": m, "edge_src": src, "edge_dst": dst, "edge_len": np.full(m, 100.0, np.float32),
+           "edge_lanes": np.ones(m, np.uint8), "edge_vmax": np.full(m, 10.0, np.float32)}
+    dem = {"orig": o.astype(np.uint32), "dest": d.astype(np.uint32),
+           "depart_step": rng.integers(0, 4000, len(o)).astype(np.uint32),
+           "route_off": np.arange(len(o) + 1, dtype=np.uint64), "route_edges": np.zeros(len(o), np.uint32)}
+    tt = rng.integers(1, 4, (m, n_bins)).astype(np.float32)
+    host, gpu = Assignment(net, dem, seed=1), Assignment(net, dem, seed=1)
+    for period in (600, 7):
+        th, rh = _paths(host, host.shortest_paths, tt, 60, period)
+        tg, rg = _paths(gpu, gpu.shortest_paths_gpu, tt, 60, period)
+        assert np.array_equal(th.view(np.uint32), tg.view(np.uint32))
+        assert np.array_equal(rh["route_off"], rg["route_off"])
+        assert np.array_equal(rh["route_edges"], rg["route_edges"])
+        assert np.array_equal(host.load(tt, 60), gpu.load_gpu(tt, 60))
+    host.close()
+    gpu.close()

@@ -161,3 +161,19 @@ def test_a_small_engine_takes_little_device_memory(lib, n_trips, origins, period
     assert lib.fake_live_bytes() - before < (8 << 20) + (32 * 600 * 40 * 152 if trees > 4 else 4 << 20)
     e.close()
     assert lib.fake_live_bytes() == before
+
+
+@pytest.mark.parametrize("n_nodes", [200, 6200, 6400, 8600, 10500, 10600, 13300, 13400, 18000, 18200, 20480, 27500, 27530,
+                                     27640, 27700, 40000, 55800])
+def test_the_search_s_block_follows_the_occupancy(lib, n_nodes):
+    """The block a search launches is the one of which most fit an SM beside its
+    tree's labels, and among those the one with most threads, then with most
+    registers: no size runs fewer trees, or fewer threads per tree, than it could."""
+    e = _Engine(lib, n_nodes)
+    lib.fake_reset(0)
+    assert e.search(600) == 0
+    name, threads, _, _, _, smem = next(x for x in _launches(lib) if "td_trees" in x[0])
+    assert "td_trees_shared" in name
+    key = lambda t, r: (lib.fake_occupancy(t, r, smem), t, r)
+    assert key(threads, 32 if "Li8E" in name else 56) == max(key(256, 32), key(256, 56), key(512, 56), key(1024, 56))
+    e.close()
