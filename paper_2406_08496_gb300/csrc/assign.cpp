@@ -120,32 +120,67 @@ void td_dijkstra(const TD &td, uint32_t s, uint64_t t0, std::vector<uint64_t> &a
     }
 }
 
-// the candidate path becomes the route of the trips listed (ascending): the
-// flat routes are written anew, on the host's threads
-int take_candidates(lpsim_assign *a, const std::vector<uint64_t> &trips) {
-    if (trips.empty()) return LPSIM_OK;
-    std::vector<uint64_t> off(a->n + 1);
-    uint64_t o = 0;
-    size_t q = 0;
-    for (uint64_t j = 0; j < a->n; j++) {
-        off[j] = o;
-        const bool moved = q < trips.size() && trips[q] == j;
-        o += moved ? a->clen[j] : a->route_len(j);
-        q += moved;
-    }
-    off[a->n] = o;
-    if (!a->redge_next.reserve(o)) return fail(LPSIM_E_OOM, "host allocation of the routes failed");
-    uint32_t *edges = a->redge_next.p.get();
+// all routes in trip order from `to` on, trip j's at off[j], on the host's
+// threads; neighbours that stand together are copied together
+void gather_routes(const lpsim_assign *a, const uint64_t *off, uint32_t *to) {
     parallel_pieces(a->n, [&](uint64_t j0, uint64_t j1, uint64_t) {
-        size_t p = (size_t)(std::lower_bound(trips.begin(), trips.end(), j0) - trips.begin());
-        for (uint64_t j = j0; j < j1; j++) {
-            const bool moved = p < trips.size() && trips[p] == j;
-            std::memcpy(edges + off[j], moved ? a->cand(j) : a->route(j), (off[j + 1] - off[j]) * 4);
-            p += moved;
+        for (uint64_t j = j0; j < j1;) {
+            const uint64_t first = j;
+            while (++j < j1 && a->span[j].b == a->span[j - 1].e) {}
+            std::memcpy(to + off[first], a->route(first), (a->span[j - 1].e - a->span[first].b) * 4);
         }
     });
-    a->roff = std::move(off);
-    std::swap(a->redge, a->redge_next);
+}
+
+// the candidate path becomes the route of the trips listed (ascending)
+int take_candidates(lpsim_assign *a, const std::vector<uint64_t> &trips) {
+    if (trips.empty()) return LPSIM_OK;
+    // where each new route goes behind the present ones, as long as there is room
+    std::vector<uint64_t> at;
+    at.reserve(trips.size());
+    uint64_t used = a->redge_used, total = a->route_total;
+    for (uint64_t j : trips) {
+        if (used + a->clen[j] > a->redge.cap) break;
+        at.push_back(used);
+        used += a->clen[j];
+        total += a->clen[j] - a->route_len(j);
+    }
+    if (at.size() == trips.size()) {
+        uint32_t *to = a->redge.p.get();
+        parallel_pieces(trips.size(), [&](uint64_t q0, uint64_t q1, uint64_t) {
+            for (uint64_t q = q0; q < q1; q++) {
+                const uint64_t j = trips[q];
+                std::memcpy(to + at[q], a->cand(j), (size_t)a->clen[j] * 4);
+                a->span[j] = {at[q], at[q] + a->clen[j]};
+            }
+        });
+    } else {  // every route anew, in order
+        std::vector<uint64_t> off(a->n);
+        used = 0;
+        for (uint64_t j = 0, q = 0; j < a->n; j++) {
+            const bool moved = q < trips.size() && trips[q] == j;
+            off[j] = used;
+            used += moved ? a->clen[j] : a->route_len(j);
+            q += moved;
+        }
+        total = used;
+        if (!a->redge_next.reserve(used)) return fail(LPSIM_E_OOM, "host allocation of the routes failed");
+        uint32_t *to = a->redge_next.p.get();
+        parallel_pieces(a->n, [&](uint64_t j0, uint64_t j1, uint64_t) {
+            size_t q = (size_t)(std::lower_bound(trips.begin(), trips.end(), j0) - trips.begin());
+            for (uint64_t j = j0; j < j1; j++) {
+                const bool moved = q < trips.size() && trips[q] == j;
+                const uint64_t len = moved ? a->clen[j] : a->route_len(j);
+                std::memcpy(to + off[j], moved ? a->cand(j) : a->route(j), len * 4);
+                a->span[j] = {off[j], off[j] + len};
+                q += moved;
+            }
+        });
+        std::swap(a->redge, a->redge_next);
+        a->layout++;
+    }
+    a->redge_used = used;
+    a->route_total = total;
     a->routes_version++;
     return LPSIM_OK;
 }
@@ -198,9 +233,11 @@ int lpsim_assign_create(lpsim_assign **out, uint32_t n_nodes, uint32_t n_edges, 
         }
     }
     if (n_trips) {
-        a->roff.resize(n_trips + 1);
-        for (uint64_t j = 0; j <= n_trips; j++) a->roff[j] = route_off[j] - route_off[0];
-        const uint64_t n_edge_ids = a->roff[n_trips];
+        a->span.resize(n_trips);
+        for (uint64_t j = 0; j < n_trips; j++)
+            a->span[j] = {route_off[j] - route_off[0], route_off[j + 1] - route_off[0]};
+        const uint64_t n_edge_ids = a->span[n_trips - 1].e;
+        a->redge_used = a->route_total = n_edge_ids;
         if (!a->redge.reserve(n_edge_ids)) {
             delete a;
             return fail(LPSIM_E_OOM, "host allocation of the routes failed");
@@ -209,8 +246,6 @@ int lpsim_assign_create(lpsim_assign **out, uint32_t n_nodes, uint32_t n_edges, 
         parallel_pieces(n_edge_ids, [&](uint64_t q0, uint64_t q1, uint64_t) {
             std::memcpy(a->redge.p.get() + q0, from + q0, (q1 - q0) * 4);
         });
-    } else {
-        a->roff.assign(1, 0);
     }
     a->dt = dt;
     a->seed = seed;
@@ -354,7 +389,7 @@ int lpsim_assign_route_excess(lpsim_assign *a, const float *tt, uint32_t n_bins,
         for (uint64_t j = j0; j < j1; j++) {
             const uint64_t t0 = to_ms((double)a->dep[j] * a->dt);
             uint64_t t = t0;
-            for (uint64_t q = a->roff[j]; q < a->roff[j + 1]; q++) t = td.arrive(a->redge.p[q], t);
+            for (uint64_t q = a->span[j].b; q < a->span[j].e; q++) t = td.arrive(a->redge.p[q], t);
             a->excess[j] = (float)((double)(t - t0) / 1000.0 - a->tsp[j]);
         }
     });
@@ -386,16 +421,20 @@ int lpsim_assign_reroute_worst(lpsim_assign *a, double fraction, double min_rel_
 
 uint64_t lpsim_assign_route_length(const lpsim_assign *a) {
     if (!a) return 0;
-    return a->roff[a->n];
+    return a->route_total;
 }
 
 int lpsim_assign_get_routes(const lpsim_assign *a, uint64_t *route_off, uint32_t *route_edges, uint64_t capacity) {
     if (!a || !route_off || !route_edges) return fail(LPSIM_E_INVALID_ARG, "NULL argument");
     if (capacity < lpsim_assign_route_length(a)) return fail(LPSIM_E_INVALID_ARG, "route buffer too small");
-    std::memcpy(route_off, a->roff.data(), (a->n + 1) * sizeof(uint64_t));
-    parallel_pieces(a->roff[a->n], [&](uint64_t q0, uint64_t q1, uint64_t) {
-        std::memcpy(route_edges + q0, a->redge.p.get() + q0, (q1 - q0) * 4);
-    });
+    route_off[0] = 0;
+    for (uint64_t j = 0; j < a->n; j++) route_off[j + 1] = route_off[j] + a->route_len(j);
+    if (a->redge_used == a->route_total)  // none moved since they were last written in order
+        parallel_pieces(a->route_total, [&](uint64_t q0, uint64_t q1, uint64_t) {
+            std::memcpy(route_edges + q0, a->redge.p.get() + q0, (q1 - q0) * 4);
+        });
+    else
+        gather_routes(a, route_off, route_edges);
     return LPSIM_OK;
 }
 
@@ -406,7 +445,7 @@ int lpsim_assign_load(const lpsim_assign *a, const float *tt, uint32_t n_bins, u
     parallel_pieces(a->n, [&](uint64_t j0, uint64_t j1, uint64_t) {
         for (uint64_t j = j0; j < j1; j++) {
             uint64_t t = to_ms((double)a->dep[j] * a->dt);
-            for (uint64_t q = a->roff[j]; q < a->roff[j + 1]; q++) {
+            for (uint64_t q = a->span[j].b; q < a->span[j].e; q++) {
                 const uint32_t e = a->redge.p[q];
                 const uint64_t b = t / td.bin_ms;
                 if (b < n_bins) __atomic_fetch_add(&inflow[(size_t)e * n_bins + b], 1u, __ATOMIC_RELAXED);

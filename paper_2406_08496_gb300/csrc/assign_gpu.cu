@@ -663,13 +663,13 @@ __global__ void init_nodes(NodeRec *nd, size_t n) {
 // planned departure with the arrival rule of the table, counting one entry
 // in the bin of every link entry time (the host's lpsim_assign_load, on the
 // device: integer counts, so the order of the atomics does not matter).
-__global__ void load_routes(const unsigned long long *roff, const uint32_t *redge, const uint32_t *dep_ms,
+__global__ void load_routes(const ulonglong2 *span, const uint32_t *redge, const uint32_t *dep_ms,
                             uint64_t n, const uint2 *cms, const uint32_t *pos, uint32_t n_edges, uint32_t n_bins,
                             uint32_t bin_ms, uint32_t *inflow) {
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < n; j += (uint64_t)gridDim.x * blockDim.x) {
         uint64_t t = dep_ms[j];
-        const unsigned long long q1 = roff[j + 1];
-        for (unsigned long long q = roff[j]; q < q1; q++) {
+        const ulonglong2 r = span[j];
+        for (unsigned long long q = r.x; q < r.y; q++) {
             const uint32_t e = redge[q];
             const uint64_t b = t / bin_ms;
             if (b < n_bins) atomicAdd(&inflow[(size_t)e * n_bins + b], 1u);
@@ -692,10 +692,11 @@ struct AssignGpu {
     std::vector<uint64_t> order, gstart;
     unsigned long long cap = 0;
     // routes and inflow of lpsim_assign_load_gpu
-    unsigned long long *roff = nullptr;
+    ulonglong2 *span = nullptr;
     uint32_t *redge = nullptr;
     uint64_t redge_cap = 0;
-    uint64_t routes_version = ~0ull;  // of the routes on the device
+    uint64_t redge_here = 0, layout = 0;  // entries of the engine's on the device, of which layout
+    uint64_t routes_version = ~0ull;      // of the routes on the device
     float *tt = nullptr;              // link times as given
     size_t tt_cells = 0;
     // td_trees_shared: its grid at most (0: td_trees searches), its arguments where they are not A's
@@ -1008,20 +1009,27 @@ extern "C" int lpsim_assign_load_gpu(const lpsim_assign *ac, const float *tt, ui
     CU(cudaGetDevice(&dev));
     if (dev != g->device) return fail(LPSIM_E_STATE, "the device current at the first GPU call must be current");
     TRY(gpu_table(a, tt, n_bins, bin_steps, false));
-    // the engine's routes stay on the device until a re-routing changes them
-    if (!g->roff) {
-        g->roff = static_cast<unsigned long long *>(g->alloc((a->n + 1) * 8));
-        if (!g->roff) return fail(LPSIM_E_OOM, "device allocation of the route offsets failed");
+    // the engine's routes stay on the device; a re-routing brings what it wrote
+    if (!g->span) {
+        g->span = static_cast<ulonglong2 *>(g->alloc(a->n * sizeof(ulonglong2)));
+        if (!g->span) return fail(LPSIM_E_OOM, "device allocation of the route offsets failed");
     }
     if (g->routes_version != a->routes_version) {
-        const uint64_t total = a->roff[a->n];
         g->routes_version = ~0ull;
-        if (total > g->redge_cap && !g->regrow(g->redge, g->redge_cap, total + total / 4))
-            return fail(LPSIM_E_OOM, "device allocation of the routes failed");
-        CU(cudaMemcpyAsync(g->roff, a->roff.data(), (a->n + 1) * 8, cudaMemcpyHostToDevice, g->stream));
-        if (total)
-            CU(cudaMemcpyAsync(g->redge, a->redge.p.get(), total * 4, cudaMemcpyHostToDevice, g->stream));
+        if (g->layout != a->layout) g->redge_here = 0;
+        if (a->redge_used > g->redge_cap) {
+            g->redge_here = 0;
+            if (!g->regrow(g->redge, g->redge_cap, a->redge.cap))
+                return fail(LPSIM_E_OOM, "device allocation of the routes failed");
+        }
+        static_assert(sizeof(RouteSpan) == sizeof(ulonglong2), "route spans");
+        CU(cudaMemcpyAsync(g->span, a->span.data(), a->n * sizeof(ulonglong2), cudaMemcpyHostToDevice, g->stream));
+        if (a->redge_used > g->redge_here)
+            CU(cudaMemcpyAsync(g->redge + g->redge_here, a->redge.p.get() + g->redge_here,
+                               (a->redge_used - g->redge_here) * 4, cudaMemcpyHostToDevice, g->stream));
         CU(cudaStreamSynchronize(g->stream));
+        g->redge_here = a->redge_used;
+        g->layout = a->layout;
         g->routes_version = a->routes_version;
     }
     const size_t cells = (size_t)a->n_edges * n_bins;
@@ -1029,7 +1037,7 @@ extern "C" int lpsim_assign_load_gpu(const lpsim_assign *ac, const float *tt, ui
         return fail(LPSIM_E_OOM, "device allocation of the inflow table failed");
     CU(cudaMemsetAsync(g->inflow, 0, cells * 4, g->stream));
     load_routes<<<(unsigned)std::min<uint64_t>((a->n + 255) / 256, 65535), 256, 0, g->stream>>>(
-        g->roff, g->redge, g->A.dep_ms, a->n, g->A.cms, g->A.pos, a->n_edges, n_bins, g->A.bin_ms, g->inflow);
+        g->span, g->redge, g->A.dep_ms, a->n, g->A.cms, g->A.pos, a->n_edges, n_bins, g->A.bin_ms, g->inflow);
     CU(cudaGetLastError());
     CU(cudaMemcpyAsync(inflow, g->inflow, cells * 4, cudaMemcpyDeviceToHost, g->stream));
     CU(cudaStreamSynchronize(g->stream));
@@ -1056,7 +1064,7 @@ extern "C" int lpsim_assign_shortest_paths_gpu(lpsim_assign *a, const float *tt,
         return fail(LPSIM_E_OOM, "device allocation of the search workspaces failed");
     // path buffer: room for the current routes' length and half as much again
     if (!g->cap) {
-        const uint64_t total = a->roff[a->n];
+        const uint64_t total = a->route_total;
         if (!g->regrow(A.edges, g->cap, std::max<uint64_t>(total + total / 2, 1u << 20)))
             return fail(LPSIM_E_OOM, "device allocation of the path buffer failed");
     }

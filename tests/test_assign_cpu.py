@@ -230,3 +230,61 @@ def test_worst_first_reroute(A):
     arr = np.full(n, 0xFFFFFFFF, np.uint32)  # nobody arrived: no excess, nothing moves
     a.gap(dep_act, arr)
     assert a.reroute_worst(0.5) == 0
+
+
+def _lattice_engine(A, side, n_trips, seed):
+    """Trips on a lattice, each on its shortest path under some link times."""
+    rng = np.random.default_rng(seed)
+    i = np.arange(side * side)
+    r, c = np.divmod(i, side)
+    src = np.concatenate([i[c < side - 1], i[c > 0], i[r < side - 1], i[r > 0]])
+    dst = np.concatenate([i[c < side - 1] + 1, i[c > 0] - 1, i[r < side - 1] + side, i[r > 0] - side])
+    net = make_net(side * side, [(int(u), int(v), 100.0, 1, 10.0) for u, v in zip(src, dst)])
+    o = rng.integers(0, side * side, 8).repeat(-(-n_trips // 8))[:n_trips]
+    d = rng.integers(0, side * side, n_trips)
+    dem = {"orig": o.astype(np.uint32), "dest": np.where(d == o, (d + 1) % side ** 2, d).astype(np.uint32),
+           "depart_step": rng.integers(0, 4000, n_trips).astype(np.uint32),
+           "route_off": np.arange(n_trips + 1, dtype=np.uint64), "route_edges": np.zeros(n_trips, np.uint32)}
+    a = A.Assignment(net, dem, seed=seed)
+    a.shortest_paths(rng.uniform(5, 30, (len(src), 4)).astype(np.float32), 900, 600)
+    a.reroute(1.0, 0)
+    return net, dem, a, rng
+
+
+def _split(routes):
+    off = routes["route_off"].astype(np.int64)
+    return [routes["route_edges"][off[j]:off[j + 1]].tolist() for j in range(len(off) - 1)]
+
+
+@pytest.mark.parametrize("n_trips", [1, 7, 500, 20000])
+def test_reroutings_of_every_size_leave_the_other_routes(A, n_trips):
+    """Small and large re-routings one after another (new routes behind the old
+    ones, all in order again when there is no room): exactly the trips counted as
+    moved have their candidate path, all others the route they had; the routes read
+    back load like those of a new engine."""
+    net, dem, a, rng = _lattice_engine(A, 9, n_trips, 3)
+    m = net["n_edges"]
+    for it, f in enumerate([0.01, 0.02, 0.0, 0.3, 0.05, 0.1, 0.1, 0.1, 1.0, 0.01, 0.6, 0.03]):
+        tt = rng.uniform(5, 30, (m, 4)).astype(np.float32)
+        before = _split(a.routes())
+        b = A.Assignment(net, dict(dem, **{k: v for k, v in a.routes().items() if k != "depart_step"}), seed=9)
+        a.shortest_paths(tt, 900, 600)
+        b.shortest_paths(tt, 900, 600)
+        b.reroute(1.0, 0)
+        cand = _split(b.routes())
+        if it % 2:
+            a.route_excess(tt, 900)
+            moved = a.reroute_worst(f)
+        else:
+            moved = a.reroute(f, it)
+        routes = a.routes()
+        after = _split(routes)
+        differ = [j for j in range(n_trips) if after[j] != before[j]]
+        assert len(differ) == moved and all(after[j] == cand[j] for j in differ)
+        if f == 1.0 and not it % 2:
+            assert after == cand
+        c = A.Assignment(net, dict(dem, route_off=routes["route_off"], route_edges=routes["route_edges"]), seed=9)
+        assert np.array_equal(a.load(tt, 900), c.load(tt, 900))
+        b.close()
+        c.close()
+    a.close()

@@ -355,3 +355,20 @@ def _compare_paths(n, src, dst, n_bins):
         assert np.array_equal(host.load(tt, 60), gpu.load_gpu(tt, 60))
     host.close()
     gpu.close()
+
+
+def test_gpu_load_follows_every_rerouting(case):
+    """Loadings on the GPU between re-routings of every size (new routes behind
+    the old ones, all anew when there is no room, two re-routings between two
+    loadings) count what the host walk counts."""
+    from paper_2406_08496_gb300.assignment import Assignment
+    net, dem = case
+    A = Assignment(net, dem, seed=2)
+    for it, f in enumerate([0.01, 0.02, 0.3, 0.05, 0.1, 0.1, 0.1, 1.0, 0.01, 0.6, 0.03]):
+        tt = _tables(net, 96, 20 + it)
+        A.shortest_paths_gpu(tt, 1800, 3600)
+        A.reroute(f, it)
+        if it % 4 == 1:
+            continue
+        assert np.array_equal(A.load(tt, 1800), A.load_gpu(tt, 1800)), it
+    A.close()

@@ -36,6 +36,8 @@ def lib(tmp_path_factory):
     lib.lpsim_assign_shortest_paths_gpu.argtypes = [P, P, u32, u32, u32, P]
     lib.lpsim_assign_load_gpu.argtypes = [P, P, u32, u32, P]
     lib.lpsim_assign_destroy.argtypes = [P]
+    lib.lpsim_assign_shortest_paths.argtypes = [P, P, u32, u32, u32, u32, P]
+    lib.lpsim_assign_reroute.argtypes = [P, ctypes.c_double, u32, P]
     lib.fake_reset.argtypes = [ctypes.c_long]
     lib.fake_next_read.argtypes = [ctypes.c_size_t, u64]
     lib.fake_launch.argtypes = [ctypes.c_int, P]
@@ -54,16 +56,16 @@ def _p(a):
 class _Engine:
     """A ring of nodes, both ways round, and trips from a few of them."""
 
-    def __init__(self, lib, n_nodes, n_trips=64, origins=4):
+    def __init__(self, lib, n_nodes, n_trips=64, origins=4, hops=2):
         self.lib, self.n = lib, n_trips
         i = np.arange(n_nodes, dtype=np.uint32)
-        src, dst = np.concatenate([i, i]), np.concatenate([(i + 1) % n_nodes, (i - 1) % n_nodes]).astype(np.uint32)
+        src, dst = np.concatenate([i, i]), np.concatenate([(i + 1) % n_nodes, (i + n_nodes - 1) % n_nodes]).astype(np.uint32)
         self.m = len(src)
         length, lanes, vmax = np.full(self.m, 100.0, np.float32), np.ones(self.m, np.uint8), np.full(self.m, 10.0, np.float32)
         orig = (np.arange(n_trips) % origins).astype(np.uint32)
-        dest, dep = ((orig + 2) % n_nodes).astype(np.uint32), np.arange(n_trips, dtype=np.uint32)
-        off = 2 * np.arange(n_trips + 1, dtype=np.uint64)
-        edges = np.stack([orig, (orig + 1) % n_nodes], 1).reshape(-1).astype(np.uint32)
+        dest, dep = ((orig + hops) % n_nodes).astype(np.uint32), np.arange(n_trips, dtype=np.uint32)
+        off = hops * np.arange(n_trips + 1, dtype=np.uint64)
+        edges = ((orig[:, None] + np.arange(hops)) % n_nodes).reshape(-1).astype(np.uint32)
         h = P()
         self._keep = (src, dst, length, lanes, vmax, orig, dest, dep, off, edges)
         assert lib.lpsim_assign_create(ctypes.byref(h), n_nodes, self.m, *[_p(a) for a in self._keep[:5]], n_trips,
@@ -176,4 +178,22 @@ def test_the_search_s_block_follows_the_occupancy(lib, n_nodes):
     assert "td_trees_shared" in name
     key = lambda t, r: (lib.fake_occupancy(t, r, smem), t, r)
     assert key(threads, 32 if "Li8E" in name else 56) == max(key(256, 32), key(256, 56), key(512, 56), key(1024, 56))
+    e.close()
+
+
+def test_a_small_rerouting_brings_little_to_the_device(lib):
+    """4,000 trips of 60 edges on a ring, one in a hundred moved to the 40 edges
+    the other way round: the next loading takes the moved routes and where each
+    trip's route stands (16 bytes) to the device, not the routes that stay."""
+    e = _Engine(lib, 100, 4000, 4, hops=60)
+    tt, t = np.full((e.m, 4), 5.0, np.float32), np.empty(e.n, np.float32)
+    assert lib.lpsim_assign_shortest_paths(e.h, _p(tt), 4, 60, 600, 2, _p(t)) == 0
+    lib.fake_reset(0)
+    assert e.load(4) == 0 and lib.fake_uploaded() > 4 * 60 * e.n
+    at, changed = lib.fake_uploaded(), ctypes.c_uint64()
+    assert lib.lpsim_assign_reroute(e.h, 0.01, 1, ctypes.byref(changed)) == 0 and 10 < changed.value < 100
+    assert e.load(4) == 0
+    assert lib.fake_uploaded() - at == tt.nbytes + 16 * e.n + 4 * 40 * changed.value
+    assert e.load(4) == 0
+    assert lib.fake_uploaded() - at == 2 * tt.nbytes + 16 * e.n + 4 * 40 * changed.value
     e.close()
