@@ -619,7 +619,7 @@ __device__ __forceinline__ void p1_slot(const Dev &d, const StepView &w, const P
             atomicAdd(sk.n + 3, 1u);
         }
     }
-    }
+}
 
 // 16-byte words of the staged records into a global list (every thread)
 template <class T>
@@ -808,9 +808,8 @@ __device__ __forceinline__ void p2_dep(const Dev &d, const StepView &w, const De
 // `late` (the intent aims at cell len - 1 and runs alongside the crossing
 // requests) a hold that a losing crosser of the target lane is placing in the
 // same kernel counts as occupying the target cell.
-// TOGETHER: both windows are loaded before either is searched (one round trip;
-// 20 registers more).
-template <bool TOGETHER>
+// The windows ahead and behind are loaded and searched one after the other
+// (both loaded first: one round trip, but 20 registers more; see step_p2).
 __device__ __forceinline__ void lane_change(const Dev &d, const StepView &w, const IntendRec &ir, uint32_t &changes,
                                           bool late) {
     const uint32_t k = w.k;
@@ -837,9 +836,8 @@ __device__ __forceinline__ void lane_change(const Dev &d, const StepView &w, con
     {
         uint4 qa[5], qb[5];
         load_ahead<5>(row2, c0, hi, qa);
-        if (TOGETHER) load_behind<5>(row2, lo, bhi, qb);
         fa = find_first<5>(qa, c0);
-        if (!TOGETHER) load_behind<5>(row2, lo, bhi, qb);
+        load_behind<5>(row2, lo, bhi, qb);
         fb = find_last<5>(qb, bhi);
     }
     const uint32_t tgt = base2 + cn;
@@ -935,7 +933,7 @@ __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) step_p2(Dev d, uint32_t k
             const IntendRec ir = list[i];
             loads_issued();
             if (i >= nint) break;
-            lane_change<false>(d, w, ir, changes, false);
+            lane_change(d, w, ir, changes, false);
         }
     } else if (blockIdx.x == gc + gi) {
         const uint32_t nlate = d.counts[6 + par];
@@ -944,7 +942,7 @@ __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) step_p2(Dev d, uint32_t k
             const IntendRec ir = *(top - i);
             loads_issued();
             if (i >= nlate) break;
-            lane_change<false>(d, w, ir, changes, true);
+            lane_change(d, w, ir, changes, true);
         }
     } else {
         const uint32_t ndep = d.counts[4 + par];
@@ -1042,14 +1040,14 @@ __global__ void __launch_bounds__(BLOCK, 1)
         for (uint32_t i = tid; i < ncross; i += BLOCK)
             p2_cross(d, w, i < kStageCross ? s_cr[i] : d.cross_list[par][i - kStageCross], ev0 + i, events);
         for (uint32_t i = tid_mid; i < nint; i += BLOCK)
-            lane_change<false>(d, w, i < kStageIntend ? s_ir[i] : d.intend_list[par][i - kStageIntend], changes, false);
+            lane_change(d, w, i < kStageIntend ? s_ir[i] : d.intend_list[par][i - kStageIntend], changes, false);
         for (uint32_t q = tid_down; q < ndep; q += BLOCK)
             p2_dep(d, w, q < kStageDep ? s_dr[q] : d.dep_rec[par][q - kStageDep], q, n, events, departed);
         if (nlate) {
             // P3: the intents at stop-line cells, after every hold
             __syncthreads();
             for (uint32_t i = tid; i < nlate; i += BLOCK)
-                lane_change<false>(d, w, d.intend_list[par][d.cap - 1 - i], changes, false);
+                lane_change(d, w, d.intend_list[par][d.cap - 1 - i], changes, false);
         }
         if (tid == 0) {  // the next step's global lists start empty
             d.counts[par ^ 1u] = 0;
