@@ -373,7 +373,7 @@ def paths_arm(args):
     """Time-dependent shortest paths of every trip of the assignment case
     (one tree per origin and 30-minute departure period) under the link
     times of one simulation of its free-flow routes, per pass: the GPU
-    search (one warp per tree) or the host search (--paths host)."""
+    search (lpsim_assign_shortest_paths_gpu) or the host search (--paths host)."""
     import workloads as W
     import paper_2406_08496_gb300 as L
     from paper_2406_08496_gb300.assignment import Assignment

@@ -98,9 +98,10 @@ typedef struct lpsim_params {
                              networks of up to ~40k lane-metres; results are the same either way;
                              measured 2% slower on a 4x4 grid, whose maps stay in L2 anyway);
                              other bits must be 0 */
-    uint32_t light_trips; /* a chunk (or a piece of one) runs in the single-block light-load kernel when at most this many
-                             trips can be on the network or waiting during it (0 = 1536); a speed
-                             setting only, results are the same for every value */
+    uint32_t light_trips; /* a chunk (or a piece of one) runs in the single-block light-load
+                             kernel when at most this many trips can be on the network or
+                             waiting during it (0 = 1536); a speed setting only, results are the
+                             same for every value */
     float dlc_prob;       /* discretionary lane change (an extension; the paper defines only the
                              mandatory change): per-step probability, in [0, 1], that a vehicle
                              outside the mandatory zone, held below its free speed by a slower
@@ -282,8 +283,10 @@ int lpsim_get_trips(lpsim_ctx *ctx, uint64_t n, uint32_t *depart_actual, uint32_
  * trips loaded) position on the edge (m), speed (m/s), edge, lane, index in
  * its route and status (0 waiting, 1 active, 2 arrived); non-active vehicles
  * read x = v = 0, edge 0xFFFFFFFF, lane 0, index 0.  Any pointer may be NULL.
- * Takes n * 17 bytes of device scratch for the call (from cudaMalloc or the
- * allocator callback) and gives it back before returning, on every path.
+ * Takes n * 18 bytes of device scratch (from cudaMalloc or the allocator
+ * callback).  A demand that needs at most 1 MiB of it uses a block of that size,
+ * which the context makes at the first such call and keeps; a larger one's is given
+ * back before returning, on every path.
  * Errors: LPSIM_E_STATE before lpsim_load_demand; LPSIM_E_INVALID_ARG when n
  * differs from the trips loaded; LPSIM_E_OOM; LPSIM_E_CUDA. */
 int lpsim_get_state(lpsim_ctx *ctx, uint64_t n, float *x, float *v, uint32_t *edge, uint8_t *lane,

@@ -61,13 +61,14 @@ int lpsim_assign_shortest_paths(lpsim_assign *a, const float *tt, uint32_t n_bin
 /* lpsim_assign_shortest_paths with the earliest-arrival trees searched on
  * the GPU (device current at the first call; label-correcting rounds, one block
  * per tree with its labels in shared memory for networks of up to some 55
- * thousand nodes, one warp per tree, thousands at a time, beyond).  Same candidate routes and t_sp, bit for bit, as the host
- * searches: link times are whole milliseconds, so every arrival is an exact
- * sum, and both keep the earliest arrival with ties to the lower entering
- * edge id.  The graph, trip table and search workspaces (at most 32
- * bytes per node for 40 trees per SM, within 48 GiB; on networks of up to
- * some 55 thousand nodes at most 2 KB per thread of the blocks that the trees
- * need) stay on the device between calls and are released by lpsim_assign_destroy.  Errors as the host call, plus
+ * thousand nodes, one warp per tree, thousands at a time, beyond).  Same
+ * candidate routes and t_sp, bit for bit, as the host searches: link times are
+ * whole milliseconds, so every arrival is an exact sum, and both keep the
+ * earliest arrival with ties to the lower entering edge id.  The graph, trip
+ * table and search workspaces (at most 32 bytes per node for 40 trees per SM,
+ * within 48 GiB; on networks of up to some 55 thousand nodes at most 2 KB per
+ * thread of the blocks that the trees need) stay on the device between calls
+ * and are released by lpsim_assign_destroy.  Errors as the host call, plus
  * LPSIM_E_CUDA, LPSIM_E_OOM and LPSIM_E_STATE (another device current). */
 int lpsim_assign_shortest_paths_gpu(lpsim_assign *a, const float *tt, uint32_t n_bins, uint32_t bin_steps,
                                     uint32_t period_steps, float *t_sp);

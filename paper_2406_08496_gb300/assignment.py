@@ -200,8 +200,8 @@ def msa(net: dict, dem: dict, mode: str = "plain", iterations: int = 10, fractio
     with the largest relative excess of their route over the shortest path
     under the iteration's link times, measured or predicted; only trips more
     than min_rel_excess worse than their shortest path).  paths: where the
-    time-dependent shortest paths are searched -- "gpu" (one warp per tree)
-    or "host" (Dijkstra on the host threads); both give the same routes and
+    time-dependent shortest paths are searched -- "gpu" (one block per
+    tree, or one warp per tree on networks past some 55 thousand nodes) or "host" (Dijkstra on the host threads); both give the same routes and
     times.  Returns the iteration history and the wall time to reach
     target_gap (None if never reached)."""
     assert mode in ("plain", "surrogate") and select in ("worst", "random") and paths in ("gpu", "host")

@@ -1703,9 +1703,12 @@ uint64_t forward_piece(const lpsim_mlp *m) { return 4ull * m->n_sm * kBM; }
 // The copy stream is waited for before the caller's rows may go away.
 int forward_pieces(lpsim_mlp *m, uint64_t n, const float *X, float *y) {
     const uint64_t piece = forward_piece(m);
-    // the rows may be written by work on the model's stream before this call
-    CU(cudaEventRecord(m->in_used[0], m->stream));
-    CU(cudaStreamWaitEvent(m->in_stream, m->in_used[0], 0));
+    // the rows may be written by work on the caller's stream before this call (no one else has a
+    // stream of the model's own)
+    if (!m->own_stream) {
+        CU(cudaEventRecord(m->in_used[0], m->stream));
+        CU(cudaStreamWaitEvent(m->in_stream, m->in_used[0], 0));
+    }
     for (uint64_t r0 = 0, i = 0; r0 < n; r0 += piece, i++) {
         const uint64_t nb = std::min(piece, n - r0);
         const int b = (int)(i & 1);
