@@ -164,7 +164,8 @@ int take_candidates(lpsim_assign *a, const std::vector<uint64_t> &trips) {
             q += moved;
         }
         total = used;
-        if (!a->redge_next.reserve(used)) return fail(LPSIM_E_OOM, "host allocation of the routes failed");
+        // (with an eighth to spare at least: the routes may have grown since the buffer was made)
+        if (!a->redge_next.reserve(used + used / 8)) return fail(LPSIM_E_OOM, "host allocation of the routes failed");
         uint32_t *to = a->redge_next.p.get();
         parallel_pieces(a->n, [&](uint64_t j0, uint64_t j1, uint64_t) {
             size_t q = (size_t)(std::lower_bound(trips.begin(), trips.end(), j0) - trips.begin());

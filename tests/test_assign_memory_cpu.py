@@ -197,3 +197,23 @@ def test_a_small_rerouting_brings_little_to_the_device(lib):
     assert e.load(4) == 0
     assert lib.fake_uploaded() - at == 2 * tt.nbytes + 16 * e.n + 4 * 40 * changed.value
     e.close()
+
+
+def test_a_rewrite_leaves_room_for_the_next_small_rerouting(lib):
+    """Routes that have grown by a fifth since the buffers were made (one trip in
+    twenty on 60 edges instead of 10): small re-routings to and fro after that
+    bring what they move, but for a few rewrites."""
+    e = _Engine(lib, 70, 4000, 4, hops=10)
+    tt, t, changed = np.full((e.m, 4), 5.0, np.float32), np.empty(e.n, np.float32), ctypes.c_uint64()
+    lib.fake_reset(0)
+    rewrites = 0
+    for it, f in enumerate([0.045] + 40 * [0.004, 0.05]):
+        back = it % 2 == 0  # the way back is 60 edges long, the way forward 10
+        tt[:70], tt[70:] = (500.0, 5.0) if back else (5.0, 500.0)
+        assert lib.lpsim_assign_shortest_paths(e.h, _p(tt), 4, 60, 600, 2, _p(t)) == 0
+        assert lib.lpsim_assign_reroute(e.h, f if back else 0.1, it, ctypes.byref(changed)) == 0
+        at = lib.fake_uploaded()
+        assert e.load(4) == 0
+        rewrites += lib.fake_uploaded() - at - tt.nbytes - 16 * e.n != 4 * (60 if back else 10) * changed.value
+    assert rewrites <= 18  # of 81; 24 with buffers that only just hold the routes
+    e.close()
